@@ -13,6 +13,7 @@
 #include "../../include/selbm.h"
 #include "selbm_kernels.cuh"
 #include "selbm_learn.cuh"
+#include "selbm_lines.h"
 #include "selbm_setup.h"
 
 using namespace slb;
@@ -48,6 +49,13 @@ struct selbm {
   // population-split step (prologue + split stages); default for hexahedral meshes at the
   // compiled orders, SELBM_SPLIT=1 / 0 in the environment forces it on / off where compiled
   bool use_split = false;
+  // any-order element kernels of the split step: hexahedra where the fused kernels are not
+  // compiled, and every FP64 order
+  bool use_lines = false;
+  void *d_geo = nullptr;         // planar metrics of curved elements (any-order kernels)
+  int *d_gexp = nullptr;
+  bool split_form() const { return use_split || use_lines; }
+  bool lines_step() const { return use_lines && !(use_split && prec == SELBM_FP32DEV); }
   std::vector<double> Vm_h, Vinv_h;   // modal <-> nodal matrices
   // learned per-element filter control
   bool learned = false;
@@ -165,6 +173,11 @@ cudaError_t upload_real(selbm *h) {
   } else {
     if ((e = upload(&p, cast_vec<Real>(S.drdx)))) return e; h->d_drdx = p; h->allocs.push_back(p);
     if ((e = upload(&p, cast_vec<Real>(S.wJ)))) return e; h->d_wJ = p; h->allocs.push_back(p);
+    if (h->lines_step()) {
+      if ((e = alloc(&h->d_geo, (size_t)S.E * S.Np * 9 * sizeof(LineVal<Real>)))) return e;
+      if ((e = alloc((void **)&h->d_gexp, (size_t)S.E * sizeof(int)))) return e;
+      if ((e = launch_curved_geo<Real>((const Real *)h->d_drdx, S.E, S.Np, (LineVal<Real> *)h->d_geo, h->d_gexp, h->stream))) return e;
+    }
   }
   if ((e = upload(&p, cast_vec<Real>(S.gll.w)))) return e; h->d_gllw = p; h->allocs.push_back(p);
   if ((e = upload(&p, cast_vec<Real>(S.gll.D)))) return e; h->d_D = p; h->allocs.push_back(p);
@@ -300,18 +313,46 @@ SplitHost split_host(selbm *h) {
 template <typename Real>
 cudaError_t launch_split_stage(selbm *h, const KParams<Real> &p) {
   const SplitHost sh = split_host(h);
+  if (h->lines_step()) {
+    const CurvedGeo<Real> cg{(const LineVal<Real> *)h->d_geo, h->d_gexp};
+    return launch_lines_stage<Real>(h->lat, h->S.N, h->S.affine, p, sh, cg, h->stream);
+  }
   cudaError_t err = cudaErrorInvalidValue;
-  if (h->lat == SELBM_D3Q19) split_stage_d3q19<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
-  else if (h->lat == SELBM_D3Q27) split_stage_d3q27<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
+  if constexpr (std::is_same<Real, float>::value) {
+    if (h->lat == SELBM_D3Q19) split_stage_d3q19<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
+    else if (h->lat == SELBM_D3Q27) split_stage_d3q27<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
+  }
   return err;
+}
+
+template <typename Real>
+cudaError_t launch_split_collide(selbm *h, int which, const KParams<Real> &p) {
+  if (h->lat == SELBM_D3Q19) return split_collide_d3q19<Real>(which, p, h->stream);
+  if (h->lat == SELBM_D3Q27) return split_collide_d3q27<Real>(which, p, h->stream);
+  return cudaErrorInvalidValue;
 }
 
 template <typename Real>
 cudaError_t launch_split_prologue(selbm *h, int mode, const KParams<Real> &p, const LearnedPtrs<Real> &lp) {
   const SplitHost sh = split_host(h);
+  if (h->lines_step()) {
+    // filter into f^0; with element transfer functions the mass-weighted average of the copies at
+    // shared nodes; then the collision in place
+    cudaError_t e = launch_lines_filter<Real>(h->lat, h->S.N, p, sh, mode == PRO_LEARNED ? lp.sigma_out : nullptr, p.f0out, h->stream);
+    KParams<Real> q = p;
+    q.fin = p.f0out;
+    if (e == cudaSuccess && mode == PRO_LEARNED) {
+      KParams<Real> a = q;
+      a.A = Real(0); a.B = Real(0); a.has_force = 0; a.dt = Real(0); a.f0 = a.fin; a.fout = p.f0out;
+      e = launch_dss<Real>(h->lat, a, h->stream);
+    }
+    return e == cudaSuccess ? launch_split_collide<Real>(h, 0, q) : e;
+  }
   cudaError_t err = cudaErrorInvalidValue;
-  if (h->lat == SELBM_D3Q19) split_prologue_d3q19<Real>(h->S.N, h->S.affine, mode, p, sh, lp, h->stream, &err);
-  else if (h->lat == SELBM_D3Q27) split_prologue_d3q27<Real>(h->S.N, h->S.affine, mode, p, sh, lp, h->stream, &err);
+  if constexpr (std::is_same<Real, float>::value) {
+    if (h->lat == SELBM_D3Q19) split_prologue_d3q19<Real>(h->S.N, h->S.affine, mode, p, sh, lp, h->stream, &err);
+    else if (h->lat == SELBM_D3Q27) split_prologue_d3q27<Real>(h->S.N, h->S.affine, mode, p, sh, lp, h->stream, &err);
+  }
   return err;
 }
 
@@ -320,13 +361,6 @@ cudaError_t launch_split_prologue(selbm *h, int mode, const KParams<Real> &p, co
 // weighted shares of boundary nodes, the drift check, the assembly + collision of shared nodes
 template <typename Real>
 cudaError_t launch_split_learned(selbm *h, const KParams<Real> &p);
-
-template <typename Real>
-cudaError_t launch_split_collide(selbm *h, int which, const KParams<Real> &p) {
-  if (h->lat == SELBM_D3Q19) return split_collide_d3q19<Real>(which, p, h->stream);
-  if (h->lat == SELBM_D3Q27) return split_collide_d3q27<Real>(which, p, h->stream);
-  return cudaErrorInvalidValue;
-}
 
 template <typename Real>
 LearnedPtrs<Real> learned_ptrs(selbm *h, bool with_drift) {
@@ -343,12 +377,17 @@ cudaError_t launch_split_learned(selbm *h, const KParams<Real> &p) {
   const SplitHost sh = split_host(h);
   const LearnedPtrs<Real> lp = learned_ptrs<Real>(h, true);
   cudaError_t e = cudaErrorInvalidValue;
+  if (!h->use_split) {
+    // orders without the split control: the one-kernel control filters the state, then the collision
+    if ((e = enqueue_learned_filter<Real>(h, p.fin, (Real *)h->FA, true))) return e;
+    return launch_split_collide<Real>(h, 0, p);
+  }
   if (h->lat == SELBM_D3Q19) split_control_d3q19<Real>(h->S.N, p, sh, lp, (Real *)h->d_nq, (Real *)h->d_X, h->d_mass, h->stream, &e);
   else if (h->lat == SELBM_D3Q27) split_control_d3q27<Real>(h->S.N, p, sh, lp, (Real *)h->d_nq, (Real *)h->d_X, h->d_mass, h->stream, &e);
   if (e) return e;
   if ((e = launch_split_prologue<Real>(h, PRO_LEARNED, p, lp))) return e;
   if ((e = launch_drift_check(h->d_acc, h->d_flag, h->mass_bound, h->ke_bound, h->has_force ? 0 : 1, h->stream))) return e;
-  return launch_split_collide<Real>(h, 1, p);
+  return h->lines_step() ? cudaSuccess : launch_split_collide<Real>(h, 1, p);
 }
 
 // one time step of the population-split form: prologue (pending filter + collision,
@@ -408,7 +447,7 @@ cudaError_t enqueue_step_printed(selbm *h, bool apply_filter) {
   const double third[4] = {2.0 / 3.0, 0, 0, 0};
   cudaError_t e;
   // stage 1 (collision and pending filter included): f1 = f0 + dt/3 L f0
-  if (h->use_split) {
+  if (h->split_form()) {
     p.stage = 1; p.A = Real(0); p.B = Real(1);
     p.fin = FA; p.f0out = F0;
     if (apply_filter && h->learned) {
@@ -454,7 +493,7 @@ cudaError_t enqueue_step_printed(selbm *h, bool apply_filter) {
     p.has_force = diff ? 0 : full.has_force;
     p.fS = diff ? nullptr : full.fS;
     p.wall_u = diff ? (const Real *)h->d_wall_u0 : full.wall_u;
-    if (h->use_split) e = launch_split_stage<Real>(h, p);
+    if (h->split_form()) e = launch_split_stage<Real>(h, p);
     else e = launch_stage_any<Real>(h, p);
     if (e) return e;
     if ((e = launch_dss<Real>(h->lat, p, h->stream))) return e;
@@ -473,7 +512,7 @@ cudaError_t enqueue_step(selbm *h, bool apply_filter) {
   }
   if (h->scheme != 0) return enqueue_step_printed<Real>(h, apply_filter);
   KParams<Real> p = base_params<Real>(h);
-  if (h->use_split) return enqueue_step_split<Real>(h, apply_filter);
+  if (h->split_form()) return enqueue_step_split<Real>(h, apply_filter);
   Real *FA = (Real *)h->FA, *F0 = (Real *)h->F0, *F2 = (Real *)h->F2;
   // Shu-Osher weights with A = 1 - B formed in the working precision: A + B = 1 exactly, so a
   // stage combination A f0 + B f' of the deviations carries no systematic scale error (with
@@ -594,6 +633,7 @@ static int create_impl(SetupFn setup, const selbm_params *params, void *cuda_str
     const char *sp = std::getenv("SELBM_SPLIT");
     const bool ok = h->use_fast && S.dim == 3 && split_compiled(h->lat, S.N);
     h->use_split = ok && (sp && sp[0] ? sp[0] == '1' : true);
+    h->use_lines = h->use_fast && S.dim == 3 && lines_compiled(h->rsz, S.N) && (sp && sp[0] ? sp[0] == '1' : true);
   }
   const size_t smem = stage_smem_bytes(h->lat, S.Np, S.n1, h->rsz);
   if (smem > 227 * 1024) { g_create_error = "element tile does not fit in shared memory (use FP32 or a lower order)"; delete h; return SELBM_ERR_ARG; }

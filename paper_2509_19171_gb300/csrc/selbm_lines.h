@@ -1,0 +1,50 @@
+// Any-order element kernels of the population-split step (hexahedra): host interface.
+#pragma once
+#include <type_traits>
+
+#include "selbm_kernels.cuh"
+
+namespace slb {
+
+template <typename Real>
+using LineVal = std::conditional_t<sizeof(Real) == 8, long long, float>;   // a line's value
+
+// velocity set at run time
+struct LatticeRT {
+  int Q;
+  uint32_t pos[3], neg[3];
+  float tf[27];
+  double td[27];
+  signed char opp[27];
+  template <typename Real>
+  __device__ __forceinline__ Real t(int a) const {
+    if constexpr (sizeof(Real) == 8) return td[a];
+    else return tf[a];
+  }
+};
+
+// planar metrics of curved elements: dr_l/dx_k [E][9][Np] (component 3 l + k); FP64: fixed point,
+// times 2^gexp[e]
+template <typename Real>
+struct CurvedGeo {
+  const LineVal<Real> *g;
+  const int *gexp;
+};
+
+// orders whose element tile fits the step's other kernels too (real_size 4 or 8)
+inline bool lines_compiled(int real_size, int N) { return N >= 2 && N <= (real_size == 8 ? 9 : 11); }
+
+// one Runge-Kutta stage of the element kernels (see selbm_split_stage.cuh for its terms)
+template <typename Real>
+cudaError_t launch_lines_stage(int lat, int N, bool affine, const KParams<Real> &p, const SplitHost &h,
+                               const CurvedGeo<Real> &cg, cudaStream_t s);
+// filtered p.fin: sigma NULL: the fixed filter, every unique node to out; else element transfer
+// functions sigma [E][n], element-interior nodes to out and shares wJ f of the others to p.T
+template <typename Real>
+cudaError_t launch_lines_filter(int lat, int N, const KParams<Real> &p, const SplitHost &h, const Real *sigma, Real *out,
+                                cudaStream_t s);
+// planar metrics from drdx [E][Np][9]
+template <typename Real>
+cudaError_t launch_curved_geo(const Real *drdx, int E, int Np, LineVal<Real> *g, int *gexp, cudaStream_t s);
+
+}  // namespace slb

@@ -1,4 +1,4 @@
-// Instantiations of the per-element prologue (pending filter + collision) for
+// Instantiations of the FP32 per-element prologue (pending filter + collision) for
 // D3Q19 (orders: 4 7).
 #include "selbm_split.cuh"
 
@@ -26,8 +26,6 @@ bool split_prologue_d3q19(int N, bool affine, int mode, const KParams<Real> &p, 
 
 template bool split_prologue_d3q19<float>(int, bool, int, const KParams<float> &, const SplitHost &,
                                          const LearnedPtrs<float> &, cudaStream_t, cudaError_t *);
-template bool split_prologue_d3q19<double>(int, bool, int, const KParams<double> &, const SplitHost &,
-                                          const LearnedPtrs<double> &, cudaStream_t, cudaError_t *);
 
 // learned control of the split form (node features, element network) -> lp.sigma_out
 template <typename Real>
