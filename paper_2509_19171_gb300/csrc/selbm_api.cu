@@ -102,6 +102,7 @@ struct selbm {
   int32_t *d_wall_off = nullptr, *d_first = nullptr;
   uint8_t *d_owner = nullptr;
   double *d_mass = nullptr, *d_partial = nullptr, *d_diag = nullptr;
+  double *d_fld = nullptr;       // [1 + dim][G] rho and u on unique nodes (allocated on first use)
   double *d_io = nullptr;  // staging for host <-> device FP64 arrays
   size_t io_bytes = 0;
   std::vector<void *> allocs;
@@ -332,20 +333,26 @@ cudaError_t launch_split_collide(selbm *h, int which, const KParams<Real> &p) {
   return cudaErrorInvalidValue;
 }
 
+// filtered p.fin on unique nodes (any-order kernels): the fixed filter, or with element transfer
+// functions sigma the mass-weighted average of the copies at shared nodes
+template <typename Real>
+cudaError_t launch_filter(selbm *h, const KParams<Real> &p, const Real *sigma, Real *out) {
+  cudaError_t e = launch_lines_filter<Real>(h->lat, h->S.N, p, split_host(h), sigma, out, h->stream);
+  if (e != cudaSuccess || !sigma) return e;
+  KParams<Real> a = p;
+  a.A = Real(0); a.B = Real(0); a.has_force = 0; a.dt = Real(0);
+  a.fin = out; a.f0 = out; a.fout = out;
+  return launch_dss<Real>(h->lat, a, h->stream);
+}
+
 template <typename Real>
 cudaError_t launch_split_prologue(selbm *h, int mode, const KParams<Real> &p, const LearnedPtrs<Real> &lp) {
   const SplitHost sh = split_host(h);
   if (h->lines_step()) {
-    // filter into f^0; with element transfer functions the mass-weighted average of the copies at
-    // shared nodes; then the collision in place
-    cudaError_t e = launch_lines_filter<Real>(h->lat, h->S.N, p, sh, mode == PRO_LEARNED ? lp.sigma_out : nullptr, p.f0out, h->stream);
+    // filter into f^0, then the collision in place
+    const cudaError_t e = launch_filter<Real>(h, p, mode == PRO_LEARNED ? lp.sigma_out : nullptr, p.f0out);
     KParams<Real> q = p;
     q.fin = p.f0out;
-    if (e == cudaSuccess && mode == PRO_LEARNED) {
-      KParams<Real> a = q;
-      a.A = Real(0); a.B = Real(0); a.has_force = 0; a.dt = Real(0); a.f0 = a.fin; a.fout = p.f0out;
-      e = launch_dss<Real>(h->lat, a, h->stream);
-    }
     return e == cudaSuccess ? launch_split_collide<Real>(h, 0, q) : e;
   }
   cudaError_t err = cudaErrorInvalidValue;
@@ -372,19 +379,26 @@ LearnedPtrs<Real> learned_ptrs(selbm *h, bool with_drift) {
   return lp;
 }
 
+// transfer functions of every element from the state p.fin (split form)
+template <typename Real>
+cudaError_t launch_split_control(selbm *h, const KParams<Real> &p, const LearnedPtrs<Real> &lp) {
+  const SplitHost sh = split_host(h);
+  cudaError_t e = cudaErrorInvalidValue;
+  if (h->lat == SELBM_D3Q19) split_control_d3q19<Real>(h->S.N, p, sh, lp, (Real *)h->d_nq, (Real *)h->d_X, h->d_mass, h->stream, &e);
+  else if (h->lat == SELBM_D3Q27) split_control_d3q27<Real>(h->S.N, p, sh, lp, (Real *)h->d_nq, (Real *)h->d_X, h->d_mass, h->stream, &e);
+  return e;
+}
+
 template <typename Real>
 cudaError_t launch_split_learned(selbm *h, const KParams<Real> &p) {
-  const SplitHost sh = split_host(h);
   const LearnedPtrs<Real> lp = learned_ptrs<Real>(h, true);
-  cudaError_t e = cudaErrorInvalidValue;
+  cudaError_t e;
   if (!h->use_split) {
     // orders without the split control: the one-kernel control filters the state, then the collision
     if ((e = enqueue_learned_filter<Real>(h, p.fin, (Real *)h->FA, true))) return e;
     return launch_split_collide<Real>(h, 0, p);
   }
-  if (h->lat == SELBM_D3Q19) split_control_d3q19<Real>(h->S.N, p, sh, lp, (Real *)h->d_nq, (Real *)h->d_X, h->d_mass, h->stream, &e);
-  else if (h->lat == SELBM_D3Q27) split_control_d3q27<Real>(h->S.N, p, sh, lp, (Real *)h->d_nq, (Real *)h->d_X, h->d_mass, h->stream, &e);
-  if (e) return e;
+  if ((e = launch_split_control<Real>(h, p, lp))) return e;
   if ((e = launch_split_prologue<Real>(h, PRO_LEARNED, p, lp))) return e;
   if ((e = launch_drift_check(h->d_acc, h->d_flag, h->mass_bound, h->ke_bound, h->has_force ? 0 : 1, h->stream))) return e;
   return h->lines_step() ? cudaSuccess : launch_split_collide<Real>(h, 1, p);
@@ -545,13 +559,22 @@ cudaError_t enqueue_step(selbm *h, bool apply_filter) {
   return cudaSuccess;
 }
 
+bool filter_waits(const selbm *h) { return h->filter_pending && (h->filter_on || h->learned); }
+
+// pending filter of the last step into BUF
 template <typename Real>
 cudaError_t enqueue_finalize(selbm *h) {
   KParams<Real> p = base_params<Real>(h);
   p.fin = (const Real *)h->FA;
   p.fout = (Real *)h->BUF;
-  if (h->filter_pending && h->learned) return enqueue_learned_filter<Real>(h, (const Real *)h->FA, (Real *)h->BUF, false);
-  p.apply_filter = (h->filter_pending && h->filter_on) ? 1 : 0;
+  if (h->learned) {
+    if (!(h->use_lines && h->use_split)) return enqueue_learned_filter<Real>(h, (const Real *)h->FA, (Real *)h->BUF, false);
+    const LearnedPtrs<Real> lp = learned_ptrs<Real>(h, false);
+    const cudaError_t e = launch_split_control<Real>(h, p, lp);
+    return e == cudaSuccess ? launch_filter<Real>(h, p, lp.sigma_out, (Real *)h->BUF) : e;
+  }
+  if (h->use_lines) return launch_filter<Real>(h, p, nullptr, (Real *)h->BUF);
+  p.apply_filter = 1;
   return launch_finalize<Real>(h->lat, p, h->stream);
 }
 
@@ -591,6 +614,41 @@ int fallback_status(selbm *h) {
   cudaError_t e = cudaMemcpy(&flag, h->d_flag, sizeof(int), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return h->cuda_fail(e, "fallback flag");
   return flag ? SELBM_OK_FALLBACK : SELBM_OK;
+}
+
+int finalize(selbm *h) {
+  cudaError_t e = h->prec == SELBM_FP64 ? enqueue_finalize<double>(h) : enqueue_finalize<float>(h);
+  if (e != cudaSuccess) return h->cuda_fail(e, "finalize");
+  return SELBM_OK;
+}
+
+// the filtered state on unique nodes: the state itself when no filter is pending
+int filtered_state(selbm *h, const void **f) {
+  *f = h->FA;
+  if (!filter_waits(h)) return SELBM_OK;
+  *f = h->BUF;
+  return finalize(h);
+}
+
+// rho and u of a state on unique nodes -> d_fld [1 + dim][G] (kept by the handle); diag: the
+// quadrature sums into d_diag too
+int node_fields(selbm *h, const void *f, bool diag) {
+  const size_t G = h->S.G;
+  if (!h->d_fld) {
+    cudaError_t e = cudaMalloc((void **)&h->d_fld, (1 + (size_t)h->S.dim) * G * sizeof(double));
+    if (e != cudaSuccess) {
+      h->d_fld = nullptr;
+      return h->cuda_fail(e, "field buffer");
+    }
+    h->allocs.push_back(h->d_fld);
+  }
+  auto run = [&](auto tag) -> cudaError_t {
+    using Real = decltype(tag);
+    return diag ? launch_diag<Real>(h->lat, (const Real *)f, h->d_mass, h->S.G, h->Gs(), h->P.rho0, h->d_fld, h->d_partial, h->d_diag, h->stream)
+                : launch_node_fields<Real>(h->lat, (const Real *)f, h->S.G, h->Gs(), h->P.rho0, h->d_fld, h->stream);
+  };
+  const cudaError_t e = h->prec == SELBM_FP64 ? run(double()) : run(float());
+  return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "moments");
 }
 
 int ensure_io(selbm *h, size_t bytes) {
@@ -790,16 +848,11 @@ int selbm_set_state(selbm_t *h, const double *f, int on_device) {
   return SELBM_OK;
 }
 
-static int finalize(selbm *h) {
-  cudaError_t e = h->prec == SELBM_FP64 ? enqueue_finalize<double>(h) : enqueue_finalize<float>(h);
-  if (e != cudaSuccess) return h->cuda_fail(e, "finalize");
-  return SELBM_OK;
-}
-
 int selbm_get_state(selbm_t *h, double *f, int on_device) {
   if (!h || !f) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
-  int rc = finalize(h);
+  const void *view;
+  int rc = filtered_state(h, &view);
   if (rc) return rc;
   const size_t nl = h->nloc(), bytes = (size_t)h->Q * nl * 8;
   double *df = f;
@@ -808,8 +861,8 @@ int selbm_get_state(selbm_t *h, double *f, int on_device) {
     df = h->d_io;
   }
   cudaError_t e = h->prec == SELBM_FP64
-                      ? launch_get_state<double>(h->lat, (const double *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, df, h->stream)
-                      : launch_get_state<float>(h->lat, (const float *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, df, h->stream);
+                      ? launch_get_state<double>(h->lat, (const double *)view, h->d_l2g, h->Gs(), nl, h->P.rho0, df, h->stream)
+                      : launch_get_state<float>(h->lat, (const float *)view, h->d_l2g, h->Gs(), nl, h->P.rho0, df, h->stream);
   if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(f, df, bytes, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "get_state");
@@ -848,7 +901,7 @@ int selbm_step(selbm_t *h, int64_t nsteps) {
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
   if (nsteps < 0) return h->fail(SELBM_ERR_ARG, "nsteps < 0");
   for (int64_t k = 0; k < nsteps; ++k) {
-    const bool filt = h->filter_pending && (h->filter_on || h->learned);
+    const bool filt = filter_waits(h);
     const int slot = filt ? 1 : 0;
     cudaError_t e = cudaSuccess;
     const bool graphable = h->graph_enabled && !h->timing;
@@ -870,17 +923,16 @@ int selbm_step(selbm_t *h, int64_t nsteps) {
 int selbm_moments(selbm_t *h, double *rho, double *u, int on_device) {
   if (!h || !rho || !u) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
-  int rc = finalize(h);
-  if (rc) return rc;
+  const void *view;
+  int rc = filtered_state(h, &view);
+  if (rc || (rc = node_fields(h, view, false))) return rc;
   const size_t nl = h->nloc(), d = h->S.dim;
   double *dr = rho, *du = u;
   if (!on_device) {
     if ((rc = ensure_io(h, nl * (1 + d) * 8))) return rc;
     dr = h->d_io; du = h->d_io + nl;
   }
-  cudaError_t e = h->prec == SELBM_FP64
-                      ? launch_moments<double>(h->lat, (const double *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, dr, du, h->stream)
-                      : launch_moments<float>(h->lat, (const float *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, dr, du, h->stream);
+  cudaError_t e = launch_expand_fields((int)d, h->d_fld, h->S.G, h->d_l2g, nl, dr, du, h->stream);
   if (e == cudaSuccess && !on_device) {
     e = cudaMemcpyAsync(rho, dr, nl * 8, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(u, du, nl * d * 8, cudaMemcpyDeviceToHost, h->stream);
@@ -893,7 +945,8 @@ int selbm_moments(selbm_t *h, double *rho, double *u, int on_device) {
 int selbm_stress(selbm_t *h, double *pi, int on_device) {
   if (!h || !pi) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
-  int rc = finalize(h);
+  const void *view;
+  int rc = filtered_state(h, &view);
   if (rc) return rc;
   const size_t nl = h->nloc(), d = h->S.dim, n = nl * d * d;
   double *dp = pi;
@@ -909,10 +962,10 @@ int selbm_stress(selbm_t *h, double *pi, int on_device) {
   const double factor = h->tau / (h->tau + 0.5);
   const double *g = h->P.body_accel;
   cudaError_t e = h->prec == SELBM_FP64
-                      ? launch_stress<double>(h->lat, (const double *)h->BUF, h->d_l2g, h->S.G, h->Gs(), nl, h->P.rho0, 0.5 * h->dt,
+                      ? launch_stress<double>(h->lat, (const double *)view, h->d_l2g, h->S.G, h->Gs(), nl, h->P.rho0, 0.5 * h->dt,
                                               factor, g, h->has_force, h->field_on ? (const double *)h->d_fS : nullptr,
                                               amp, dp, h->stream)
-                      : launch_stress<float>(h->lat, (const float *)h->BUF, h->d_l2g, h->S.G, h->Gs(), nl, h->P.rho0, 0.5 * h->dt,
+                      : launch_stress<float>(h->lat, (const float *)view, h->d_l2g, h->S.G, h->Gs(), nl, h->P.rho0, 0.5 * h->dt,
                                              factor, g, h->has_force, h->field_on ? (const float *)h->d_fS : nullptr,
                                              amp, dp, h->stream);
   if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(pi, dp, n * 8, cudaMemcpyDeviceToHost, h->stream);
@@ -923,7 +976,7 @@ int selbm_stress(selbm_t *h, double *pi, int on_device) {
 
 int selbm_set_filter(selbm_t *h, const selbm_filter *f) {
   if (!h || !f) return SELBM_ERR_ARG;
-  if (h->filter_pending && (h->filter_on || h->learned)) {
+  if (filter_waits(h)) {
     // the last step's filter (old settings) must be applied before switching
     int rc = finalize(h);
     if (rc) return rc;
@@ -1010,30 +1063,23 @@ int selbm_set_force_field(selbm_t *h, const double *S, double period, double t_e
 int selbm_diagnostics(selbm_t *h, double out[8]) {
   if (!h || !out) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
-  int rc = finalize(h);
-  if (rc) return rc;
-  cudaError_t e = h->prec == SELBM_FP64
-                      ? launch_diag<double>(h->lat, (const double *)h->BUF, h->d_mass, h->S.G, h->Gs(), h->P.rho0, h->d_partial, h->d_diag, h->stream)
-                      : launch_diag<float>(h->lat, (const float *)h->BUF, h->d_mass, h->S.G, h->Gs(), h->P.rho0, h->d_partial, h->d_diag, h->stream);
+  const void *view;
+  int rc = filtered_state(h, &view);
+  if (rc || (rc = node_fields(h, view, true))) return rc;
   // dissipation: velocity at local nodes, then per-element gradient integrals
   const size_t nl = h->nloc(), dim = h->S.dim;
-  double *d_eps = nullptr;
-  if (e == cudaSuccess && ensure_io(h, nl * (1 + dim) * 8 + (h->S.E + 1) * 8) != SELBM_OK) e = cudaErrorMemoryAllocation;
+  if ((rc = ensure_io(h, nl * (1 + dim) * 8 + (h->S.E + 1) * 8))) return rc;
+  double *u_l = h->d_io + nl, *part = h->d_io + nl * (1 + dim), *d_eps = h->d_diag + 6;
+  cudaError_t e = launch_expand_fields((int)dim, h->d_fld, h->S.G, h->d_l2g, nl, nullptr, u_l, h->stream);
   if (e == cudaSuccess) {
-    double *rho_l = h->d_io, *u_l = h->d_io + nl, *part = h->d_io + nl * (1 + dim);
-    d_eps = h->d_diag + 6;
     const double mu = h->P.rho0 * h->P.nu;
     e = h->prec == SELBM_FP64
-            ? launch_moments<double>(h->lat, (const double *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, rho_l, u_l, h->stream)
-            : launch_moments<float>(h->lat, (const float *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, rho_l, u_l, h->stream);
-    if (e == cudaSuccess)
-      e = h->prec == SELBM_FP64
-              ? launch_eps<double>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const double *)h->d_el_drdx,
-                                   (const double *)h->d_drdx, (const double *)h->d_el_J, (const double *)h->d_wJ,
-                                   (const double *)h->d_gllw, (const double *)h->d_D, mu, part, d_eps, h->stream)
-              : launch_eps<float>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const float *)h->d_el_drdx,
-                                  (const float *)h->d_drdx, (const float *)h->d_el_J, (const float *)h->d_wJ,
-                                  (const float *)h->d_gllw, (const float *)h->d_D, mu, part, d_eps, h->stream);
+            ? launch_eps<double>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const double *)h->d_el_drdx,
+                                 (const double *)h->d_drdx, (const double *)h->d_el_J, (const double *)h->d_wJ,
+                                 (const double *)h->d_gllw, (const double *)h->d_D, mu, part, d_eps, h->stream)
+            : launch_eps<float>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const float *)h->d_el_drdx,
+                                (const float *)h->d_drdx, (const float *)h->d_el_J, (const float *)h->d_wJ,
+                                (const float *)h->d_gllw, (const float *)h->d_D, mu, part, d_eps, h->stream);
   }
   double tmp[7];
   if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, h->d_diag, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
@@ -1056,15 +1102,14 @@ int selbm_wall_stress(selbm_t *h, const double dir[3], double *tau) {
   for (int c = 0; c < 3; ++c) d[c] /= std::sqrt(nrm);
   *tau = 0.0;
   if (h->n_wallpts == 0) return SELBM_OK;
-  int rc = finalize(h);
-  if (rc) return rc;
+  const void *view;
+  int rc = filtered_state(h, &view);
+  if (rc || (rc = node_fields(h, view, false))) return rc;
   const size_t nl = h->nloc();
   if ((rc = ensure_io(h, (nl * (1 + dim) + 2 * (size_t)h->n_wallpts) * 8))) return rc;
-  double *rho_l = h->d_io, *u_l = h->d_io + nl, *part = h->d_io + nl * (1 + dim);
+  double *u_l = h->d_io + nl, *part = h->d_io + nl * (1 + dim);
   const double mu = h->P.rho0 * h->P.nu;
-  cudaError_t e = h->prec == SELBM_FP64
-                      ? launch_moments<double>(h->lat, (const double *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, rho_l, u_l, h->stream)
-                      : launch_moments<float>(h->lat, (const float *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, rho_l, u_l, h->stream);
+  cudaError_t e = launch_expand_fields(dim, h->d_fld, h->S.G, h->d_l2g, nl, nullptr, u_l, h->stream);
   if (e == cudaSuccess)
     e = h->prec == SELBM_FP64
             ? launch_wall_stress<double>(u_l, dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const double *)h->d_el_drdx,
@@ -1095,8 +1140,9 @@ int selbm_radial_profile(selbm_t *h, const double origin[3], const double axis[3
   if (!(nrm > 0)) return h->fail(SELBM_ERR_ARG, "radial_profile: zero axis");
   for (int c = 0; c < 3; ++c) a[c] /= std::sqrt(nrm);
   const double o[3] = {origin[0], origin[1], dim == 3 ? origin[2] : 0.0};
-  int rc = finalize(h);
-  if (rc) return rc;
+  const void *view;
+  int rc = filtered_state(h, &view);
+  if (rc || (rc = node_fields(h, view, false))) return rc;
   cudaError_t e = cudaSuccess;
   if (!h->d_xg) {
     std::vector<double> xg((size_t)h->S.G * dim);
@@ -1105,16 +1151,10 @@ int selbm_radial_profile(selbm_t *h, const double origin[3], const double axis[3
     e = upload(&h->d_xg, xg);
     if (e != cudaSuccess) return h->cuda_fail(e, "radial_profile");
   }
-  const size_t nl = h->nloc();
   const int blocks = 256;
-  if ((rc = ensure_io(h, (nl * (1 + dim) + (size_t)blocks * 2 * nbins) * 8))) return rc;
-  double *rho_l = h->d_io, *u_l = h->d_io + nl, *part = h->d_io + nl * (1 + dim);
-  e = h->prec == SELBM_FP64
-          ? launch_moments<double>(h->lat, (const double *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, rho_l, u_l, h->stream)
-          : launch_moments<float>(h->lat, (const float *)h->BUF, h->d_l2g, h->Gs(), nl, h->P.rho0, rho_l, u_l, h->stream);
-  if (e == cudaSuccess)
-    e = launch_radial_profile(u_l, dim, h->d_first, h->d_xg, h->d_mass, h->S.G, o, a, radius, nbins, blocks, part,
-                              h->stream);
+  if ((rc = ensure_io(h, (size_t)blocks * 2 * nbins * 8))) return rc;
+  double *part = h->d_io;
+  e = launch_radial_profile(h->d_fld + h->S.G, dim, h->d_xg, h->d_mass, h->S.G, o, a, radius, nbins, blocks, part, h->stream);
   std::vector<double> hp((size_t)blocks * 2 * nbins);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hp.data(), part, hp.size() * 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
@@ -1194,7 +1234,7 @@ int selbm_set_learned_filter(selbm_t *h, const float *params, const float *lo, c
     return h->fail(SELBM_ERR_ARG, "learned filter: element tile does not fit in shared memory (use FP32 or a lower order)");
   for (int i = 0; i < nin; ++i)
     if (!(hi[i] > lo[i])) return h->fail(SELBM_ERR_ARG, "learned filter: hi must exceed lo for every feature");
-  if (h->filter_pending && (h->filter_on || h->learned)) {
+  if (filter_waits(h)) {
     // apply the pending filter with the old settings first
     int rc = finalize(h);
     if (rc) return rc;

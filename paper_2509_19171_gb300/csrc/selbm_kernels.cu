@@ -424,66 +424,11 @@ cudaError_t launch_finalize(int lat, const KParams<Real> &p, cudaStream_t s) {
 // state import / export and diagnostics
 // ---------------------------------------------------------------------------
 
-// f_bar = f^eq(rho, u) - dt/2 F** stored as g = f_bar - t rho0 (Sec. 2.1, f at equilibrium)
-template <typename Real, int LAT>
-__global__ void init_kernel(const double *rho, const double *u, const int32_t *first, int G, int Gs, double rho0,
-                            double half_dt, double gx, double gy, double gz, int has_force, const Real *fS,
-                            double amp, Real *out) {
-  constexpr int Q = Lat<LAT>::Q, DIM = Lat<LAT>::D;
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-    const size_t q = first[g];
-    const double r = rho[q];
-    double uv[3] = {0, 0, 0}, F[3] = {0, 0, 0}, gg[3] = {gx, gy, gz};
-    if (fS)
-      for (int k = 0; k < 3; ++k) gg[k] += amp * (double)fS[(size_t)k * G + g];
-    double uu = 0, uF = 0;
-    for (int k = 0; k < DIM; ++k) {
-      uv[k] = u[q * DIM + k];
-      uu += uv[k] * uv[k];
-      F[k] = has_force ? r * gg[k] : 0.0;
-      uF += uv[k] * F[k];
-    }
-    for (int a = 0; a < Q; ++a) {
-      double eu = 0, eF = 0;
-      for (int k = 0; k < DIM; ++k) { eu += c_e[LAT][a][k] * uv[k]; eF += c_e[LAT][a][k] * F[k]; }
-      const double t = c_td[LAT][a];
-      const double feq = t * r * (1.0 + 3.0 * eu + 4.5 * eu * eu - 1.5 * uu);
-      const double Fss = t * (9.0 * eu * eF - 3.0 * uF);
-      out[(size_t)a * Gs + g] = (Real)(feq - half_dt * Fss - t * rho0);
-    }
-  }
-}
-
 template <typename Real, int LAT>
 __global__ void set_state_kernel(const double *f, const int32_t *first, int G, int Gs, size_t nloc, double rho0, Real *out) {
   constexpr int Q = Lat<LAT>::Q;
   for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x)
     for (int a = 0; a < Q; ++a) out[(size_t)a * Gs + g] = (Real)(f[(size_t)a * nloc + first[g]] - c_td[LAT][a] * rho0);
-}
-
-template <typename Real, int LAT>
-__global__ void get_state_kernel(const Real *buf, const int32_t *l2g, int Gs, size_t nloc, double rho0, double *f) {
-  constexpr int Q = Lat<LAT>::Q;
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < nloc; q += (size_t)gridDim.x * blockDim.x)
-    for (int a = 0; a < Q; ++a) f[(size_t)a * nloc + q] = (double)buf[(size_t)a * Gs + l2g[q]] + c_td[LAT][a] * rho0;
-}
-
-// rho = sum f_bar, rho u = sum e f_bar at every local node (FP64 sums)
-template <typename Real, int LAT>
-__global__ void moments_kernel(const Real *buf, const int32_t *l2g, int Gs, size_t nloc, double rho0, double *rho, double *u) {
-  constexpr int Q = Lat<LAT>::Q, DIM = Lat<LAT>::D;
-  for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < nloc; q += (size_t)gridDim.x * blockDim.x) {
-    const size_t g = l2g[q];
-    double d = 0, j[3] = {0, 0, 0};
-    for (int a = 0; a < Q; ++a) {
-      const double v = (double)buf[(size_t)a * Gs + g];
-      d += v;
-      for (int k = 0; k < DIM; ++k) j[k] += c_e[LAT][a][k] * v;
-    }
-    const double r = rho0 + d;
-    rho[q] = r;
-    for (int k = 0; k < DIM; ++k) u[q * DIM + k] = j[k] / r;
-  }
 }
 
 // non-equilibrium second moment at every local node, Pi_ij = factor sum_a e_ai e_aj (f_a - f_a^eq
@@ -528,37 +473,6 @@ __global__ void stress_kernel(const Real *buf, const int32_t *l2g, int G, int Gs
     for (int i = 0; i < DIM; ++i)
       for (int k = 0; k < DIM; ++k) out[(q * DIM + i) * DIM + k] = factor * pi[i][k];
   }
-}
-
-// per-block partial sums: mass, momentum[3], KE, non-finite count (deterministic two-pass)
-template <typename Real, int LAT>
-__global__ void diag_partial_kernel(const Real *buf, const double *mass, int G, int Gs, double rho0, double *partial) {
-  constexpr int Q = Lat<LAT>::Q, DIM = Lat<LAT>::D;
-  __shared__ double red[6][256];
-  double acc[6] = {0, 0, 0, 0, 0, 0};
-  for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < G; g += gridDim.x * blockDim.x) {
-    double d = 0, j[3] = {0, 0, 0};
-    for (int a = 0; a < Q; ++a) {
-      const double v = (double)buf[(size_t)a * Gs + g];
-      if (!isfinite(v)) acc[5] += 1.0;
-      d += v;
-      for (int k = 0; k < DIM; ++k) j[k] += c_e[LAT][a][k] * v;
-    }
-    const double r = rho0 + d, M = mass[g];
-    acc[0] += M * r;
-    double uu = 0;
-    for (int k = 0; k < DIM; ++k) { acc[1 + k] += M * j[k]; uu += (j[k] / r) * (j[k] / r); }
-    acc[4] += 0.5 * rho0 * M * uu;
-  }
-  for (int c = 0; c < 6; ++c) red[c][threadIdx.x] = acc[c];
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s)
-      for (int c = 0; c < 6; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + s];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0)
-    for (int c = 0; c < 6; ++c) partial[blockIdx.x * 6 + c] = red[c][0];
 }
 
 // viscous dissipation integral of the velocity u [E][Np][dim] (local nodes):
@@ -644,15 +558,6 @@ template cudaError_t launch_eps<float>(const double *, int, int, int, int, int, 
                                        const float *, const float *, const float *, const float *, double, double *,
                                        double *, cudaStream_t);
 
-__global__ void diag_final_kernel(const double *partial, int nblocks, double *out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double acc[6] = {0, 0, 0, 0, 0, 0};
-    for (int b = 0; b < nblocks; ++b)
-      for (int c = 0; c < 6; ++c) acc[c] += partial[b * 6 + c];
-    for (int c = 0; c < 6; ++c) out[c] = acc[c];
-  }
-}
-
 static int grid_for(size_t n, int threads) { return (int)std::min<size_t>((n + threads - 1) / threads, 152 * 16); }
 
 #define SELBM_LAT_SWITCH(lat, CALL)                  \
@@ -662,14 +567,6 @@ static int grid_for(size_t n, int threads) { return (int)std::min<size_t>((n + t
     case SELBM_D3Q27: { constexpr int L = SELBM_D3Q27; CALL; } break; \
     default: return cudaErrorInvalidValue;           \
   }
-
-template <typename Real>
-cudaError_t launch_init(int lat, const double *rho, const double *u, const int32_t *first, int G, int Gs, double rho0,
-                        double half_dt, const double g[3], int has_force, const Real *fS, double amp, Real *out,
-                        cudaStream_t s) {
-  SELBM_LAT_SWITCH(lat, (init_kernel<Real, L><<<grid_for(G, 256), 256, 0, s>>>(rho, u, first, G, Gs, rho0, half_dt, g[0], g[1], g[2], has_force, fS, amp, out)));
-  return cudaGetLastError();
-}
 
 template <typename Real>
 __global__ void combine_kernel(size_t n, const Real *f0, const Real *f1, const Real *f2, const Real *f3, int m,
@@ -728,16 +625,6 @@ cudaError_t launch_set_state(int lat, const double *f, const int32_t *first, int
   return cudaGetLastError();
 }
 template <typename Real>
-cudaError_t launch_get_state(int lat, const Real *buf, const int32_t *l2g, int Gs, size_t nloc, double rho0, double *f, cudaStream_t s) {
-  SELBM_LAT_SWITCH(lat, (get_state_kernel<Real, L><<<grid_for(nloc, 256), 256, 0, s>>>(buf, l2g, Gs, nloc, rho0, f)));
-  return cudaGetLastError();
-}
-template <typename Real>
-cudaError_t launch_moments(int lat, const Real *buf, const int32_t *l2g, int Gs, size_t nloc, double rho0, double *rho, double *u, cudaStream_t s) {
-  SELBM_LAT_SWITCH(lat, (moments_kernel<Real, L><<<grid_for(nloc, 256), 256, 0, s>>>(buf, l2g, Gs, nloc, rho0, rho, u)));
-  return cudaGetLastError();
-}
-template <typename Real>
 cudaError_t launch_stress(int lat, const Real *buf, const int32_t *l2g, int G, int Gs, size_t nloc, double rho0, double half_dt,
                           double factor, const double g[3], int has_force, const Real *fS, double amp, double *out,
                           cudaStream_t s) {
@@ -745,27 +632,14 @@ cudaError_t launch_stress(int lat, const Real *buf, const int32_t *l2g, int G, i
                              buf, l2g, G, Gs, nloc, rho0, half_dt, factor, g[0], g[1], g[2], has_force, fS, amp, out)));
   return cudaGetLastError();
 }
-int diag_blocks() { return 152 * 4; }
-template <typename Real>
-cudaError_t launch_diag(int lat, const Real *buf, const double *mass, int G, int Gs, double rho0, double *partial, double *out, cudaStream_t s) {
-  SELBM_LAT_SWITCH(lat, (diag_partial_kernel<Real, L><<<diag_blocks(), 256, 0, s>>>(buf, mass, G, Gs, rho0, partial)));
-  diag_final_kernel<<<1, 32, 0, s>>>(partial, diag_blocks(), out);
-  return cudaGetLastError();
-}
-
 #define SELBM_INST_UTIL(Real)                                                                                              \
-  template cudaError_t launch_init<Real>(int, const double *, const double *, const int32_t *, int, int, double, double,      \
-                                         const double[3], int, const Real *, double, Real *, cudaStream_t);              \
   template cudaError_t launch_force_field<Real>(const double *, const int32_t *, int, int, Real *, cudaStream_t);         \
   template cudaError_t launch_combine<Real>(size_t, const Real *, const Real *, const Real *, const Real *, int,         \
                                             const double[4], const Real *, double, Real *, Real *, cudaStream_t);        \
   template cudaError_t launch_force_amp<Real>(double *, Real *, double, double, double, cudaStream_t);                    \
   template cudaError_t launch_stress<Real>(int, const Real *, const int32_t *, int, int, size_t, double, double, double,        \
                                            const double[3], int, const Real *, double, double *, cudaStream_t);          \
-  template cudaError_t launch_set_state<Real>(int, const double *, const int32_t *, int, int, size_t, double, Real *, cudaStream_t); \
-  template cudaError_t launch_get_state<Real>(int, const Real *, const int32_t *, int, size_t, double, double *, cudaStream_t); \
-  template cudaError_t launch_moments<Real>(int, const Real *, const int32_t *, int, size_t, double, double *, double *, cudaStream_t); \
-  template cudaError_t launch_diag<Real>(int, const Real *, const double *, int, int, double, double *, double *, cudaStream_t);
+  template cudaError_t launch_set_state<Real>(int, const double *, const int32_t *, int, int, size_t, double, Real *, cudaStream_t);
 SELBM_INST_UTIL(double)
 SELBM_INST_UTIL(float)
 

@@ -101,11 +101,17 @@ template <typename Real>
 cudaError_t launch_set_state(int lat, const double *f, const int32_t *first, int G, int Gs, size_t nloc, double rho0, Real *out, cudaStream_t s);
 template <typename Real>
 cudaError_t launch_get_state(int lat, const Real *buf, const int32_t *l2g, int Gs, size_t nloc, double rho0, double *f, cudaStream_t s);
+// rho and u on unique nodes, fld [1 + dim][G]
 template <typename Real>
-cudaError_t launch_moments(int lat, const Real *buf, const int32_t *l2g, int Gs, size_t nloc, double rho0, double *rho, double *u, cudaStream_t s);
+cudaError_t launch_node_fields(int lat, const Real *buf, int G, int Gs, double rho0, double *fld, cudaStream_t s);
+// the same with the sums out[0..5]: mass, momentum[3], kinetic energy, non-finite entries
 int diag_blocks();
 template <typename Real>
-cudaError_t launch_diag(int lat, const Real *buf, const double *mass, int G, int Gs, double rho0, double *partial, double *out, cudaStream_t s);
+cudaError_t launch_diag(int lat, const Real *buf, const double *mass, int G, int Gs, double rho0, double *fld, double *partial,
+                        double *out, cudaStream_t s);
+// fields of unique nodes to local nodes: rho [nloc] (or NULL), u [nloc][dim]
+cudaError_t launch_expand_fields(int dim, const double *fld, int G, const int32_t *l2g, size_t nloc, double *rho, double *u,
+                                 cudaStream_t s);
 
 // host copies of the matrices of the register-blocked stage kernel
 struct FastHost {
@@ -170,8 +176,8 @@ template <typename Real>
 cudaError_t launch_wall_stress(const double *u, int dim, int n, int Np, int E, int affine, const Real *el_drdx,
                                const Real *drdx, const Real *Dm, const void *walls, const int32_t *wall_off,
                                const double dir[3], double mu, double *out, cudaStream_t s);
-cudaError_t launch_radial_profile(const double *u, int dim, const int32_t *first, const double *xg, const double *mass,
-                                  int G, const double origin[3], const double axis[3], double radius, int nbins,
+cudaError_t launch_radial_profile(const double *u, int dim, const double *xg, const double *mass, int G,
+                                  const double origin[3], const double axis[3], double radius, int nbins,
                                   int blocks, double *partial, cudaStream_t s);
 
 template <typename Real>

@@ -813,19 +813,21 @@ __global__ void __launch_bounds__(256) curved_geo_kernel(const Real *drdx, int N
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-#define SLB_RAISE_SMEM(kernel, smem)                                                                           \
-  do {                                                                                                         \
-    static thread_local int attr_dev_ = -1;                                                                    \
-    static thread_local size_t attr_smem_ = 0;                                                                 \
-    int dev_ = 0;                                                                                              \
-    cudaGetDevice(&dev_);                                                                                      \
-    if (attr_dev_ != dev_ || attr_smem_ < (smem)) {                                                            \
-      cudaError_t err_ = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem)); \
-      if (err_ != cudaSuccess) return err_;                                                                    \
-      attr_dev_ = dev_;                                                                                        \
-      attr_smem_ = (smem);                                                                                     \
-    }                                                                                                          \
-  } while (0)
+// dynamic shared-memory limit of kernel K, raised once per device and thread (one set of statics
+// per kernel: kernels of one type are different template values)
+template <auto K>
+cudaError_t raise_smem(size_t smem) {
+  static thread_local int attr_dev = -1;
+  static thread_local size_t attr_smem = 0;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (attr_dev == dev && attr_smem >= smem) return cudaSuccess;
+  const cudaError_t err = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (err != cudaSuccess) return err;
+  attr_dev = dev;
+  attr_smem = smem;
+  return cudaSuccess;
+}
 
 // Q populations in ng groups of pb, as even as they come
 template <typename Real, int n>
@@ -840,13 +842,15 @@ cudaError_t launch_lines_stage_t(bool affine, const KParams<Real> &p, const Spli
   int pb, ng;
   line_groups<Real, n>(lt.Q, &pb, &ng);
   const StageMats<Real, n> m = make_stage_mats<Real, n>(h);
-  auto go = [&](auto k, size_t smem) -> cudaError_t {
-    SLB_RAISE_SMEM(k, smem);
-    k<<<p.E * ng, LineShape<Real, n>::T, smem, s>>>(p, m, lt, cg, pb, ng);
+  auto go = [&](auto ac) -> cudaError_t {
+    constexpr bool AFFINE = decltype(ac)::value;
+    const size_t smem = lines_stage_smem<Real, n, AFFINE>(pb, p.wall_max);
+    const cudaError_t err = raise_smem<lines_stage_kernel<Real, n, AFFINE>>(smem);
+    if (err != cudaSuccess) return err;
+    lines_stage_kernel<Real, n, AFFINE><<<p.E * ng, LineShape<Real, n>::T, smem, s>>>(p, m, lt, cg, pb, ng);
     return cudaGetLastError();
   };
-  return affine ? go(lines_stage_kernel<Real, n, true>, lines_stage_smem<Real, n, true>(pb, p.wall_max))
-                : go(lines_stage_kernel<Real, n, false>, lines_stage_smem<Real, n, false>(pb, p.wall_max));
+  return affine ? go(std::true_type{}) : go(std::false_type{});
 }
 
 template <typename Real, int n>
@@ -856,12 +860,14 @@ cudaError_t launch_lines_filter_t(const KParams<Real> &p, const SplitHost &h, in
   line_groups<Real, n>(Q, &pb, &ng);
   const FilterMats<Real, n> m = make_filter_mats<Real, n>(h);
   const size_t smem = lines_filter_smem<Real, n>(pb);
-  auto go = [&](auto k) -> cudaError_t {
-    SLB_RAISE_SMEM(k, smem);
-    k<<<p.E * ng, LineShape<Real, n>::T, smem, s>>>(p, m, sigma, out, Q, pb, ng);
+  auto go = [&](auto lc) -> cudaError_t {
+    constexpr bool LEARNED = decltype(lc)::value;
+    const cudaError_t err = raise_smem<lines_filter_kernel<Real, n, LEARNED>>(smem);
+    if (err != cudaSuccess) return err;
+    lines_filter_kernel<Real, n, LEARNED><<<p.E * ng, LineShape<Real, n>::T, smem, s>>>(p, m, sigma, out, Q, pb, ng);
     return cudaGetLastError();
   };
-  return sigma ? go(lines_filter_kernel<Real, n, true>) : go(lines_filter_kernel<Real, n, false>);
+  return sigma ? go(std::true_type{}) : go(std::false_type{});
 }
 
 // translation units by order: part 0 N <= 6, part 1 above

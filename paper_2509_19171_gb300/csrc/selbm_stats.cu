@@ -1,6 +1,6 @@
 // Turbulent pipe statistics (Sec. 4, pipe flow): wall shear stress from the wall-face
-// nodes and the radially binned mean axial velocity.  Both read the velocity at local
-// nodes (moments_kernel output, [E][Np][dim]) of the filtered state.
+// nodes and the radially binned mean axial velocity.  Both read the velocity of the
+// filtered state, at local nodes [E][Np][dim] and on unique nodes [dim][G].
 #include <cuda_runtime.h>
 
 #include "selbm_kernels.cuh"
@@ -55,7 +55,7 @@ __global__ void wall_stress_kernel(const double *u, int dim, int n, int Np, int 
 
 // per-block partial sums over unique nodes: bin b of node g = min(floor(r nbins / R),
 // nbins - 1) with r its distance from the axis line; sums of M_g (u.a) and M_g
-__global__ void radial_profile_kernel(const double *u, int dim, const int32_t *first, const double *xg,
+__global__ void radial_profile_kernel(const double *u, int dim, const double *xg,
                                       const double *mass, int G, double o0, double o1, double o2, double a0, double a1,
                                       double a2, double radius, int nbins, double *partial) {
   extern __shared__ double hist[];   // [nbins][2]
@@ -75,9 +75,8 @@ __global__ void radial_profile_kernel(const double *u, int dim, const int32_t *f
     }
     int b = (int)floor(sqrt(r2) * nbins / radius);
     b = b < 0 ? 0 : (b >= nbins ? nbins - 1 : b);
-    const double *ug = u + (size_t)first[g] * dim;
     double ua = 0;
-    for (int c = 0; c < dim; ++c) ua += ug[c] * a[c];
+    for (int c = 0; c < dim; ++c) ua += u[(size_t)c * G + g] * a[c];
     atomicAdd(&hist[2 * b], mass[g] * ua);
     atomicAdd(&hist[2 * b + 1], mass[g]);
   }
@@ -100,11 +99,11 @@ template cudaError_t launch_wall_stress<float>(const double *, int, int, int, in
                                                const float *, const void *, const int32_t *, const double *, double,
                                                double *, cudaStream_t);
 
-cudaError_t launch_radial_profile(const double *u, int dim, const int32_t *first, const double *xg, const double *mass,
-                                  int G, const double origin[3], const double axis[3], double radius, int nbins,
+cudaError_t launch_radial_profile(const double *u, int dim, const double *xg, const double *mass, int G,
+                                  const double origin[3], const double axis[3], double radius, int nbins,
                                   int blocks, double *partial, cudaStream_t s) {
   radial_profile_kernel<<<blocks, 256, 2 * nbins * sizeof(double), s>>>(
-      u, dim, first, xg, mass, G, origin[0], origin[1], origin[2], axis[0], axis[1], axis[2], radius, nbins, partial);
+      u, dim, xg, mass, G, origin[0], origin[1], origin[2], axis[0], axis[1], axis[2], radius, nbins, partial);
   return cudaGetLastError();
 }
 
