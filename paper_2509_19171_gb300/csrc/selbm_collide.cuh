@@ -34,24 +34,39 @@ __device__ __forceinline__ Real bgk_collide(Real (&g)[LT<LAT>::v.Q], Real rho0, 
     uu += u[k] * u[k];
     if (has_force) { F[k] = rho * gacc[k]; uF += u[k] * F[k]; }
   }
-  const Real base = Real(1.5) * uu;
-  static_for<0, Q>([&](auto ac) {
-    constexpr int a = decltype(ac)::value;
-    Real eu = 0, eF = 0;
+  // opposite velocities share the even part of f^eq (and F**); f + omega (f^eq - f) keeps an
+  // equilibrium exactly.  The rounded weights carry momentum 3 sum t e e = 1 + delta (delta the
+  // relative rounding of t, one value for all moving classes): 3 j is formed with 1 - delta, else
+  // the velocity would drift by omega delta every step (7e-9 in FP32; a folded constant 3 t: 3e-8).
+  constexpr double delta = (double)Real(V.t[1]) / V.t[1] - 1.0;
+  const Real r45 = Real(4.5) * rho, base = drho - Real(1.5) * rho * uu;
+  Real j3[3] = {0, 0, 0};
 #pragma unroll
-    for (int k = 0; k < DIM; ++k) {
-      if (V.e[a][k] > 0) { eu += u[k]; eF += F[k]; }
-      else if (V.e[a][k] < 0) { eu -= u[k]; eF -= F[k]; }
+  for (int k = 0; k < DIM; ++k) j3[k] = Real(3) * j[k] - Real(3.0 * delta) * j[k];
+  static_for<0, Q>([&](auto ac) {
+    constexpr int a = decltype(ac)::value, o = LT<LAT>::v.opp[a];
+    if constexpr (o >= a) {
+      Real eu = 0, ej = 0, eF = 0;
+#pragma unroll
+      for (int k = 0; k < DIM; ++k) {
+        if (V.e[a][k] > 0) { eu += u[k]; ej += j3[k]; eF += F[k]; }
+        else if (V.e[a][k] < 0) { eu -= u[k]; ej -= j3[k]; eF -= F[k]; }
+      }
+      const Real t = Real(V.t[a]);
+      Real even = o == a ? t * base : t * (base + (r45 * eu) * eu);
+      const Real odd = t * ej;
+      Real Fss = 0;
+      if (has_force) {
+        Fss = t * (Real(9) * eu * eF - Real(3) * uF);
+        even -= half_dt * Fss;
+      }
+      const Real fa = g[a];
+      g[a] = fa + omega * (even + odd - fa) + dt * Fss;
+      if constexpr (o != a) {
+        const Real fo = g[o];
+        g[o] = fo + omega * (even - odd - fo) + dt * Fss;
+      }
     }
-    const Real t = Real(V.t[a]);
-    Real feq = t * (drho + rho * (Real(3) * eu + Real(4.5) * eu * eu - base));
-    Real Fss = 0;
-    if (has_force) {
-      Fss = t * (Real(9) * eu * eF - Real(3) * uF);
-      feq -= half_dt * Fss;
-    }
-    const Real fa = g[a];
-    g[a] = fa - omega * (fa - feq) + dt * Fss;
   });
   return rho;
 }

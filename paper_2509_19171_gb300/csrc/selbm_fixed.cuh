@@ -70,6 +70,15 @@ __device__ __forceinline__ long long to_fixed(double v, int emax) {
   return (u ^ s) - s;
 }
 
+// the same rounded to nearest (ties away from zero)
+template <int SHIFT>
+__device__ __forceinline__ long long to_fixed_rn(double v, int emax) {
+  const long long q = to_fixed<SHIFT + 1>(v, emax), s = q >> 63;
+  return (q - s) >> 1;                                   // |q| odd: away from zero
+}
+
+// the same beyond the range of normal FP64 numbers (out of line: the code of the usual case counts)
+static __device__ __noinline__ double from_fixed_rare(long long r, int ex) { return scalbn((double)r, ex); }
 // r 2^ex as FP64, rounded to nearest
 __device__ __forceinline__ double from_fixed(long long r, int ex) {
   const long long s = r >> 63;
@@ -78,7 +87,7 @@ __device__ __forceinline__ double from_fixed(long long r, int ex) {
   a <<= (lz & 63);
   const unsigned long long mant = (a >> 11) + ((a >> 10) & 1ull);   // 2^52 .. 2^53
   const int E = 1086 - lz + ex;                          // biased exponent of the result
-  if ((unsigned)(E - 1) >= 2045u) return r == 0 ? 0.0 : scalbn((double)r, ex);
+  if ((unsigned)(E - 1) >= 2045u) return r == 0 ? 0.0 : from_fixed_rare(r, ex);
   unsigned long long bits = ((unsigned long long)(unsigned)(E - 1) << 52) + mant;
   bits = r == 0 ? 0ull : bits;
   return __longlong_as_double((long long)(bits | ((unsigned long long)s & 0x8000000000000000ull)));

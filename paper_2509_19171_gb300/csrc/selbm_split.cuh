@@ -27,6 +27,7 @@
 
 #include "selbm_collide.cuh"
 #include "selbm_fast.cuh"
+#include "selbm_moments.cuh"
 #include "selbm_split_stage.cuh"
 
 namespace slb {
@@ -651,17 +652,25 @@ __global__ void __launch_bounds__(256) dss_collide_kernel(const KParams<Real> p)
 }
 
 // collision on unique nodes (no pending filter)
+constexpr int kCollideThreads = 128;
 template <typename Real, int LAT>
-__global__ void __launch_bounds__(256) collide_nodes_kernel(const KParams<Real> p) {
+__global__ void __launch_bounds__(kCollideThreads, sizeof(Real) == 8 ? 4 : 8) collide_nodes_kernel(const KParams<Real> p, const CollideFix cf) {
   constexpr int Q = LT<LAT>::v.Q;
   for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < (size_t)p.G; g += (size_t)gridDim.x * blockDim.x) {
-    Real s[Q], gacc[3];
-#pragma unroll
-    for (int a = 0; a < Q; ++a) s[a] = p.fin[(size_t)a * p.Gs + g];
+    Real gacc[3], rho;
     node_accel(p, g, gacc);
-    const Real rho = bgk_collide<Real, LAT>(s, p.rho0, p.omega, p.dt, p.half_dt, gacc, p.has_force != 0);
+    if constexpr (sizeof(Real) == 8) {
+      rho = collide_fixed<LAT>(cf, p.rho0, p.omega, p.dt, p.half_dt, gacc, p.has_force != 0,
+                               [&](int a) { return p.fin[(size_t)a * p.Gs + g]; },
+                               [&](int a, double v) { p.f0out[(size_t)a * p.Gs + g] = v; });
+    } else {
+      Real s[Q];
 #pragma unroll
-    for (int a = 0; a < Q; ++a) p.f0out[(size_t)a * p.Gs + g] = s[a];
+      for (int a = 0; a < Q; ++a) s[a] = p.fin[(size_t)a * p.Gs + g];
+      rho = bgk_collide<Real, LAT>(s, p.rho0, p.omega, p.dt, p.half_dt, gacc, p.has_force != 0);
+#pragma unroll
+      for (int a = 0; a < Q; ++a) p.f0out[(size_t)a * p.Gs + g] = s[a];
+    }
     if (p.has_force) p.rho[g] = rho;
   }
 }
@@ -752,9 +761,9 @@ cudaError_t launch_dss_collide_t(const KParams<Real> &p, cudaStream_t s) {
 
 template <typename Real, int LAT>
 cudaError_t launch_collide_nodes_t(const KParams<Real> &p, cudaStream_t s) {
-  const int threads = 256;
-  const int blocks = (int)std::min<size_t>(((size_t)p.G + threads - 1) / threads, 152 * 32);
-  collide_nodes_kernel<Real, LAT><<<blocks, threads, 0, s>>>(p);
+  const int threads = kCollideThreads;
+  const int blocks = (int)std::min<size_t>(((size_t)p.G + threads - 1) / threads, 152 * 64);
+  collide_nodes_kernel<Real, LAT><<<blocks, threads, 0, s>>>(p, make_collide_fix<LAT>((double)p.omega, (double)p.dt));
   return cudaGetLastError();
 }
 
