@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "../../include/selbm.h"
+#include "selbm_flow2d.h"
 #include "selbm_kernels.cuh"
 #include "selbm_learn.cuh"
 #include "selbm_lines.h"
@@ -67,6 +68,14 @@ struct selbm {
   void *d_nq = nullptr;          // [2][Gs] rho - rho0 and |u| on unique nodes (learned control, split form)
   void *d_X = nullptr;           // [E][2n] element features (learned control, split form)
   int *d_flag = nullptr, *d_nfb = nullptr;
+  // resident step of 2D meshes that fit the SMs' shared memory (flow_epc elements per CTA, else 0)
+  int flow_epc = 0;
+  unsigned flow_epoch = 0;
+  int32_t *d_loc_u = nullptr, *d_loc_off = nullptr, *d_loc_slot = nullptr, *d_loc_base = nullptr, *d_rem_off = nullptr,
+          *d_rem = nullptr, *d_bas_off = nullptr, *d_bas = nullptr;
+  int flow_rmax = 0, flow_bmax = 0;
+  void *d_flow_T = nullptr, *d_flow_base = nullptr;
+  int *abort_host = nullptr;     // mapped host memory: a bounded wait of the resident step gave up
   int wall_max = 0;
   int n_wallpts = 0;             // wall points (element, node) over all elements
   double *d_xg = nullptr;        // [G][dim] coordinates of unique nodes (uploaded on first use)
@@ -141,6 +150,100 @@ struct selbm {
 };
 
 namespace {
+
+SplitHost split_host(selbm *h) {
+  return SplitHost{h->S.gll.D.data(), h->FU.data(), h->FW.data(), h->S.gll.w.data(), h->Fr,
+                   h->Vm_h.data(), h->Vinv_h.data(), h->sigma.data()};
+}
+
+// tables of the resident 2D step: where a CTA finds the copies and the owner of every boundary
+// node of its elements, and what it fetches from other CTAs
+template <typename Real>
+cudaError_t setup_flow2d(selbm *h) {
+  const Setup &S = h->S;
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
+  const int epc = (S.E + sms - 1) / sms, grid = (S.E + epc - 1) / epc, Nb = S.Nb;
+  std::vector<int32_t> u((size_t)S.E * Nb), off((size_t)S.E * Nb + 1, 0), slot, base((size_t)S.E * Nb), rem, rem_off(1, 0), bas,
+      bas_off(1, 0), at((size_t)S.E * Nb, -1), at_u(S.Gb, -1);
+  for (int k = 0; k < S.Gb; ++k)
+    for (int c = S.bnode_off[k]; c < S.bnode_off[k + 1]; ++c) u[S.bnode_slot[c]] = k;
+  int rmax = 0, bmax = 0;
+  for (int cta = 0; cta < grid; ++cta) {
+    const int e0 = cta * epc, e1 = std::min(S.E, e0 + epc);
+    const size_t rem0 = rem.size(), bas0 = bas.size();
+    for (size_t lb = (size_t)e0 * Nb; lb < (size_t)e1 * Nb; ++lb) {
+      off[lb] = (int32_t)slot.size();
+      const int k = u[lb];
+      for (int c = S.bnode_off[k]; c < S.bnode_off[k + 1]; ++c) {
+        const int s = S.bnode_slot[c], e2 = s / Nb;
+        if (e2 >= e0 && e2 < e1) {
+          slot.push_back(-3 - (s - e0 * Nb));
+          continue;
+        }
+        if (at[s] < 0) { at[s] = (int32_t)(rem.size() - rem0); rem.push_back(e2 * 9 * Nb + s % Nb); }
+        slot.push_back(at[s]);
+      }
+      // the first copy owns the node
+      const int s = S.bnode_slot[S.bnode_off[k]];
+      if ((size_t)s == lb) base[lb] = -1;
+      else if (s / Nb >= e0 && s / Nb < e1) base[lb] = -3 - (s - e0 * Nb);
+      else {
+        if (at_u[k] < 0) { at_u[k] = (int32_t)(bas.size() - bas0); bas.push_back(k); }
+        base[lb] = at_u[k];
+      }
+    }
+    for (size_t r = rem0; r < rem.size(); ++r) at[(size_t)rem[r] / (9 * Nb) * Nb + rem[r] % (9 * Nb)] = -1;
+    for (size_t r = bas0; r < bas.size(); ++r) at_u[bas[r]] = -1;
+    rem_off.push_back((int32_t)rem.size());
+    bas_off.push_back((int32_t)bas.size());
+    rmax = std::max(rmax, (int)(rem.size() - rem0));
+    bmax = std::max(bmax, (int)(bas.size() - bas0));
+  }
+  off[(size_t)S.E * Nb] = (int32_t)slot.size();
+  if (rem.empty()) rem.push_back(0);
+  if (bas.empty()) bas.push_back(0);
+  Flow2DArgs<Real> a{};
+  a.E = S.E; a.epc = epc; a.rmax = rmax; a.bmax = bmax;
+  bool fits = false;
+  e = launch_flow2d<Real>(S.N, S.affine, true, a, split_host(h), &fits, h->stream);
+  if (e != cudaSuccess || !fits) return e;
+  auto keep = [&](int32_t **d, const std::vector<int32_t> &v) -> cudaError_t {
+    const cudaError_t r = upload(d, v);
+    if (r == cudaSuccess) h->allocs.push_back(*d);
+    return r;
+  };
+  if ((e = keep(&h->d_loc_u, u)) || (e = keep(&h->d_loc_off, off)) || (e = keep(&h->d_loc_slot, slot)) ||
+      (e = keep(&h->d_loc_base, base)) || (e = keep(&h->d_rem_off, rem_off)) || (e = keep(&h->d_rem, rem)) ||
+      (e = keep(&h->d_bas_off, bas_off)) || (e = keep(&h->d_bas, bas)))
+    return e;
+  h->flow_rmax = rmax;
+  h->flow_bmax = bmax;
+  auto alloc = [&](void **p, size_t bytes) -> cudaError_t {
+    cudaError_t r = cudaMalloc(p, bytes);
+    if (r == cudaSuccess) { h->allocs.push_back(*p); r = cudaMemsetAsync(*p, 0, bytes, h->stream); }
+    return r;
+  };
+  if ((e = alloc(&h->d_flow_T, (size_t)4 * S.E * 9 * Nb * sizeof(Real)))) return e;
+  if ((e = alloc(&h->d_flow_base, (size_t)S.Gb * 20 * sizeof(Real)))) return e;
+  if (!S.affine && sizeof(Real) == 8) {
+    std::vector<int> ex(S.E);
+    for (int el = 0; el < S.E; ++el) {
+      double mx = 0;
+      for (size_t k = (size_t)el * S.Np * 4; k < (size_t)(el + 1) * S.Np * 4; ++k) mx = std::max(mx, std::fabs(S.drdx[k]));
+      ex[el] = mx > 0 ? 57 - std::ilogb(mx) : 0;
+    }
+    int *d = nullptr;
+    if ((e = upload(&d, ex))) return e;
+    h->allocs.push_back(d);
+    h->d_gexp = d;
+  }
+  if ((e = cudaHostAlloc((void **)&h->abort_host, sizeof(int), cudaHostAllocMapped))) return e;
+  *h->abort_host = 0;
+  h->flow_epc = epc;
+  return cudaSuccess;
+}
 
 template <typename Real>
 cudaError_t upload_real(selbm *h) {
@@ -238,7 +341,7 @@ cudaError_t upload_real(selbm *h) {
   if ((e = upload(&dw, wp))) return e; h->d_walls = dw; if (dw) h->allocs.push_back(dw);
   int32_t *q;
   if ((e = upload(&q, woff))) return e; h->d_wall_off = q; h->allocs.push_back(q);
-  return cudaSuccess;
+  return S.dim == 2 && h->use_fast ? setup_flow2d<Real>(h) : cudaSuccess;
 }
 
 template <typename Real>
@@ -304,11 +407,6 @@ cudaError_t launch_stage_any(selbm *h, const KParams<Real> &p) {
     if (done) return err;
   }
   return launch_stage<Real>(h->lat, h->S.affine, p, h->stream);
-}
-
-SplitHost split_host(selbm *h) {
-  return SplitHost{h->S.gll.D.data(), h->FU.data(), h->FW.data(), h->S.gll.w.data(), h->Fr,
-                   h->Vm_h.data(), h->Vinv_h.data(), h->sigma.data()};
 }
 
 template <typename Real>
@@ -651,6 +749,44 @@ int node_fields(selbm *h, const void *f, bool diag) {
   return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "moments");
 }
 
+// SELBM_ERR_TIMEOUT when a bounded wait has given up (the caller has synchronised the stream)
+int wait_status(selbm *h) {
+  return h->abort_host && *(volatile int *)h->abort_host ? h->fail(SELBM_ERR_TIMEOUT, "a wait of the resident 2D step gave up") : SELBM_OK;
+}
+
+// nsteps steps of the resident 2D step, in launches of a bounded length
+template <typename Real>
+cudaError_t run_flow2d(selbm *h, int64_t nsteps) {
+  const KParams<Real> k = base_params<Real>(h);
+  Flow2DArgs<Real> a{};
+  a.E = k.E; a.Gs = k.Gs; a.epc = h->flow_epc;
+  a.filter = h->filter_on; a.has_force = k.has_force;
+  a.dt = k.dt; a.half_dt = k.half_dt; a.omega = k.omega; a.rho0 = k.rho0;
+  for (int c = 0; c < 3; ++c) a.g[c] = k.g[c];
+  a.l2g = k.l2g; a.bslot = k.bslot; a.owner = k.owner;
+  a.el_drdx = k.el_drdx; a.el_J = k.el_J; a.drdx = k.drdx; a.wJ = k.wJ; a.minv = k.bnode_minv; a.gexp = h->d_gexp;
+  a.walls = k.walls; a.wall_off = k.wall_off; a.wall_u = k.wall_u;
+  a.loc_u = h->d_loc_u; a.loc_off = h->d_loc_off; a.loc_slot = h->d_loc_slot; a.loc_base = h->d_loc_base;
+  a.rem_off = h->d_rem_off; a.rem = h->d_rem; a.bas_off = h->d_bas_off; a.bas = h->d_bas;
+  a.rmax = h->flow_rmax; a.bmax = h->flow_bmax;
+  a.abort = h->abort_host;
+  a.T = h->d_flow_T; a.base = h->d_flow_base; a.f = (Real *)h->FA;
+  const SplitHost sh = split_host(h);
+  while (nsteps > 0) {
+    a.nsteps = (int)std::min<int64_t>(nsteps, 20000);
+    a.pending = h->filter_pending;
+    a.epoch = h->flow_epoch;
+    const cudaError_t e = launch_flow2d<Real>(h->S.N, h->S.affine, false, a, sh, nullptr, h->stream);
+    if (e != cudaSuccess) return e;
+    h->flow_epoch += 3u * (unsigned)a.nsteps;
+    h->filter_pending = true;
+    for (int s = 0; s < a.nsteps; ++s) h->time += h->dt;
+    h->steps += a.nsteps;
+    nsteps -= a.nsteps;
+  }
+  return cudaSuccess;
+}
+
 int ensure_io(selbm *h, size_t bytes) {
   if (h->io_bytes >= bytes) return SELBM_OK;
   if (h->d_io) cudaFree(h->d_io);
@@ -762,6 +898,7 @@ void selbm_destroy(selbm_t *h) {
   for (auto &u : h->ev_used) { cudaEventDestroy(u.second.first); cudaEventDestroy(u.second.second); }
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
   for (void *p : h->allocs) cudaFree(p);
+  if (h->abort_host) cudaFreeHost(h->abort_host);
   void *own[] = {h->d_l2g, h->d_owner, h->d_bslot, h->d_bnode_g, h->d_bnode_off, h->d_bnode_slot, h->d_first,
                  h->d_mass, h->d_partial, h->d_diag, h->d_io, h->d_xg};
   for (void *p : own)
@@ -866,7 +1003,7 @@ int selbm_get_state(selbm_t *h, double *f, int on_device) {
   if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(f, df, bytes, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "get_state");
-  return SELBM_OK;
+  return wait_status(h);
 }
 
 // capture one step of the given variant into a graph (after one eager step of that
@@ -900,6 +1037,10 @@ int selbm_step(selbm_t *h, int64_t nsteps) {
   if (!h) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
   if (nsteps < 0) return h->fail(SELBM_ERR_ARG, "nsteps < 0");
+  if (h->flow_epc > 0 && !h->timing && !h->learned && !h->field_on && h->scheme == 0) {
+    const cudaError_t e = h->prec == SELBM_FP64 ? run_flow2d<double>(h, nsteps) : run_flow2d<float>(h, nsteps);
+    return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "step");
+  }
   for (int64_t k = 0; k < nsteps; ++k) {
     const bool filt = filter_waits(h);
     const int slot = filt ? 1 : 0;
@@ -939,7 +1080,7 @@ int selbm_moments(selbm_t *h, double *rho, double *u, int on_device) {
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "moments");
-  return SELBM_OK;
+  return wait_status(h);
 }
 
 int selbm_stress(selbm_t *h, double *pi, int on_device) {
@@ -971,7 +1112,7 @@ int selbm_stress(selbm_t *h, double *pi, int on_device) {
   if (e == cudaSuccess && !on_device) e = cudaMemcpyAsync(pi, dp, n * 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "stress");
-  return SELBM_OK;
+  return wait_status(h);
 }
 
 int selbm_set_filter(selbm_t *h, const selbm_filter *f) {
@@ -1085,6 +1226,7 @@ int selbm_diagnostics(selbm_t *h, double out[8]) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(tmp, h->d_diag, 7 * sizeof(double), cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "diagnostics");
+  if ((rc = wait_status(h))) return rc;
   out[0] = tmp[0];
   for (int k = 0; k < 3; ++k) out[1 + k] = tmp[1 + k];
   out[4] = tmp[4]; out[5] = tmp[6]; out[6] = h->dt; out[7] = h->time;
@@ -1122,6 +1264,7 @@ int selbm_wall_stress(selbm_t *h, const double dir[3], double *tau) {
   if (e == cudaSuccess) e = cudaMemcpyAsync(hp.data(), part, hp.size() * 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "wall_stress");
+  if ((rc = wait_status(h))) return rc;
   double num = 0, den = 0;
   for (int k = 0; k < h->n_wallpts; ++k) { num += hp[2 * k]; den += hp[2 * k + 1]; }
   *tau = den > 0 ? num / den : 0.0;
@@ -1391,6 +1534,7 @@ int selbm_sync(selbm_t *h) {
   if (!h) return SELBM_ERR_ARG;
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "sync");
+  if (const int rc = wait_status(h)) return rc;
   return fallback_status(h);
 }
 
