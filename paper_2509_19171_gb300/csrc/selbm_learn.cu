@@ -19,7 +19,6 @@
 namespace slb {
 
 constexpr int kH = 64;
-constexpr int kTile = 64;     // samples per training tile
 
 int mlp_nparams(int nin) { return kH * nin + kH + kH * kH + kH + 2 * kH + 2; }
 
@@ -327,7 +326,7 @@ cudaError_t launch_element_errors(int E, int dim, int n, int nR, const double *r
 }
 
 // ---------------------------------------------------------------------------
-// MLP training: one CTA per 64-sample tile computes the tile's loss and gradient sums
+// MLP training: one CTA per tile of samples computes the tile's loss and gradient sums
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t mix32(uint32_t x, uint64_t key, uint32_t r) {
   uint64_t z = (uint64_t)x ^ (key + 0x9E3779B97F4A7C15ull * (r + 1));
@@ -367,143 +366,241 @@ struct TileArgs {
 
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
 
-__global__ void __launch_bounds__(256) mlp_tile_kernel(const TileArgs a, int forward_only) {
+// One CTA per TS samples: forward pass, loss and the tile's gradient sums.  A minibatch of the
+// training (1024 samples, 33 MFLOP) is latency, not work: tiles of 8 samples spread it over the SMs
+// (64-sample tiles left 136 of 152 idle), and the weights are kept transposed where lanes run over a
+// layer's outputs, so that no shared-memory access has bank conflicts (W2 read by rows had 32-way
+// ones).  Thread (j, group): output j of samples group, group + 4, ...
+constexpr int kMlpT = 256;
+constexpr int kGrp = kMlpT / kH;
+template <int TS>
+__global__ void __launch_bounds__(kMlpT) mlp_tile_kernel(const TileArgs a, int forward_only) {
+  constexpr int SP = TS / kGrp;                        // samples per thread
   extern __shared__ __align__(16) float sm[];
   const int nin = a.nin, P = kH * nin + kH + kH * kH + kH + 2 * kH + 2;
-  float *W = sm;                       // [P]
-  float *S = W + P;                    // [64][nin]
-  float *H1 = S + kTile * nin;         // [64][64]
-  float *H2 = H1 + kTile * kH;         // [64][64]
-  float *D2 = H2 + kTile * kH;         // [64][64]  dZ2
-  float *D1 = D2 + kTile * kH;         // [64][64]  dZ1
-  float *O = D1 + kTile * kH;          // [64][2]
-  float *dO = O + kTile * 2;           // [64][2]
-  float *Yt = dO + kTile * 2;          // [64][2]
-  int *idx = reinterpret_cast<int *>(Yt + kTile * 2);   // [64] sample index or -1
-  const int tid = threadIdx.x, T = blockDim.x;
-  const float *W1 = W, *b1 = W1 + kH * nin, *W2 = b1 + kH, *b2 = W2 + kH * kH, *W3 = b2 + kH, *b3 = W3 + 2 * kH;
-  for (int k = tid; k < P; k += T) W[k] = a.bf16 ? bf16r(a.params[k]) : a.params[k];
-  for (int s = tid; s < kTile; s += T) {
-    const int64_t pos = (int64_t)blockIdx.x * kTile + s;
+  float *W2 = sm;                      // [64][64]
+  float *W2T = W2 + kH * kH;           // [64][65]  W2T[m][j]
+  float *H1 = W2T + kH * (kH + 1);     // [TS][64]
+  float *H2 = H1 + TS * kH;            // [TS][64]
+  float *D2 = H2 + TS * kH;            // [TS][64]  dZ2
+  float *D1 = D2 + TS * kH;            // [TS][64]  dZ1
+  float *W1T = D1 + TS * kH;           // [nin][64] W1T[i][j]
+  float *S = W1T + nin * kH;           // [TS][nin]
+  float *b1 = S + TS * nin, *b2 = b1 + kH, *W3 = b2 + kH, *b3 = W3 + 2 * kH;
+  float *O = b3 + 2;                   // [TS][2]
+  float *dO = O + 2 * TS;              // [TS][2]
+  float *Yt = dO + 2 * TS;             // [TS][2]
+  int *idx = reinterpret_cast<int *>(Yt + 2 * TS);   // [TS] sample index or -1
+  const int tid = threadIdx.x, j = tid & (kH - 1), grp = tid / kH;
+  const float *p1 = a.params, *q1 = p1 + kH * nin, *p2 = q1 + kH, *q2 = p2 + kH * kH, *p3 = q2 + kH, *q3 = p3 + 2 * kH;
+  auto rd = [&](const float *p) { return a.bf16 ? bf16r(*p) : *p; };
+  if (tid < TS) {
+    const int64_t pos = (int64_t)blockIdx.x * TS + tid;
     int64_t sidx = -1;
     if (pos < a.count) {
       const int64_t g = a.start + pos;
       sidx = a.h > 0 ? shuffle_index(g, a.M, a.h, a.key) : g;
     }
-    idx[s] = (int)sidx;
+    idx[tid] = (int)sidx;
   }
+  for (int k = tid; k < kH * kH; k += kMlpT) {
+    const float w = rd(p2 + k);
+    W2[k] = w;
+    W2T[(k & (kH - 1)) * (kH + 1) + k / kH] = w;
+  }
+  for (int k = tid; k < kH * nin; k += kMlpT) W1T[(k % nin) * kH + k / nin] = rd(p1 + k);
+  if (tid < kH) { b1[tid] = rd(q1 + tid); b2[tid] = rd(q2 + tid); }
+  if (tid < 2 * kH) W3[tid] = rd(p3 + tid);
+  if (tid < 2) b3[tid] = rd(q3 + tid);
   __syncthreads();
-  for (int k = tid; k < kTile * nin; k += T) {
-    const int s = k / nin, i = k - s * nin;
-    S[k] = idx[s] >= 0 ? a.X[(size_t)idx[s] * nin + i] : 0.f;
+  for (int k = tid; k < TS * nin; k += kMlpT) {
+    const int s = k / nin;
+    S[k] = idx[s] >= 0 ? a.X[(size_t)idx[s] * nin + k - s * nin] : 0.f;
   }
-  for (int k = tid; k < kTile * 2; k += T) {
+  for (int k = tid; k < TS * 2; k += kMlpT) {
     const int s = k / 2;
     Yt[k] = (idx[s] >= 0 && !forward_only) ? a.Y[(size_t)idx[s] * 2 + (k & 1)] : 0.f;
   }
   __syncthreads();
-  for (int k = tid; k < kTile * kH; k += T) {
-    const int s = k / kH, j = k - s * kH;
-    float z = b1[j];
-    for (int i = 0; i < nin; ++i) z += W1[j * nin + i] * S[s * nin + i];
-    H1[k] = tanhf(z);
+  {
+    float z[SP];
+#pragma unroll
+    for (int s = 0; s < SP; ++s) z[s] = b1[j];
+    for (int i = 0; i < nin; ++i) {
+      const float w = W1T[i * kH + j];
+#pragma unroll
+      for (int s = 0; s < SP; ++s) z[s] += w * S[(grp + kGrp * s) * nin + i];
+    }
+#pragma unroll
+    for (int s = 0; s < SP; ++s) H1[(grp + kGrp * s) * kH + j] = tanhf(z[s]);
   }
   __syncthreads();
-  for (int k = tid; k < kTile * kH; k += T) {
-    const int s = k / kH, j = k - s * kH;
-    float z = b2[j];
-    for (int m = 0; m < kH; ++m) z += W2[j * kH + m] * H1[s * kH + m];
-    H2[k] = tanhf(z);
+  {
+    float z[SP];
+#pragma unroll
+    for (int s = 0; s < SP; ++s) z[s] = b2[j];
+#pragma unroll 4
+    for (int m = 0; m < kH; m += 4) {
+      const float w0 = W2T[m * (kH + 1) + j], w1 = W2T[(m + 1) * (kH + 1) + j], w2 = W2T[(m + 2) * (kH + 1) + j],
+                  w3 = W2T[(m + 3) * (kH + 1) + j];
+#pragma unroll
+      for (int s = 0; s < SP; ++s) {
+        const float *h = H1 + (grp + kGrp * s) * kH + m;
+        z[s] += w0 * h[0];
+        z[s] += w1 * h[1];
+        z[s] += w2 * h[2];
+        z[s] += w3 * h[3];
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < SP; ++s) H2[(grp + kGrp * s) * kH + j] = tanhf(z[s]);
   }
   __syncthreads();
+  // outputs: one warp per (sample, output), the products summed by a fixed tree
   const float Nm3 = (float)(a.N - 3);
-  for (int k = tid; k < kTile * 2; k += T) {
-    const int s = k / 2, c = k & 1;
-    float z = b3[c];
-    for (int m = 0; m < kH; ++m) z += W3[c * kH + m] * H2[s * kH + m];
+  for (int k = tid >> 5; k < TS * 2; k += kMlpT / 32) {
+    const int s = k / 2, c = k & 1, lane = tid & 31;
+    float z = W3[c * kH + lane] * H2[s * kH + lane] + W3[c * kH + 32 + lane] * H2[s * kH + 32 + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+    z += b3[c];
     const float sg = 1.f / (1.f + expf(-z));
     const float val = c == 0 ? 0.5f * sg : 2.f + Nm3 * sg;
-    O[k] = val;
-    if (forward_only) {
-      if (idx[s] >= 0) a.out[(size_t)idx[s] * 2 + c] = val;
-    } else {
-      const float scale = c == 0 ? 0.5f : Nm3;
-      const float r = idx[s] >= 0 ? (val - Yt[k]) / scale : 0.f;
-      dO[k] = 2.f * r / scale * (c == 0 ? 0.5f : Nm3) * sg * (1.f - sg);   // dL/dz (unscaled by batch)
-      O[k] = r * r;
+    if (lane == 0) {
+      if (forward_only) {
+        if (idx[s] >= 0) a.out[(size_t)idx[s] * 2 + c] = val;
+      } else {
+        const float scale = c == 0 ? 0.5f : Nm3;
+        const float r = idx[s] >= 0 ? (val - Yt[k]) / scale : 0.f;
+        dO[k] = 2.f * r / scale * (c == 0 ? 0.5f : Nm3) * sg * (1.f - sg);   // dL/dz (unscaled by batch)
+        O[k] = r * r;
+      }
     }
   }
   if (forward_only) return;
   __syncthreads();
   float *g = a.gpart + (size_t)blockIdx.x * P;
   float *gW1 = g, *gb1 = gW1 + kH * nin, *gW2 = gb1 + kH, *gb2 = gW2 + kH * kH, *gW3 = gb2 + kH, *gb3 = gW3 + 2 * kH;
-  if (tid == 0) {
+  if (tid < 32) {
     float l = 0.f;
-    for (int k = 0; k < kTile * 2; ++k) l += O[k];
-    a.lpart[blockIdx.x] = l;
+    for (int k = tid; k < TS * 2; k += 32) l += O[k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (tid == 0) a.lpart[blockIdx.x] = l;
   }
-  // output layer
-  for (int k = tid; k < 2 * kH; k += T) {
-    const int c = k / kH, m = k - c * kH;
+  // output layer; dZ2
+  if (tid < 2 * kH) {
+    const int c = tid / kH, m = tid - c * kH;
     float s = 0.f;
-    for (int t = 0; t < kTile; ++t) s += dO[t * 2 + c] * H2[t * kH + m];
-    gW3[k] = s;
+#pragma unroll
+    for (int t = 0; t < TS; ++t) s += dO[t * 2 + c] * H2[t * kH + m];
+    gW3[tid] = s;
   }
   if (tid < 2) {
     float s = 0.f;
-    for (int t = 0; t < kTile; ++t) s += dO[t * 2 + tid];
+    for (int t = 0; t < TS; ++t) s += dO[t * 2 + tid];
     gb3[tid] = s;
   }
-  for (int k = tid; k < kTile * kH; k += T) {
-    const int s = k / kH, m = k - s * kH;
-    const float dh = dO[s * 2] * W3[m] + dO[s * 2 + 1] * W3[kH + m];
-    D2[k] = dh * (1.f - H2[k] * H2[k]);
+#pragma unroll
+  for (int s = 0; s < SP; ++s) {
+    const int k = (grp + kGrp * s) * kH + j, t = grp + kGrp * s;
+    D2[k] = (dO[t * 2] * W3[j] + dO[t * 2 + 1] * W3[kH + j]) * (1.f - H2[k] * H2[k]);
   }
   __syncthreads();
-  for (int k = tid; k < kH * kH; k += T) {
-    const int j = k / kH, m = k - j * kH;
-    float s = 0.f;
-    for (int t = 0; t < kTile; ++t) s += D2[t * kH + j] * H1[t * kH + m];
-    gW2[k] = s;
+  // gW2[jj][m] = sum_t D2[t][jj] H1[t][m]: thread (m = j, 16 rows of its group)
+  {
+    constexpr int RW = kH / kGrp;
+    float s[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) s[r] = 0.f;
+#pragma unroll 4
+    for (int t = 0; t < TS; ++t) {
+      const float h = H1[t * kH + j];
+      const float4 *d = reinterpret_cast<const float4 *>(D2 + t * kH + grp * RW);
+#pragma unroll
+      for (int r = 0; r < RW / 4; ++r) {
+        const float4 v = d[r];
+        s[4 * r] += v.x * h;
+        s[4 * r + 1] += v.y * h;
+        s[4 * r + 2] += v.z * h;
+        s[4 * r + 3] += v.w * h;
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < RW; ++r) gW2[(grp * RW + r) * kH + j] = s[r];
   }
-  for (int j = tid; j < kH; j += T) {
+  {
     float s = 0.f;
-    for (int t = 0; t < kTile; ++t) s += D2[t * kH + j];
-    gb2[j] = s;
+    if (tid < kH) {
+#pragma unroll
+      for (int t = 0; t < TS; ++t) s += D2[t * kH + tid];
+      gb2[tid] = s;
+    }
   }
-  for (int k = tid; k < kTile * kH; k += T) {
-    const int s = k / kH, m = k - s * kH;
-    float dh = 0.f;
-    for (int j = 0; j < kH; ++j) dh += D2[s * kH + j] * W2[j * kH + m];
-    D1[k] = dh * (1.f - H1[k] * H1[k]);
+  // dZ1
+  {
+    float d[SP];
+#pragma unroll
+    for (int s = 0; s < SP; ++s) d[s] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < kH; k += 4) {
+      const float w0 = W2[k * kH + j], w1 = W2[(k + 1) * kH + j], w2 = W2[(k + 2) * kH + j], w3 = W2[(k + 3) * kH + j];
+#pragma unroll
+      for (int s = 0; s < SP; ++s) {
+        const float4 v = *reinterpret_cast<const float4 *>(D2 + (grp + kGrp * s) * kH + k);
+        d[s] += v.x * w0;
+        d[s] += v.y * w1;
+        d[s] += v.z * w2;
+        d[s] += v.w * w3;
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < SP; ++s) {
+      const int k = (grp + kGrp * s) * kH + j;
+      D1[k] = d[s] * (1.f - H1[k] * H1[k]);
+    }
   }
   __syncthreads();
-  for (int k = tid; k < kH * nin; k += T) {
-    const int j = k / nin, i = k - j * nin;
+  for (int k = tid; k < kH * nin; k += kMlpT) {
+    const int jj = k / nin, i = k - jj * nin;
     float s = 0.f;
-    for (int t = 0; t < kTile; ++t) s += D1[t * kH + j] * S[t * nin + i];
+#pragma unroll 4
+    for (int t = 0; t < TS; ++t) s += D1[t * kH + jj] * S[t * nin + i];
     gW1[k] = s;
   }
-  for (int j = tid; j < kH; j += T) {
+  if (tid < kH) {
     float s = 0.f;
-    for (int t = 0; t < kTile; ++t) s += D1[t * kH + j];
-    gb1[j] = s;
+#pragma unroll
+    for (int t = 0; t < TS; ++t) s += D1[t * kH + tid];
+    gb1[tid] = s;
   }
 }
 
-// sum tile partials in tile order (deterministic), scale, then optionally Adam
-__global__ void mlp_reduce_kernel(const float *gpart, const float *lpart, int tiles, int P, float scale, float *grad,
-                                  float *loss, float *params, float *m, float *v, float lr, float b1c, float b2c,
-                                  int adam) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p == 0 && loss) {
-    float l = 0.f;
-    for (int t = 0; t < tiles; ++t) l += lpart[t];
-    *loss = l * scale;
-  }
-  if (p >= P) return;
+// sum tile partials in a fixed order (kRedSlices interleaved sums per parameter, then their sum),
+// scale, then optionally Adam.  32 parameters per CTA, so that the partials are read by all SMs.
+constexpr int kRedP = 32, kRedSlices = 16;
+__global__ void __launch_bounds__(kRedP * kRedSlices)
+mlp_reduce_kernel(const float *gpart, const float *lpart, int tiles, int P, float scale, float *grad, float *loss,
+                  float *params, float *m, float *v, float lr, float b1c, float b2c, int adam) {
+  __shared__ float part[kRedSlices][kRedP];
+  const int lane = threadIdx.x % kRedP, slice = threadIdx.x / kRedP, p = blockIdx.x * kRedP + lane;
   float gs = 0.f;
-  for (int t = 0; t < tiles; ++t) gs += gpart[(size_t)t * P + p];
+  if (p < P)
+#pragma unroll 8
+    for (int t = slice; t < tiles; t += kRedSlices) gs += gpart[(size_t)t * P + p];
+  part[slice][lane] = gs;
+  if (blockIdx.x == 0 && slice == 1 && loss) {
+    float l = 0.f;
+    for (int t = lane; t < tiles; t += 32) l += lpart[t];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+    if (lane == 0) *loss = l * scale;
+  }
+  __syncthreads();
+  if (slice != 0 || p >= P) return;
+  gs = 0.f;
+#pragma unroll
+  for (int k = 0; k < kRedSlices; ++k) gs += part[k][lane];
   gs *= scale;
   if (grad) grad[p] = gs;
   if (adam) {
@@ -515,29 +612,52 @@ __global__ void mlp_reduce_kernel(const float *gpart, const float *lpart, int ti
   }
 }
 
-static size_t tile_smem(int nin) {
-  const int P = mlp_nparams(nin);
-  return (size_t)(P + kTile * nin + 4 * kTile * kH + 6 * kTile) * sizeof(float) + kTile * sizeof(int);
+static size_t tile_smem(int nin, int ts) {
+  return (size_t)(kH * kH + kH * (kH + 1) + 4 * ts * kH + nin * kH + ts * nin + 4 * kH + 2 + 6 * ts) * sizeof(float) +
+         ts * sizeof(int);
 }
 
-static cudaError_t tile_attr(int nin) {
-  return cudaFuncSetAttribute(mlp_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tile_smem(nin));
+// samples per tile: about one tile per SM, so that neither the samples of one CTA nor the number of
+// gradient partials grows beyond what the batch needs
+static int tile_samples(int64_t count) { return count <= 8 * 152 ? 8 : (count <= 16 * 304 ? 16 : (count <= 32 * 608 ? 32 : 64)); }
+
+static cudaError_t launch_tiles(int ts, int tiles, const TileArgs &a, int forward_only, cudaStream_t s) {
+  const size_t smem = tile_smem(a.nin, ts);
+  auto go = [&](auto k) -> cudaError_t {
+    if (smem > 48 * 1024) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    k<<<tiles, kMlpT, smem, s>>>(a, forward_only);
+    return cudaGetLastError();
+  };
+  switch (ts) {
+    case 8: return go(mlp_tile_kernel<8>);
+    case 16: return go(mlp_tile_kernel<16>);
+    case 32: return go(mlp_tile_kernel<32>);
+    default: return go(mlp_tile_kernel<64>);
+  }
+}
+
+static cudaError_t launch_reduce(const float *gpart, const float *lpart, int tiles, int P, float scale, float *grad, float *loss,
+                                 float *params, float *m, float *v, float lr, float b1c, float b2c, int adam, cudaStream_t s) {
+  mlp_reduce_kernel<<<(P + kRedP - 1) / kRedP, kRedP * kRedSlices, 0, s>>>(gpart, lpart, tiles, P, scale, grad, loss, params, m,
+                                                                         v, lr, b1c, b2c, adam);
+  return cudaGetLastError();
 }
 
 cudaError_t mlp_grad(const float *params, int nin, int N, const float *X, const float *Y, int64_t M, float *grad,
                      float *loss, cudaStream_t s) {
-  const int P = mlp_nparams(nin);
-  const int tiles = (int)((M + kTile - 1) / kTile);
+  const int P = mlp_nparams(nin), ts = tile_samples(M);
+  const int tiles = (int)((M + ts - 1) / ts);
   float *gpart = nullptr, *lpart = nullptr;
   cudaError_t e = cudaMalloc(&gpart, (size_t)tiles * P * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&lpart, (size_t)tiles * sizeof(float));
-  if (e == cudaSuccess) e = tile_attr(nin);
   if (e == cudaSuccess) {
     TileArgs a{params, nin, N, X, Y, M, 0, M, 0, 0, gpart, lpart, nullptr, 0};
-    mlp_tile_kernel<<<tiles, 256, tile_smem(nin), s>>>(a, 0);
-    mlp_reduce_kernel<<<(P + 255) / 256, 256, 0, s>>>(gpart, lpart, tiles, P, 1.f / (float)M, grad, loss, nullptr,
-                                                     nullptr, nullptr, 0.f, 1.f, 1.f, 0);
-    e = cudaGetLastError();
+    e = launch_tiles(ts, tiles, a, 0, s);
+    if (e == cudaSuccess)
+      e = launch_reduce(gpart, lpart, tiles, P, 1.f / (float)M, grad, loss, nullptr, nullptr, nullptr, 0.f, 1.f, 1.f, 0, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   }
   cudaFree(gpart);
@@ -547,12 +667,9 @@ cudaError_t mlp_grad(const float *params, int nin, int N, const float *X, const 
 
 cudaError_t mlp_forward(const float *params, int nin, int N, const float *X, int64_t M, int bf16, float *out,
                         cudaStream_t s) {
-  cudaError_t e = tile_attr(nin);
-  if (e != cudaSuccess) return e;
-  const int tiles = (int)((M + kTile - 1) / kTile);
+  const int ts = tile_samples(M), tiles = (int)((M + ts - 1) / ts);
   TileArgs a{params, nin, N, X, nullptr, M, 0, M, 0, 0, nullptr, nullptr, out, bf16};
-  mlp_tile_kernel<<<tiles, 256, tile_smem(nin), s>>>(a, 1);
-  e = cudaGetLastError();
+  cudaError_t e = launch_tiles(ts, tiles, a, 1, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   return e;
 }
@@ -561,37 +678,35 @@ cudaError_t mlp_train(float *params, float *m, float *v, int nin, int N, const f
                       int batch, int epochs, float lr, uint64_t seed, int64_t *adam_t, float *loss_hist,
                       cudaStream_t s) {
   const int P = mlp_nparams(nin);
-  const int tiles = (batch + kTile - 1) / kTile;
+  const int64_t most = std::min<int64_t>(batch, M), nb = (M + batch - 1) / batch;
+  const int ts = tile_samples(most), tiles = (int)((most + ts - 1) / ts);
   int h = 1;
   while ((int64_t)1 << (2 * h) < M) ++h;
+  // the loss of every minibatch stays on the device and is read once an epoch
   float *gpart = nullptr, *lpart = nullptr, *dloss = nullptr;
   cudaError_t e = cudaMalloc(&gpart, (size_t)tiles * P * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&lpart, (size_t)tiles * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&dloss, sizeof(float));
-  if (e == cudaSuccess) e = tile_attr(nin);
+  if (e == cudaSuccess) e = cudaMalloc(&dloss, (size_t)nb * sizeof(float));
+  std::vector<float> hl((size_t)nb);
   for (int ep = 0; ep < epochs && e == cudaSuccess; ++ep) {
-    double lsum = 0.0;
-    int64_t nb = 0;
     const uint64_t key = seed * 0x9E3779B97F4A7C15ull + (uint64_t)ep;
-    for (int64_t start = 0; start < M && e == cudaSuccess; start += batch) {
-      const int64_t cnt = std::min<int64_t>(batch, M - start);
-      const int tl = (int)((cnt + kTile - 1) / kTile);
+    for (int64_t k = 0; k < nb && e == cudaSuccess; ++k) {
+      const int64_t start = k * batch, cnt = std::min<int64_t>(batch, M - start);
+      const int tl = (int)((cnt + ts - 1) / ts);
       TileArgs a{params, nin, N, X, Y, M, start, cnt, h, key, gpart, lpart, nullptr, 0};
-      mlp_tile_kernel<<<tl, 256, tile_smem(nin), s>>>(a, 0);
+      e = launch_tiles(ts, tl, a, 0, s);
       const int64_t t = ++(*adam_t);
       const float b1c = 1.f - powf(0.9f, (float)t), b2c = 1.f - powf(0.999f, (float)t);
-      mlp_reduce_kernel<<<(P + 255) / 256, 256, 0, s>>>(gpart, lpart, tl, P, 1.f / (float)cnt, nullptr, dloss, params,
-                                                       m, v, lr, b1c, b2c, 1);
-      e = cudaGetLastError();
-      if (loss_hist && e == cudaSuccess) {
-        float l = 0.f;
-        e = cudaMemcpyAsync(&l, dloss, sizeof(float), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        lsum += l * (double)cnt;
-        nb += cnt;
-      }
+      if (e == cudaSuccess)
+        e = launch_reduce(gpart, lpart, tl, P, 1.f / (float)cnt, nullptr, dloss + k, params, m, v, lr, b1c, b2c, 1, s);
     }
-    if (loss_hist && nb > 0) loss_hist[ep] = (float)(lsum / (double)nb);
+    if (loss_hist && e == cudaSuccess) {
+      e = cudaMemcpyAsync(hl.data(), dloss, (size_t)nb * sizeof(float), cudaMemcpyDeviceToHost, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      double lsum = 0.0;
+      for (int64_t k = 0; k < nb; ++k) lsum += (double)hl[k] * (double)std::min<int64_t>(batch, M - k * batch);
+      if (M > 0) loss_hist[ep] = (float)(lsum / (double)M);
+    }
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   cudaFree(gpart);
