@@ -74,7 +74,9 @@ struct selbm {
   int32_t *d_loc_u = nullptr, *d_loc_off = nullptr, *d_loc_slot = nullptr, *d_loc_base = nullptr, *d_rem_off = nullptr,
           *d_rem = nullptr, *d_bas_off = nullptr, *d_bas = nullptr;
   int flow_rmax = 0, flow_bmax = 0;
-  void *d_flow_T = nullptr, *d_flow_base = nullptr;
+  void *d_flow_T = nullptr, *d_flow_base = nullptr, *d_flow_sums = nullptr;
+  int flow_learned = -1;         // whether the resident step with the learned control fits (-1: not asked)
+  int flow_pass = 0;
   int *abort_host = nullptr;     // mapped host memory: a bounded wait of the resident step gave up
   int wall_max = 0;
   int n_wallpts = 0;             // wall points (element, node) over all elements
@@ -207,7 +209,7 @@ cudaError_t setup_flow2d(selbm *h) {
   Flow2DArgs<Real> a{};
   a.E = S.E; a.epc = epc; a.rmax = rmax; a.bmax = bmax;
   bool fits = false;
-  e = launch_flow2d<Real>(S.N, S.affine, true, a, split_host(h), &fits, h->stream);
+  e = launch_flow2d<Real>(S.N, S.affine, true, a, split_host(h), nullptr, &fits, h->stream);
   if (e != cudaSuccess || !fits) return e;
   auto keep = [&](int32_t **d, const std::vector<int32_t> &v) -> cudaError_t {
     const cudaError_t r = upload(d, v);
@@ -226,6 +228,7 @@ cudaError_t setup_flow2d(selbm *h) {
     return r;
   };
   if ((e = alloc(&h->d_flow_T, (size_t)4 * S.E * 9 * Nb * sizeof(Real)))) return e;
+  if ((e = alloc((void **)&h->d_flow_sums, (size_t)2 * grid * 2 * 16))) return e;
   if ((e = alloc(&h->d_flow_base, (size_t)S.Gb * 20 * sizeof(Real)))) return e;
   if (!S.affine && sizeof(Real) == 8) {
     std::vector<int> ex(S.E);
@@ -756,7 +759,7 @@ int wait_status(selbm *h) {
 
 // nsteps steps of the resident 2D step, in launches of a bounded length
 template <typename Real>
-cudaError_t run_flow2d(selbm *h, int64_t nsteps) {
+cudaError_t run_flow2d(selbm *h, int64_t nsteps, bool probe = false) {
   const KParams<Real> k = base_params<Real>(h);
   Flow2DArgs<Real> a{};
   a.E = k.E; a.Gs = k.Gs; a.epc = h->flow_epc;
@@ -772,13 +775,31 @@ cudaError_t run_flow2d(selbm *h, int64_t nsteps) {
   a.abort = h->abort_host;
   a.T = h->d_flow_T; a.base = h->d_flow_base; a.f = (Real *)h->FA;
   const SplitHost sh = split_host(h);
+  Learn2DArgs<Real> lc{};
+  if (h->learned) {
+    a.filter = 1;
+    lc.W = h->d_W; lc.lo = (const Real *)h->d_lo; lc.hi = (const Real *)h->d_hi; lc.Vinv = (const Real *)h->d_Vinv;
+    lc.flag = h->d_flag; lc.n_fallback = h->d_nfb; lc.acc = h->d_acc; lc.sigma_out = (Real *)h->d_sigma_e;
+    lc.sums = (Packet<double> *)h->d_flow_sums;
+    lc.mass_bound = h->mass_bound; lc.ke_bound = h->ke_bound; lc.check_ke = h->has_force ? 0 : 1;
+  }
+  if (probe) {
+    bool fits = false;
+    const cudaError_t e = launch_flow2d<Real>(h->S.N, h->S.affine, true, a, sh, &lc, &fits, h->stream);
+    h->flow_learned = e == cudaSuccess && fits ? 1 : 0;
+    cudaGetLastError();
+    return cudaSuccess;
+  }
   while (nsteps > 0) {
     a.nsteps = (int)std::min<int64_t>(nsteps, 20000);
     a.pending = h->filter_pending;
     a.epoch = h->flow_epoch;
-    const cudaError_t e = launch_flow2d<Real>(h->S.N, h->S.affine, false, a, sh, nullptr, h->stream);
+    lc.pass = h->flow_pass;
+    const cudaError_t e = launch_flow2d<Real>(h->S.N, h->S.affine, false, a, sh, h->learned ? &lc : nullptr, nullptr, h->stream);
     if (e != cudaSuccess) return e;
-    h->flow_epoch += 3u * (unsigned)a.nsteps;
+    const int passes = h->learned ? a.nsteps - (h->filter_pending ? 0 : 1) : 0;
+    h->flow_epoch += 3u * (unsigned)a.nsteps + (unsigned)passes;
+    h->flow_pass = (h->flow_pass + passes) & 1;
     h->filter_pending = true;
     for (int s = 0; s < a.nsteps; ++s) h->time += h->dt;
     h->steps += a.nsteps;
@@ -1037,7 +1058,11 @@ int selbm_step(selbm_t *h, int64_t nsteps) {
   if (!h) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
   if (nsteps < 0) return h->fail(SELBM_ERR_ARG, "nsteps < 0");
-  if (h->flow_epc > 0 && !h->timing && !h->learned && !h->field_on && h->scheme == 0) {
+  if (h->learned && h->flow_epc > 0 && h->flow_learned < 0) {
+    if (h->prec == SELBM_FP64) run_flow2d<double>(h, 0, true);
+    else run_flow2d<float>(h, 0, true);
+  }
+  if (h->flow_epc > 0 && !h->timing && !h->field_on && h->scheme == 0 && (!h->learned || h->flow_learned == 1)) {
     const cudaError_t e = h->prec == SELBM_FP64 ? run_flow2d<double>(h, nsteps) : run_flow2d<float>(h, nsteps);
     return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "step");
   }

@@ -33,6 +33,11 @@ struct Flow2DShape {
   // most threads of a CTA (FP64 and long lines need the registers)
   static constexpr int TMAX = F64 || n > 10 ? 512 : 768;
   static constexpr int COPIES = 4;                       // copies of a node kept in shared memory (more: from L2)
+  // learned control: network, V^-1; per element features, hidden layers, transfer function
+  static constexpr size_t learned_bytes(int epc) {
+    return (size_t)(2 * n * 64 + 64 * 65 + 2 * 64 + 2 * 64 + 2) * sizeof(float) + (size_t)(n * n + 4 * n) * sizeof(Real) + 64 +
+           (size_t)epc * ((2 * n + 2 * 64 + 2) * sizeof(Real) + n * sizeof(Val) + n * sizeof(Real) + 2 * sizeof(int));
+  }
   // shared memory of one element: f, f^0, sums; weights and rho; wall terms; coefficients; copies
   static constexpr size_t element_bytes(bool affine, bool node) {
     return (node ? (size_t)9 * PS * sizeof(Limb) : 0) +
@@ -43,12 +48,6 @@ struct Flow2DShape {
   static constexpr size_t fixed_bytes(bool node) { return (node ? (size_t)n * n * sizeof(Limb) : 0) + (size_t)n * (sizeof(Val) + sizeof(Real)) + (size_t)(Nb + Np + M * M) * sizeof(int) + 64; }
 };
 
-// a value and the number of its exchange: 8 bytes per 32 bits of the value, each written and read
-// as one access
-template <typename Real>
-struct Packet {
-  unsigned long long w[sizeof(Real) / 4];
-};
 __device__ __forceinline__ void put_packet(Packet<float> *p, float v, unsigned tag) {
   __stcg(&p->w[0], ((unsigned long long)tag << 32) | __float_as_uint(v));
 }
@@ -108,9 +107,10 @@ __device__ __forceinline__ float as_val(float v) { return v; }
 __device__ __forceinline__ long long as_val(double v) { return __double_as_longlong(v); }
 
 // NODE (FP64): one thread per (population, node) and stage instead of lines; see launch_flow2d_t
-template <typename Real, int n, bool AFFINE, bool NODE>
+template <typename Real, int n, bool AFFINE, bool NODE, bool LEARNED>
 __global__ void __launch_bounds__(Flow2DShape<Real, n>::TMAX, 1)
-flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const FilterMats<Real, n> fm, const CollideFix cfix) {
+flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const FilterMats<Real, n> fm, const CollideFix cfix,
+              const Learn2DArgs<Real> lc) {
   using S = Flow2DShape<Real, n>;
   using Val = LineVal<Real>;
   constexpr bool F64 = S::F64;
@@ -120,7 +120,20 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int epc = p.epc, e0 = blockIdx.x * epc, ne = min(epc, p.E - e0), tid = threadIdx.x, T = blockDim.x;
   Val *X = reinterpret_cast<Val *>(smem_raw);          // [ne][9][PS] sums of the passes
-  Val *cf = X + (size_t)epc * 9 * PS;                   // affine [ne][9][2]: -dt e.grad r_l; curved [ne][4][PS]: dr_l/dx_k
+  Val *sge = X + (size_t)epc * 9 * PS;                  // LEARNED: [ne][n] sigma_k - 1 of the elements
+  Real *sVi = reinterpret_cast<Real *>(sge + (LEARNED ? (size_t)epc * n : 0));   // LEARNED: [n][n] V^-1, ...
+  Real *sX = sVi + (LEARNED ? n * n : 0);               // [ne][2n] features, then scaled inputs
+  Real *sH1 = sX + (LEARNED ? epc * 2 * n : 0);         // [ne][64]
+  Real *sH2 = sH1 + (LEARNED ? epc * 64 : 0);           // [ne][64]
+  Real *sO = sH2 + (LEARNED ? epc * 64 : 0);            // [ne][2]
+  Real *slh = sO + (LEARNED ? epc * 2 : 0);             // [4n] lo, hi
+  Real *sged = slh + (LEARNED ? 4 * n : 0);             // [ne][n] sigma_k - 1 as a Real
+  float *sW1 = reinterpret_cast<float *>(sged + (LEARNED ? epc * n : 0));   // [2n][64] W1 transposed
+  float *sW2 = sW1 + (LEARNED ? 2 * n * 64 : 0);        // [64][65] W2 transposed
+  float *sb = sW2 + (LEARNED ? 64 * 65 : 0);            // b1[64], b2[64], W3[2][64], b3[2]
+  int *sin = reinterpret_cast<int *>(sb + (LEARNED ? 4 * 64 + 2 : 0));      // [ne] features in range
+  Val *cf = reinterpret_cast<Val *>(smem_raw + (LEARNED ? (((unsigned char *)(sin + epc) - smem_raw) + 15) / 16 * 16
+                                                        : (size_t)epc * 9 * PS * sizeof(Val)));   // affine [ne][9][2]: -dt e.grad r_l; curved [ne][4][PS]: dr_l/dx_k
   Limb *FQ = reinterpret_cast<Limb *>(cf + (size_t)epc * (AFFINE ? 18 : 4 * PS));   // NODE: [ne][9][PS] f in fixed point
   Limb *sD = FQ + (NODE ? (size_t)epc * 9 * PS : 0);    // NODE: [n][n] D_hat
   Val *sgk = reinterpret_cast<Val *>(sD + (NODE ? n * n : 0));   // [n] sigma_k - 1
@@ -144,7 +157,8 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   int *bi = sbrem + p.bmax;                             // [Nb] tile offset of boundary node b
   int *off = bi + Nb;                                   // [Np] tile offset of local node i
   int *ini = off + Np;                                  // [M M] tile offset of the element-interior nodes
-  __shared__ int s_fail;
+  __shared__ int s_fail, s_flag;
+  __shared__ double s_red[2][Flow2DShape<Real, n>::TMAX / 32], s_prev[3];
   __shared__ Real s_t[9], s_c[9];                       // weights; B dt 3 t_a e_a . g / B
   __shared__ signed char s_e[9][2], s_o[9];
   __shared__ Limb s_tc[9];                              // t_a / 2 in fixed point
@@ -259,6 +273,26 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
       }
     }
   }
+  if constexpr (LEARNED) {
+    const __nv_bfloat16 *W1 = lc.W, *B1 = W1 + 64 * 2 * n, *W2 = B1 + 64, *B2 = W2 + 64 * 64, *W3 = B2 + 64, *B3 = W3 + 128;
+#pragma unroll 1
+    for (int k = tid; k < 64 * 2 * n; k += T) sW1[(k % (2 * n)) * 64 + k / (2 * n)] = __bfloat162float(W1[k]);
+#pragma unroll 1
+    for (int k = tid; k < 64 * 64; k += T) sW2[(k % 64) * 65 + k / 64] = __bfloat162float(W2[k]);
+#pragma unroll 1
+    for (int k = tid; k < 64; k += T) {
+      sb[k] = __bfloat162float(B1[k]);
+      sb[64 + k] = __bfloat162float(B2[k]);
+      sb[128 + k] = __bfloat162float(W3[k]);
+      sb[192 + k] = __bfloat162float(W3[64 + k]);
+    }
+    if (tid < 2) sb[256 + tid] = __bfloat162float(B3[tid]);
+#pragma unroll 1
+    for (int k = tid; k < n * n; k += T) sVi[k] = lc.Vinv[k];
+    if (tid < 2 * n) { slh[tid] = lc.lo[tid]; slh[2 * n + tid] = lc.hi[tid]; }
+    if (tid < 3) s_prev[tid] = lc.acc[2 + tid];
+    if (tid == 0) s_flag = *lc.flag;
+  }
   auto track = [&](int par, int el, int a, Real v) {     // exponent of a value written to F
     if constexpr (F64) atomicMax(&em[(par * epc + el) * 9 + a], exp_of(v));
   };
@@ -327,11 +361,172 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   using Cn = std::integral_constant<int, n>;
   const int ntile = 9 * ne;
 
+  // packets of other CTAs into shared memory: a thread looks at two before it waits for one
+        auto fetch = [&](int pops, int count, auto address, Real *dst) {   // dst [pops][count]
+          constexpr int U = 2;
+          const int blocks = (count + 31) >> 5;
+  #pragma unroll 1
+          for (int w = warp; w < pops * blocks; w += U * nwarp) {
+            Real v[U];
+            const Packet<Real> *src[U];
+            Real *to[U];
+            bool ok[U];
+  #pragma unroll
+            for (int c = 0; c < U; ++c) {
+              const int wc = w + c * nwarp, a = wc / blocks, r = (wc - a * blocks) * 32 + lane;
+              ok[c] = true;
+              to[c] = nullptr;
+              if (wc < pops * blocks && r < count) {
+                src[c] = address(a, r);
+                to[c] = dst + a * count + r;
+                ok[c] = get_packet(src[c], epoch, v[c]);
+              }
+            }
+  #pragma unroll
+            for (int c = 0; c < U; ++c) {
+              if (!ok[c]) v[c] = wait_packet(src[c]);
+              if (to[c]) *to[c] = v[c];
+            }
+          }
+        };
+  // sum of the shares of local boundary node b's copies, population tile q, in ascending copy order
+  auto copies_sum = [&](int q, int b) -> Real {
+    const int el = q / 9, a = q - 9 * el, lb = el * Nb + b;
+    const Real *xa = reinterpret_cast<const Real *>(X) + a * PS, *ra = R + a * nrem;
+    const int *sl = sslot + lb * COPIES;
+    Real sum = 0;
+    if (sl[0] != -2) {
+#pragma unroll
+      for (int c = 0; c < COPIES; ++c) {
+        const int s = sl[c];
+        if (s != -1) sum += s >= 0 ? ra[s] : xa[-3 - s];
+      }
+    } else {
+      const size_t lg = (size_t)e0 * Nb + lb;
+#pragma unroll 1
+      for (int c = p.loc_off[lg]; c < p.loc_off[lg + 1]; ++c) {
+        const int s = local(p.loc_slot[c]);
+        sum += s >= 0 ? ra[s] : xa[-3 - s];
+      }
+    }
+    return sum;
+  };
+
   // The phases are rolled loops over axes, populations and nodes where that costs little: the code
   // of a step has to stay in the instruction cache, since every phase runs it once.
 #pragma unroll 1
   for (int step = 0; step < p.nsteps; ++step) {
     const bool filt = p.filter && (step > 0 || p.pending);
+    const bool owners = filt && !LEARNED;                  // copies filtered apart: the owner's f^0 stands
+    const int pass = LEARNED ? lc.pass + step - (p.pending ? 0 : 1) : 0;   // control pass of this step
+    const unsigned pass_tag = epoch + 1;
+    // ---- learned control: the element's transfer function from the modal energies of rho - rho0
+    //      and |u|, the drift sums, the network (BF16 weights)
+    if (LEARNED && filt) {
+      Real *fld = reinterpret_cast<Real *>(X);             // [ne][9][PS]: planes 0, 1 of each element
+      double pm = 0, pk = 0;
+      tiles(CNp{}, ne, [&](int el, int i) {
+        const int o = off[i], at = el * 9 * PS + o;
+        Real drho = 0, jx = 0, jy = 0;
+#pragma unroll
+        for (int a = 0; a < 9; ++a) {
+          const Real v = F[at + a * PS];
+          drho += v;
+          if (V.e[a][0] > 0) jx += v;
+          else if (V.e[a][0] < 0) jx -= v;
+          if (V.e[a][1] > 0) jy += v;
+          else if (V.e[a][1] < 0) jy -= v;
+        }
+        const Real rho = p.rho0 + drho, ux = jx / rho, uy = jy / rho, uu = ux * ux + uy * uy;
+        fld[at] = drho;
+        fld[at + PS] = sqrt(uu);
+        const Real wq = AFFINE ? p.el_J[e0 + el] * m.w[i % n] * m.w[i / n] : p.wJ[(size_t)(e0 + el) * Np + i];
+        pm += wide(wq) * wide(rho);
+        pk += wide(wq) * wide(uu);
+      });
+      pm = warp_sum(pm);
+      pk = warp_sum(pk);
+      if (lane == 0) { s_red[0][warp] = pm; s_red[1][warp] = pk; }
+      __syncthreads();
+      if (tid < 2) {
+        double s = 0;
+        for (int w = 0; w < nwarp; ++w) s += s_red[tid][w];
+        if (tid == 1) s *= 0.5 * (double)p.rho0;
+        put_packet(lc.sums + ((size_t)(pass & 1) * gridDim.x + blockIdx.x) * 2 + tid, s, epoch + 1);
+      }
+#pragma unroll 1
+      for (int ax = 0; ax < 2; ++ax) {
+        const int lst = ax ? 1 : LS, stp = ax ? LS : 1;
+        tiles(Cn{}, 2 * ne, [&](int q, int L) {
+          Real *row = fld + ((q >> 1) * 9 + (q & 1)) * PS + lst * L;
+          Real v[n];
+#pragma unroll
+          for (int k = 0; k < n; ++k) v[k] = row[k * stp];
+#pragma unroll 1
+          for (int j = 0; j < n; ++j) {
+            Real s = 0;
+#pragma unroll
+            for (int k = 0; k < n; ++k) s += sVi[j * n + k] * v[k];
+            row[j * stp] = s;
+          }
+        });
+        if (tid < ne) sin[tid] = 1;
+        __syncthreads();
+      }
+      // shell k: modes whose larger index is k
+      tiles(Cn{}, 2 * ne, [&](int q, int k) {
+        const int el = q >> 1, fi = q & 1;
+        const Real *c = fld + (el * 9 + fi) * PS;
+        Real s = 0;
+        for (int i = 0; i <= k; ++i) s += c[i + LS * k] * c[i + LS * k];
+        for (int i = 0; i < k; ++i) s += c[k + LS * i] * c[k + LS * i];
+        const Real x = log10(s + Real(1e-30)), lo = slh[fi * n + k], hi = slh[2 * n + fi * n + k];
+        if (!(x >= lo && x <= hi)) sin[el] = 0;
+        sX[el * 2 * n + fi * n + k] = Real(2) * (x - lo) / (hi - lo) - Real(1);
+      });
+      __syncthreads();
+      using C64 = std::integral_constant<int, 64>;
+      tiles(C64{}, ne, [&](int el, int o) {
+        Real z = (Real)sb[o];
+        for (int i = 0; i < 2 * n; ++i) z += (Real)sW1[i * 64 + o] * sX[el * 2 * n + i];
+        sH1[el * 64 + o] = tanh(z);
+      });
+      __syncthreads();
+      tiles(C64{}, ne, [&](int el, int o) {
+        Real z = (Real)sb[64 + o];
+        for (int i = 0; i < 64; ++i) z += (Real)sW2[i * 65 + o] * sH1[el * 64 + i];
+        sH2[el * 64 + o] = tanh(z);
+      });
+      __syncthreads();
+#pragma unroll 1
+      for (int t = warp; t < 2 * ne; t += nwarp) {
+        const int el = t >> 1, o = t & 1;
+        Real z = (Real)sb[128 + 64 * o + lane] * sH2[el * 64 + lane] + (Real)sb[128 + 64 * o + 32 + lane] * sH2[el * 64 + 32 + lane];
+        z = warp_sum(z);
+        if (lane == 0) sO[t] = z + (Real)sb[256 + o];
+      }
+      __syncthreads();
+      tiles(Cn{}, ne, [&](int el, int k) {
+        const bool use_net = sin[el] && !s_flag;
+        Real g = fm.g[k];
+        if (use_net) {
+          const Real gam = Real(0.5) / (Real(1) + exp(-sO[2 * el])), kc = Real(2) + Real(n - 4) / (Real(1) + exp(-sO[2 * el + 1]));
+          g = 0;
+          if (k > kc) {
+            const Real r = (Real(k) - kc) / (Real(n - 1) - kc);
+            // sigma = 1 - gamma r^2 rounded as the transfer function that is handed out
+            g = (Real(1) - gam * r * r) - Real(1);
+          }
+        } else if (k == 0) {
+          atomicAdd(lc.n_fallback, 1);
+        }
+        sged[el * n + k] = g;
+        if constexpr (F64) sge[el * n + k] = __double2ll_rn(g * 0x1p60);
+        else sge[el * n + k] = g;
+        lc.sigma_out[(size_t)(e0 + el) * n + k] = g + Real(1);
+      });
+      __syncthreads();
+    }
     // ---- explicit filter of the previous step (Sec. 2.4), r- then s-lines
     if (filt) {
       Val *Y = X;                                           // FP64: the tile in fixed point
@@ -352,11 +547,11 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
           for (int k = 0; k < n; ++k) v[k] = row[k * st];
           if constexpr (F64) {
             if (em[par * epc * 9 + q] == 2047) {
-              slow_filter_row<n>(fm, sgd, row, st);
+              slow_filter_row<n>(fm, LEARNED ? sged + q / 9 * n : sgd, row, st);
               return;
             }
-            line_filter<n>(fm, sgk, v);
-          } else line_filter<n>(fm, sgk, v);
+            line_filter<n>(fm, LEARNED ? sge + q / 9 * n : sgk, v);
+          } else line_filter<n>(fm, LEARNED ? sge + q / 9 * n : sgk, v);
 #pragma unroll
           for (int k = 1; k < n - 1; ++k) row[k * st] = v[k];
         });
@@ -369,6 +564,22 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
         });
         __syncthreads();
       }
+    }
+    // ---- element-dependent filters: the copies of a shared node take their mass-weighted average
+    if (LEARNED && filt) {
+      ++epoch;
+      Packet<Real> *Tb = reinterpret_cast<Packet<Real> *>(p.T) + (size_t)(epoch & 1u) * p.E * Nb * 9;
+      tiles(CNb{}, ntile, [&](int q, int b) {
+        const int at = q * PS + bi[b];
+        const Real v = wj[q / 9 * Nb + b] * F[at];
+        put_packet(Tb + (e0 * 9 + q) * Nb + b, v, epoch);
+        X[at] = as_val(v);
+      });
+      fetch(9, nrem, [&](int a, int r) { return Tb + srem[r] + a * Nb; }, R);
+      __syncthreads();
+      tiles(CNb{}, ntile, [&](int q, int b) { F[q * PS + bi[b]] = copies_sum(q, b) * sminv[q / 9 * Nb + b]; });
+      __syncthreads();
+      if (s_fail) return;
     }
     // ---- BGK collision at every local node; after a filter the owner's f^0 of a shared node
     //      stands for all copies (their lines were filtered in different element frames)
@@ -423,7 +634,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
         }
         if (forced) {
           srho[el * PS + off[i]] = rho;
-          if (filt) publish(el, i, 9, rho);
+          if (owners) publish(el, i, 9, rho);
         }
       });
       __syncthreads();
@@ -443,7 +654,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
         }
         F[at] = v;
         F0[at] = v;
-        if (filt) publish(el, i, a, v);
+        if (owners) publish(el, i, a, v);
         track_max(emn, q, exp_of(v));
       });
     } else {
@@ -459,7 +670,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
           F0[at + a * PS] = f[a];
         }
         if (forced) srho[el * PS + off[i]] = rho;
-        if (filt) {
+        if (owners) {
           const int b = p.bslot[i];
           if (b >= 0 && p.owner[(size_t)(e0 + el) * Np + i]) {
             Packet<Real> *base = reinterpret_cast<Packet<Real> *>(p.base) + (size_t)p.loc_u[(size_t)(e0 + el) * Nb + b] * 10;
@@ -611,36 +822,8 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
         F[at] = v;
         if (F64) track_max(emn, q, exp_of(v));
       });
-      // the shares of other CTAs (and after a filter the owners' f^0): a thread looks at several
-      // packets before it waits for one
-      const bool owner_base = st == 0 && filt;
-      auto fetch = [&](int pops, int count, auto address, Real *dst) {   // dst [pops][count]
-        constexpr int U = 2;
-        const int blocks = (count + 31) >> 5;
-#pragma unroll 1
-        for (int w = warp; w < pops * blocks; w += U * nwarp) {
-          Real v[U];
-          const Packet<Real> *src[U];
-          Real *to[U];
-          bool ok[U];
-#pragma unroll
-          for (int c = 0; c < U; ++c) {
-            const int wc = w + c * nwarp, a = wc / blocks, r = (wc - a * blocks) * 32 + lane;
-            ok[c] = true;
-            to[c] = nullptr;
-            if (wc < pops * blocks && r < count) {
-              src[c] = address(a, r);
-              to[c] = dst + a * count + r;
-              ok[c] = get_packet(src[c], epoch, v[c]);
-            }
-          }
-#pragma unroll
-          for (int c = 0; c < U; ++c) {
-            if (!ok[c]) v[c] = wait_packet(src[c]);
-            if (to[c]) *to[c] = v[c];
-          }
-        }
-      };
+      // the shares of other CTAs (and after a filter the owners' f^0)
+      const bool owner_base = st == 0 && owners;
       fetch(9, nrem, [&](int a, int r) { return Tb + srem[r] + a * Nb; }, R);
       if (owner_base)
         fetch(forced ? 10 : 9, nbas,
@@ -649,22 +832,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
       // assembly at the element-boundary nodes: f^0 + B (f^{s-1} - f^0) + sum_c T_c / M + B dt F*
       tiles(CNb{}, ntile, [&](int q, int b) {
         const int el = q / 9, a = q - 9 * el, lb = el * Nb + b, o = bi[b], at = q * PS + o;
-        const Real *xa = reinterpret_cast<const Real *>(X) + a * PS, *ra = R + a * nrem;
-        const int *sl = sslot + lb * COPIES;
-        Real sum = 0;
-        if (sl[0] != -2) {
-#pragma unroll
-          for (int c = 0; c < COPIES; ++c) {
-            const int s = sl[c];
-            if (s != -1) sum += s >= 0 ? ra[s] : xa[-3 - s];
-          }
-        } else {
-          const size_t lg = (size_t)e0 * Nb + lb;
-          for (int c = p.loc_off[lg]; c < p.loc_off[lg + 1]; ++c) {
-            const int s = local(p.loc_slot[c]);
-            sum += s >= 0 ? ra[s] : xa[-3 - s];
-          }
-        }
+        const Real sum = copies_sum(q, b);
         Real f0v = F0[at], fv = F[at];
         const int ob = owner_base ? sbase[lb] : -1;
         if (ob != -1) f0v = fv = ob >= 0 ? Rb[a * nbas + ob] : F0[-3 - ob + a * PS];
@@ -679,6 +847,39 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
         F[at] = y;
         if (F64) track_max(emn, q, exp_of(y));
       });
+      // learned control, last stage: the drift sums of this step's pass over all CTAs, in a fixed
+      // order, against those of the pass before (the fallback holds from the next pass on)
+      if (LEARNED && st == 2 && filt && warp == nwarp - 1) {
+        double sum[2] = {0, 0};
+#pragma unroll 1
+        for (int c = lane; c < (int)gridDim.x; c += 32)
+#pragma unroll 1
+          for (int k = 0; k < 2; ++k) {
+            const Packet<double> *src = lc.sums + ((size_t)(pass & 1) * gridDim.x + c) * 2 + k;
+            double v;
+            int spin = 0;
+            while (!get_packet(src, pass_tag, v)) {
+              if (++spin >= kFlowSpins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
+                *(volatile int *)p.abort = 1;
+                s_fail = 1;
+                break;
+              }
+            }
+            sum[k] += v;
+          }
+        sum[0] = warp_sum(sum[0]);
+        sum[1] = warp_sum(sum[1]);
+        if (lane == 0) {
+          if (s_prev[2] != 0.0) {
+            const double dm = fabs(sum[0] - s_prev[0]) / fabs(s_prev[0]);
+            const bool up = lc.check_ke && lc.ke_bound > 0.0 && sum[1] > s_prev[1] * (1.0 + lc.ke_bound);
+            if (dm > lc.mass_bound || up) s_flag = 1;
+          }
+          s_prev[0] = sum[0];
+          s_prev[1] = sum[1];
+          s_prev[2] = 1.0;
+        }
+      }
       __syncthreads();
       if (s_fail) return;
       // the owner's f^0 and rho stand for all copies in the later stages too (the owners' own
@@ -695,6 +896,10 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
       par ^= 1;
     }
   }
+  if (LEARNED && blockIdx.x == 0) {
+    if (tid < 3) lc.acc[2 + tid] = s_prev[tid];
+    if (tid == 0) *lc.flag = s_flag;
+  }
   // ---- the state back to the unique nodes (every copy of a shared node holds the same bits)
 #pragma unroll 1
   for (int k = tid; k < ne * Np; k += T) {
@@ -706,8 +911,10 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   }
 }
 
-template <typename Real, int n>
-cudaError_t launch_flow2d_t(const Flow2DArgs<Real> &p, const SplitHost &h, bool affine, bool probe, bool *fits, cudaStream_t s) {
+// L2D: the kernels with the learned control
+template <typename Real, int n, bool L2D>
+cudaError_t launch_flow2d_t(const Flow2DArgs<Real> &p, const SplitHost &h, bool affine, bool probe,
+                            const Learn2DArgs<Real> *lc, bool *fits, cudaStream_t s) {
   using S = Flow2DShape<Real, n>;
   int dev = 0, sms = 0, most = 0, coop = 0;
   cudaError_t e;
@@ -716,30 +923,45 @@ cudaError_t launch_flow2d_t(const Flow2DArgs<Real> &p, const SplitHost &h, bool 
       (e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev)))
     return e;
   const size_t fetched = p.rmax * (9 * sizeof(Real) + sizeof(int)) + p.bmax * (10 * sizeof(Real) + sizeof(int));
-  auto bytes = [&](bool node) { return S::fixed_bytes(node) + p.epc * S::element_bytes(affine, node) + fetched; };
+  auto bytes = [&](bool node) {
+    return S::fixed_bytes(node) + p.epc * S::element_bytes(affine, node) + fetched + (lc ? S::learned_bytes(p.epc) : 0);
+  };
   if (probe) {
     *fits = coop && (p.E + p.epc - 1) / p.epc <= sms && bytes(false) <= (size_t)most - 1024;
     return cudaSuccess;
   }
-  auto go = [&](auto ac, auto nc) -> cudaError_t {
-    constexpr bool AFFINE = decltype(ac)::value, NODE = decltype(nc)::value;
+  auto go = [&](auto ac, auto nc, auto lrn) -> cudaError_t {
+    constexpr bool AFFINE = decltype(ac)::value, NODE = decltype(nc)::value, LEARNED = decltype(lrn)::value;
     const size_t smem = bytes(NODE);
     // a warp per tile of the boundary passes, more where a thread takes a node
     const int T = std::min(S::TMAX, 32 * std::max(4, 9 * p.epc * (NODE ? (S::Np + 31) / 32 : 1)));
-    cudaError_t err = raise_smem<flow2d_kernel<Real, n, AFFINE, NODE>>(smem);
+    cudaError_t err = raise_smem<flow2d_kernel<Real, n, AFFINE, NODE, LEARNED>>(smem);
     if (err != cudaSuccess) return err;
     StageMats<Real, n> m = make_stage_mats<Real, n>(h);
     FilterMats<Real, n> fm = make_filter_mats<Real, n>(h);
     Flow2DArgs<Real> a = p;
     CollideFix cf = make_collide_fix<SELBM_D2Q9>((double)p.omega, (double)p.dt);
-    void *args[] = {&a, &m, &fm, &cf};
-    return cudaLaunchCooperativeKernel((const void *)flow2d_kernel<Real, n, AFFINE, NODE>, dim3((p.E + p.epc - 1) / p.epc),
+    Learn2DArgs<Real> la = lc ? *lc : Learn2DArgs<Real>{};
+    void *args[] = {&a, &m, &fm, &cf, &la};
+    return cudaLaunchCooperativeKernel((const void *)flow2d_kernel<Real, n, AFFINE, NODE, LEARNED>, dim3((p.E + p.epc - 1) / p.epc),
                                        dim3(T), args, smem, s);
   };
-  if constexpr (S::F64) {
-    if (p.epc * 9 * S::Np <= kNodeTasks && bytes(true) <= (size_t)most - 1024) return affine ? go(std::true_type{}, std::true_type{}) : go(std::false_type{}, std::true_type{});
+  using Yes = std::true_type;
+  using No = std::false_type;
+  if constexpr (L2D) {
+    return affine ? go(Yes{}, No{}, Yes{}) : go(No{}, No{}, Yes{});
+  } else {
+    if constexpr (S::F64) {
+      if (p.epc * 9 * S::Np <= kNodeTasks && bytes(true) <= (size_t)most - 1024)
+        return affine ? go(Yes{}, Yes{}, No{}) : go(No{}, Yes{}, No{});
+    }
+    return affine ? go(Yes{}, No{}, No{}) : go(No{}, No{}, No{});
   }
-  return affine ? go(std::true_type{}, std::false_type{}) : go(std::false_type{}, std::false_type{});
 }
+
+// translation units: part 0 without the learned control (FP64: N <= 8), 1 FP64 above, 2 with it
+template <typename Real, int PART>
+cudaError_t flow2d_part(int N, bool affine, bool probe, const Flow2DArgs<Real> &p, const SplitHost &h, const Learn2DArgs<Real> *lc,
+                        bool *fits, cudaStream_t s);
 
 }  // namespace slb

@@ -4,6 +4,13 @@
 
 namespace slb {
 
+// a value and the number of its exchange: 8 bytes per 32 bits of the value, each written and read
+// as one access
+template <typename Real>
+struct Packet {
+  unsigned long long w[sizeof(Real) / 4];
+};
+
 template <typename Real>
 struct Flow2DArgs {
   int E, Gs, epc, nsteps;
@@ -30,8 +37,22 @@ struct Flow2DArgs {
   Real *f;                      // [9][Gs] state
 };
 
+// learned control of the resident step (see selbm_set_learned_filter)
+template <typename Real>
+struct Learn2DArgs {
+  const __nv_bfloat16 *W;       // network parameters
+  const Real *lo, *hi, *Vinv;   // [2n] training range; [n][n] nodal -> modal
+  int *flag, *n_fallback;
+  double *acc;                  // [2..4] mass, kinetic energy of the last pass, whether there was one
+  Real *sigma_out;              // [E][n]
+  Packet<double> *sums;         // [2][CTAs][2] packets: drift sums of a pass
+  double mass_bound, ke_bound;
+  int check_ke, pass;           // number of the first control pass of this launch
+};
+
 // probe: *fits = whether the SMs hold the mesh at p.epc elements a CTA; else launches p.nsteps steps
 template <typename Real>
-cudaError_t launch_flow2d(int N, bool affine, bool probe, const Flow2DArgs<Real> &p, const SplitHost &h, bool *fits, cudaStream_t s);
+cudaError_t launch_flow2d(int N, bool affine, bool probe, const Flow2DArgs<Real> &p, const SplitHost &h,
+                          const Learn2DArgs<Real> *lc, bool *fits, cudaStream_t s);
 
 }  // namespace slb

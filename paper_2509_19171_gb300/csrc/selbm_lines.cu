@@ -1,6 +1,6 @@
 // Dispatch of the any-order element kernels and of the resident 2D step to the translation units
 // of their orders.
-#include "selbm_flow2d.h"
+#include "selbm_flow2d.cuh"
 #include "selbm_lines.cuh"
 
 namespace slb {
@@ -25,13 +25,14 @@ cudaError_t launch_curved_geo(const Real *drdx, int E, int Np, LineVal<Real> *g,
   return cudaGetLastError();
 }
 
-template <typename Real, int PART>
-cudaError_t flow2d_part(int N, bool affine, bool probe, const Flow2DArgs<Real> &p, const SplitHost &h, bool *fits, cudaStream_t s);
-
 template <typename Real>
-cudaError_t launch_flow2d(int N, bool affine, bool probe, const Flow2DArgs<Real> &p, const SplitHost &h, bool *fits, cudaStream_t s) {
-  if (sizeof(Real) == 8 && N > 8) return flow2d_part<double, 1>(N, affine, probe, reinterpret_cast<const Flow2DArgs<double> &>(p), h, fits, s);
-  return flow2d_part<Real, 0>(N, affine, probe, p, h, fits, s);
+cudaError_t launch_flow2d(int N, bool affine, bool probe, const Flow2DArgs<Real> &p, const SplitHost &h, const Learn2DArgs<Real> *lc,
+                          bool *fits, cudaStream_t s) {
+  if (lc && N < 4) return cudaErrorInvalidValue;
+  if (lc) return flow2d_part<Real, 2>(N, affine, probe, p, h, lc, fits, s);
+  if constexpr (sizeof(Real) == 8)
+    if (N > 8) return flow2d_part<Real, 1>(N, affine, probe, p, h, lc, fits, s);
+  return flow2d_part<Real, 0>(N, affine, probe, p, h, lc, fits, s);
 }
 
 #define SLB_INST(Real)                                                                                                    \
@@ -40,7 +41,8 @@ cudaError_t launch_flow2d(int N, bool affine, bool probe, const Flow2DArgs<Real>
   template cudaError_t launch_lines_filter<Real>(int, int, const KParams<Real> &, const SplitHost &, const Real *, Real *, \
                                                  cudaStream_t);                                                          \
   template cudaError_t launch_curved_geo<Real>(const Real *, int, int, LineVal<Real> *, int *, cudaStream_t);             \
-  template cudaError_t launch_flow2d<Real>(int, bool, bool, const Flow2DArgs<Real> &, const SplitHost &, bool *, cudaStream_t);
+  template cudaError_t launch_flow2d<Real>(int, bool, bool, const Flow2DArgs<Real> &, const SplitHost &,              \
+                                             const Learn2DArgs<Real> *, bool *, cudaStream_t);
 SLB_INST(float)
 SLB_INST(double)
 

@@ -10,6 +10,7 @@ import pytest
 
 import workloads as W
 from oracle import gll
+from oracle import learned as Lr
 from oracle.selbm import OracleSELBM
 
 pytestmark = pytest.mark.gpu
@@ -109,3 +110,37 @@ def test_nonfinite_state(P):
     assert np.isnan(g).any() and np.isfinite(g).any()
     with pytest.raises(P.SelbmError):
         s.diagnostics()
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("N", [4, 7, 11, 14])
+def test_learned_control(P, N, prec):
+    """The learned control inside the resident step, one call per step and all steps in one call, then
+    the drift fallback (a negative mass bound trips at the second pass) and the transfer functions."""
+    mesh = channel(5, 4)
+    filt = {"shape": 0, "gamma": 0.1, "kc": float(N - 2)}
+    nin = 2 * (N + 1)
+    lo, hi = np.full(nin, -35.0), np.full(nin, 5.0)
+    params = np.float64(np.float32(Lr.init_params(nin, seed=11) * 1.5))
+    tol = 1e-10 if prec == 0 else 1e-6
+    o = OracleSELBM(mesh, "D2Q9", N, 1e-2, filt=filt)
+    f = f0 = rough_state(o, 0.02, 3)
+    one, many, drift = (P.SELBM(mesh, "D2Q9", N, 1e-2, filt=filt, precision=prec) for _ in range(3))
+    for s, bound in ((one, 1.0), (many, 1.0), (drift, -1.0)):
+        s.set_learned_filter(params, lo, hi, mass_bound=bound, ke_bound=0.0)
+        s.set_state(np.ascontiguousarray(o.to_local(f0)))
+    for k in range(4):
+        sig, _, _ = o.learned_sigma(o.stream(*o.collide(f)), params, lo, hi)
+        f = o.step_learned(f, params, lo, hi)
+        one.step(1)
+        assert rel(one.get_state(), o.to_local(f)) <= tol
+        assert np.abs(one.element_sigma() - sig).max() <= (1e-9 if prec == 0 else 1e-4)
+    assert one.learned_status()["fixed_element_steps"] == 0
+    many.step(4)
+    assert np.array_equal(many.get_state(), one.get_state())
+    g = o.step_learned(o.step_learned(f0, params, lo, hi), params, lo, hi)
+    g = o.step(o.step(g))
+    drift.step(4)
+    assert rel(drift.get_state(), o.to_local(g)) <= tol
+    st = drift.learned_status()
+    assert st["fallback_flag"] == 1 and st["fixed_element_steps"] == mesh.nelem
