@@ -53,7 +53,7 @@ struct selbm {
   // any-order element kernels of the split step: hexahedra where the fused kernels are not
   // compiled, and every FP64 order
   bool use_lines = false;
-  void *d_geo = nullptr;         // planar metrics of curved elements (any-order kernels)
+  void *d_geo = nullptr, *d_w3 = nullptr;   // metrics of the any-order kernels (CurvedGeo)
   int *d_gexp = nullptr;
   bool split_form() const { return use_split || use_lines; }
   bool lines_step() const { return use_lines && !(use_split && prec == SELBM_FP32DEV); }
@@ -277,6 +277,16 @@ cudaError_t upload_real(selbm *h) {
     }
     if ((e = upload(&p, cast_vec<Real>(em)))) return e; h->d_el_drdx = p; h->allocs.push_back(p);
     if ((e = upload(&p, cast_vec<Real>(S.el_J)))) return e; h->d_el_J = p; h->allocs.push_back(p);
+    if constexpr (sizeof(Real) == 8) {
+      if (h->lines_step()) {
+        if ((e = alloc(&h->d_geo, (size_t)S.E * h->Q * 3 * sizeof(long long)))) return e;
+        if ((e = alloc((void **)&h->d_gexp, (size_t)S.E * h->Q * sizeof(int)))) return e;
+        if ((e = launch_affine_geo(h->lat, (const double *)h->d_el_drdx, S.E, h->dt, (long long *)h->d_geo, h->d_gexp, h->stream))) return e;
+        std::vector<double> w3(S.Np);
+        for (int i = 0; i < S.Np; ++i) w3[i] = S.gll.w[i % S.n1] * S.gll.w[i / S.n1 % S.n1] * S.gll.w[i / (S.n1 * S.n1)];
+        if ((e = upload(&p, w3))) return e; h->d_w3 = p; h->allocs.push_back(p);
+      }
+    }
   } else {
     if ((e = upload(&p, cast_vec<Real>(S.drdx)))) return e; h->d_drdx = p; h->allocs.push_back(p);
     if ((e = upload(&p, cast_vec<Real>(S.wJ)))) return e; h->d_wJ = p; h->allocs.push_back(p);
@@ -416,7 +426,7 @@ template <typename Real>
 cudaError_t launch_split_stage(selbm *h, const KParams<Real> &p) {
   const SplitHost sh = split_host(h);
   if (h->lines_step()) {
-    const CurvedGeo<Real> cg{(const LineVal<Real> *)h->d_geo, h->d_gexp};
+    const CurvedGeo<Real> cg{(const LineVal<Real> *)h->d_geo, h->d_gexp, (const Real *)h->d_w3};
     return launch_lines_stage<Real>(h->lat, h->S.N, h->S.affine, p, sh, cg, h->stream);
   }
   cudaError_t err = cudaErrorInvalidValue;

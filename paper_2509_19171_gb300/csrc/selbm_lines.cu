@@ -25,6 +25,30 @@ cudaError_t launch_curved_geo(const Real *drdx, int E, int Np, LineVal<Real> *g,
   return cudaGetLastError();
 }
 
+// affine elements, FP64: -dt sum_k e_k dr_l/dx_k in fixed point, c [E][Q][3] times 2^cexp[E][Q]
+__global__ static void affine_geo_kernel(const double *el_drdx, int E, const LatticeRT lt, double dt, long long *c, int *cexp) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= E * lt.Q) return;
+  const int e = t / lt.Q, a = t - e * lt.Q;
+  double v[3];
+  int ex = 1;
+  for (int l = 0; l < 3; ++l) {
+    double s = 0;
+    for (int k = 0; k < 3; ++k)
+      s += (double)((int)((lt.pos[k] >> a) & 1u) - (int)((lt.neg[k] >> a) & 1u)) * el_drdx[((size_t)e * 3 + l) * 3 + k];
+    v[l] = -dt * s;
+    ex = max(ex, exp_of(v[l]));
+  }
+  cexp[t] = 1082 - ex;                                   // magnitudes below 2^60
+  for (int l = 0; l < 3; ++l) c[(size_t)t * 3 + l] = __double2ll_rn(scalbn(v[l], 1082 - ex));
+}
+
+cudaError_t launch_affine_geo(int lat, const double *el_drdx, int E, double dt, long long *c, int *cexp, cudaStream_t s) {
+  const LatticeRT lt = lat == SELBM_D3Q19 ? lattice_rt<SELBM_D3Q19>() : lattice_rt<SELBM_D3Q27>();
+  affine_geo_kernel<<<(E * lt.Q + 255) / 256, 256, 0, s>>>(el_drdx, E, lt, dt, c, cexp);
+  return cudaGetLastError();
+}
+
 template <typename Real>
 cudaError_t launch_flow2d(int N, bool affine, bool probe, const Flow2DArgs<Real> &p, const SplitHost &h, const Learn2DArgs<Real> *lc,
                           bool *fits, cudaStream_t s) {

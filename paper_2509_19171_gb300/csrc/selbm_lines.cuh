@@ -77,6 +77,7 @@ struct StageMats {
   Real D[sizeof(Real) == 8 ? n * n : 1];    // FP64 fallback of a tile that holds infinities or NaN
   Real w[n];
   int cb;                                    // fixed point: coefficients times 2^cb
+  LineCoef<Real> B;                          // stage weight; fixed point: times 2^62
 };
 // filter v + sum_k g_k U_k (W_k . v) over the modes k >= 2: mode k has the parity of k, so W_k
 // reads the even or the odd half of the line and U_k adds to that half (end rows are zero)
@@ -366,10 +367,10 @@ template <typename Real, int n, bool AFFINE>
 constexpr size_t lines_stage_smem(int pb, int wall_max) {
   using S = LineShape<Real, n>;
   size_t b = (size_t)(2 * pb + (AFFINE ? 0 : 3)) * S::PS * sizeof(LineVal<Real>);   // tile, sums, metrics of one axis
-  b += (size_t)pb * 3 * (sizeof(LineVal<Real>) + sizeof(Real));                     // coefficients of the axes
+  b += (size_t)pb * 3 * sizeof(LineVal<Real>);                                      // coefficients of the axes
   b += (size_t)(2 * pb + (size_t)pb * wall_max) * sizeof(Real);                     // force, wall terms
   if (S::F64 && AFFINE) b += (size_t)S::Np * sizeof(double);                        // quadrature weights
-  return b + (size_t)2 * pb * sizeof(int) + 16;
+  return b + (size_t)3 * pb * sizeof(int) + 16;
 }
 
 template <typename Real, int n, bool AFFINE>
@@ -386,12 +387,12 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
   Val *acc = tile + pb * PS;                           // [pb][PS] sums of the passes
   Val *sg = acc + pb * PS;                             // curved: [3][PS] dr_l/dx_k of the axis in hand
   Val *cf = sg + (AFFINE ? 0 : 3 * PS);                // [pb][3] affine: -B dt sum_k e_k dr_l/dx_k
-  Real *cd = reinterpret_cast<Real *>(cf + pb * 3);    // [pb][3] the same as a Real
-  Real *fc = cd + pb * 3;                              // [2][pb] B dt F*_a / rho; B dt 3 t_a
+  Real *fc = reinterpret_cast<Real *>(cf + pb * 3);    // [2][pb] B dt F*_a / rho; B dt 3 t_a
   Real *wbuf = fc + 2 * pb;                            // [wall nodes][pb]
   Real *sw = wbuf + (size_t)pb * p.wall_max;           // FP64, affine: [Np] J w w w
   int *em = reinterpret_cast<int *>(sw + (F64 && AFFINE ? Np : 0));   // [pb] exponent of the tile
   int *ge = em + pb;                                   // [pb] exponent of the coefficients
+  int *axes = ge + pb;                                 // [pb] bit l: the axis has a coefficient
   const int e = blockIdx.x / ng, a0 = (blockIdx.x - e * ng) * pb;
   const int na = min(pb, lt.Q - a0);
   const int tid = threadIdx.x;
@@ -401,27 +402,33 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
   auto sgn = [&](int k, int a) -> int { return (int)((lt.pos[k] >> a) & 1u) - (int)((lt.neg[k] >> a) & 1u); };
 
   if (F64 && tid < pb) em[tid] = kMinExp;
-  if (AFFINE && tid < na) {
-    Real c[3];
+  if (tid < na) {
+    int on = 0;
+    if constexpr (AFFINE && F64) {
+      // -dt sum_k e_k dr_l/dx_k in fixed point from the table, times B
+      const size_t row = (size_t)e * lt.Q + a0 + tid;
+      ge[tid] = cg.gexp[row];
 #pragma unroll
-    for (int l = 0; l < 3; ++l) {
-      Real s = 0;
+      for (int l = 0; l < 3; ++l) {
+        const long long c = cg.g[row * 3 + l];
+        Fix128 t{0, 1ll << 29};
+        fix_mac(t, m.B, limbs(c));
+        cf[tid * 3 + l] = fix_top<2>(t);
+        on |= (c != 0) << l;
+      }
+    } else if constexpr (AFFINE) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) s += Real(sgn(k, a0 + tid)) * p.el_drdx[((size_t)e * 3 + l) * 3 + k];
-      c[l] = -Bdt * s;
-      cd[tid * 3 + l] = c[l];
-    }
-    if constexpr (F64) {
-      int ex = 1;
+      for (int l = 0; l < 3; ++l) {
+        Real c = 0;
 #pragma unroll
-      for (int l = 0; l < 3; ++l) ex = max(ex, exp_of(c[l]));
-      ge[tid] = 1082 - ex;                             // coefficients below 2^61 in magnitude
-#pragma unroll
-      for (int l = 0; l < 3; ++l) cf[tid * 3 + l] = __double2ll_rn(scalbn(c[l], 1082 - ex));
+        for (int k = 0; k < 3; ++k) c += Real(sgn(k, a0 + tid)) * p.el_drdx[((size_t)e * 3 + l) * 3 + k];
+        cf[tid * 3 + l] = -Bdt * c;
+        on |= (c != Real(0)) << l;
+      }
     } else {
-#pragma unroll
-      for (int l = 0; l < 3; ++l) cf[tid * 3 + l] = c[l];
+      on = ((lt.pos[0] | lt.neg[0] | lt.pos[1] | lt.neg[1] | lt.pos[2] | lt.neg[2]) >> (a0 + tid)) & 1u ? 7 : 0;
     }
+    axes[tid] = on;
   }
   if (p.has_force && tid < na) {
     Real g3 = 0;
@@ -433,7 +440,7 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
   }
   if constexpr (F64 && AFFINE) {
     const double J = p.el_J[e];
-    for (int i = tid; i < Np; i += T) sw[i] = J * m.w[i % n] * m.w[(i / n) % n] * m.w[i / (n * n)];
+    for (int i = tid; i < Np; i += T) sw[i] = J * cg.w3[i];
   }
   if (F64) __syncthreads();                            // em
   gather_lines<Real, n, SHIFT>(tile, em, p.fin + (size_t)a0 * G, G, l2g, na, tid);
@@ -496,7 +503,7 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
     if constexpr (F64) {
       double c = 0;
       if (AFFINE) {
-        c = cd[pl * 3 + ax];
+        c = from_fixed(cf[pl * 3 + ax], -ge[pl]);
         if (c == 0) return 0.0;
       } else {
         const int off = base + j * st;
@@ -507,16 +514,11 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
       return c * slow_deriv<n>(m.D, tile + pl * PS + base, st, j);
     } else return 0.0;
   };
-  const auto active = [&](int ax, int pl) -> bool {
-    if (AFFINE) return cd[pl * 3 + ax] != Real(0);
-    return ((lt.pos[0] | lt.neg[0] | lt.pos[1] | lt.neg[1] | lt.pos[2] | lt.neg[2]) >> (a0 + pl)) & 1u;
-  };
-
   // ---- r-pass: sums start; s-pass: sums grow
   stage_metrics(0);
   for (int t = tid; t < na * NL; t += T) {
     const int pl = t / NL, base = line_base<Real, n, 0>(t - pl * NL);
-    if (!active(0, pl)) continue;
+    if (!(axes[pl] & 1)) continue;
     Val *dst = acc + pl * PS + base;
     if (F64 && em[pl] == 2047) {
       if constexpr (F64)
@@ -534,10 +536,11 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
   if (AFFINE) __syncthreads();
   for (int t = tid; t < na * NL; t += T) {
     const int pl = t / NL, base = line_base<Real, n, 1>(t - pl * NL);
-    if (!active(1, pl)) continue;
+    const int on = axes[pl];
+    if (!(on & 2)) continue;
     constexpr int ST = line_stride<Real, n, 1>();
     Val *dst = acc + pl * PS + base;
-    const bool more = active(0, pl);
+    const bool more = on & 1;
     if (F64 && em[pl] == 2047) {
       if constexpr (F64)
         for (int j = 0; j < n; ++j)
@@ -585,34 +588,30 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
     const int pl = t / NL, L = t - pl * NL, a = a0 + pl;
     const int base = line_base<Real, n, 2>(L), i0 = L % n, i1 = L / n;
     constexpr int ST = line_stride<Real, n, 2>();
-    const bool more = active(0, pl) || active(1, pl);
+    const int on = axes[pl];
+    const bool more = on & 3;
     const bool slow = F64 && em[pl] == 2047;
     const bool lin = i0 > 0 && i0 < n - 1 && i1 > 0 && i1 < n - 1;
+    // interior lines read f^0 (and f^{s-1}) and write f^s, edge lines write their shares: node k of the
+    // middle planes is `step` values after node k - 1 in either, so one code path serves both
     const size_t gi = (size_t)a * G + (size_t)e * S::NI + (lin ? (i0 - 1) + S::M * (i1 - 1) : 0);   // node k: + MM (k - 1)
     Real f0v[S::M], fv[S::M];
-    if (lin) {
 #pragma unroll
-      for (int k = 0; k < S::M; ++k) {
-        f0v[k] = use_f0 ? __ldg(p.f0 + gi + (size_t)S::MM * k) : Real(0);
-        if (F64) fv[k] = __ldg(p.fin + gi + (size_t)S::MM * k);
-      }
+    for (int k = 0; k < S::M; ++k) {
+      f0v[k] = lin && use_f0 ? __ldg(p.f0 + gi + (size_t)(S::MM * k)) : Real(0);
+      if constexpr (F64) fv[k] = lin ? __ldg(p.fin + gi + (size_t)(S::MM * k)) : Real(0);
+      else fv[k] = lin ? tile[pl * PS + base + (k + 1) * ST] : Real(0);
     }
     Val s[n];
     const Val *ac = acc + pl * PS + base;
     if (!slow) {
 #pragma unroll
       for (int j = 0; j < n; ++j) s[j] = more ? ac[j * ST] : Val(0);
-      if (active(2, pl)) line_terms(std::integral_constant<int, 2>{}, pl, base, s);
+      if (on & 4) line_terms(std::integral_constant<int, 2>{}, pl, base, s);
     } else if constexpr (F64) {
 #pragma unroll
       for (int j = 0; j < n; ++j)
-        s[j] = __double_as_longlong((more ? __longlong_as_double(ac[j * ST]) : 0.0) + (active(2, pl) ? slow_term(2, pl, base, ST, j) : 0.0));
-    }
-    if constexpr (!F64) {
-      if (lin) {
-#pragma unroll
-        for (int k = 0; k < S::M; ++k) fv[k] = tile[pl * PS + base + (k + 1) * ST];
-      }
+        s[j] = __double_as_longlong((more ? __longlong_as_double(ac[j * ST]) : 0.0) + (on & 4 ? slow_term(2, pl, base, ST, j) : 0.0));
     }
     // value of a sum: curved elements carry -B dt here
     int ex = 0;
@@ -625,36 +624,56 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
       else return x;
     };
     const Real scale = AFFINE ? Real(1) : -Bdt;
-    const Real w01 = AFFINE ? (F64 ? Real(0) : p.el_J[e] * m.w[i0] * m.w[i1]) : Real(0);
+    const Real w01 = AFFINE && !F64 ? p.el_J[e] * m.w[i0] * m.w[i1] : Real(0);
+    auto share_weight = [&](int k) -> Real {
+      if constexpr (!AFFINE) return scale * p.wJ[(size_t)e * Np + L + k * NL];
+      else if constexpr (F64) return sw[L + k * NL];
+      else return w01 * m.w[k];
+    };
     // boundary slots: nodes before this one, less the interior ones among them
     const int before = min(max(i1 - 1, 0), S::M) * S::M + (i1 >= 1 && i1 <= S::M ? min(max(i0 - 1, 0), S::M) : 0);
     Real *tp = p.T + (size_t)a * EN + (size_t)e * S::NB + L;
-    Real rg[3] = {0, 0, 0};
-    const Real famp = p.fS ? *p.famp : Real(0);
+    tp[0] = share_weight(0) * value(s[0]);
+    tp[(n - 1) * NL - S::NI] = share_weight(n - 1) * value(s[n - 1]);
+    Real *dst = lin ? p.fout + gi : tp + NL - before;
+    const int step = lin ? S::MM : NL - S::MM;
+    const Real Bl = lin ? p.B : Real(0), Al = lin && use_f0 ? p.A : Real(0);
+    if (!p.has_force) {
 #pragma unroll
-    for (int k = 0; k < n; ++k) {
-      const Real x = value(s[k]);
-      if (k > 0 && k < n - 1 && lin) {
-        Real out = AFFINE ? p.B * fv[k - 1] + x : scale * x + p.B * fv[k - 1];
-        if (use_f0) out += p.A * f0v[k - 1];
-        if (p.has_force) {
+      for (int k = 1; k < n - 1; ++k) {
+        const Real x = value(s[k]);
+        Real c = scale;
+        if (!lin) c = share_weight(k);
+        Real out = (AFFINE && F64 && lin) ? Bl * fv[k - 1] + x : Bl * fv[k - 1] + c * x;
+        if (!F64 || (lin && use_f0)) out += Al * f0v[k - 1];
+        *dst = out;
+        dst += step;
+      }
+    } else {
+      const Real famp = p.fS ? *p.famp : Real(0);
+#pragma unroll 1
+      for (int k = 1; k < n - 1; ++k) {
+        Real fk = 0, f0k = 0;
+        Val sk = 0;
+#pragma unroll
+        for (int q = 1; q < n - 1; ++q)
+          if (q == k) { sk = s[q]; fk = fv[q - 1]; f0k = f0v[q - 1]; }
+        const Real x = value(sk);
+        if (lin) {
+          Real out = Bl * fk + scale * x + Al * f0k;
           const size_t g = (size_t)e * S::NI + (i0 - 1) + S::M * ((i1 - 1) + S::M * (k - 1));
           Real fa = fc[pl];
           if (p.fS) {
+            Real es = 0;
 #pragma unroll
-            for (int c = 0; c < 3; ++c) rg[c] = famp * p.fS[(size_t)c * p.G + g];
-            fa += fc[pb + pl] * (Real(sgn(0, a)) * rg[0] + Real(sgn(1, a)) * rg[1] + Real(sgn(2, a)) * rg[2]);
+            for (int c = 0; c < 3; ++c) es += Real(sgn(c, a)) * p.fS[(size_t)c * p.G + g];
+            fa += fc[pb + pl] * famp * es;
           }
-          out += fa * p.rho[g];
+          *dst = out + fa * p.rho[g];
+        } else {
+          *dst = share_weight(k) * x;
         }
-        p.fout[gi + (size_t)S::MM * (k - 1)] = out;
-      } else {
-        const int full = k == 0 ? 0 : (k == n - 1 ? S::NI : (k - 1) * S::MM);   // interior nodes of lower planes
-        const int slot = k * NL - full - (k > 0 && k < n - 1 ? before : 0);
-        Real wq;
-        if (AFFINE) wq = F64 ? sw[L + k * NL] : w01 * m.w[k];
-        else wq = scale * p.wJ[(size_t)e * Np + L + k * NL];
-        tp[slot] = wq * x;
+        dst += step;
       }
     }
   }
@@ -747,37 +766,36 @@ lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Re
   };
   pass(std::integral_constant<int, 0>{});
   pass(std::integral_constant<int, 1>{});
+  pass(std::integral_constant<int, 2>{});
+  // one node per thread: its destination is looked up once for the group
   const size_t EN = (size_t)p.E * S::NB;
-  for (int t = tid; t < na * NL; t += T) {
-    const int pl = t / NL, L = t - pl * NL, a = a0 + pl;
-    const int base = line_base<Real, n, 2>(L), i0 = L % n, i1 = L / n;
-    constexpr int ST = line_stride<Real, n, 2>();
-    const Val *row = tile + pl * PS + base;
-    Val v[n];
-#pragma unroll
-    for (int k = 0; k < n; ++k) v[k] = row[k * ST];
-    filter_line(pl, v);
-    const bool lin = i0 > 0 && i0 < n - 1 && i1 > 0 && i1 < n - 1;
-    const size_t gi = (size_t)a * G + (size_t)e * S::NI + (lin ? (i0 - 1) + S::M * (i1 - 1) : 0);
-    const int before = min(max(i1 - 1, 0), S::M) * S::M + (i1 >= 1 && i1 <= S::M ? min(max(i0 - 1, 0), S::M) : 0);
-    const bool slow = F64 && em[pl] == 2047;
-    auto value = [&](Val x) -> Real {
-      if constexpr (F64) return slow ? __longlong_as_double(x) : from_fixed(x, em[pl] - (1023 + 52 + kFilterShift));
-      else return x;
+#pragma unroll 1
+  for (int i = tid; i < Np; i += T) {
+    const Val *v = tile + tile_offset<Real, n>(i);
+    auto value = [&](int pl) -> Real {
+      if constexpr (F64) {
+        const int ex = em[pl];
+        return ex == 2047 ? __longlong_as_double(v[pl * PS]) : from_fixed(v[pl * PS], ex - (1023 + 52 + kFilterShift));
+      } else return v[pl * PS];
     };
-#pragma unroll
-    for (int k = 0; k < n; ++k) {
-      const int i = L + k * NL;
-      if (k > 0 && k < n - 1 && lin) {
-        out[gi + (size_t)S::MM * (k - 1)] = value(v[k]);
-      } else if (LEARNED) {
-        const int full = k == 0 ? 0 : (k == n - 1 ? S::NI : (k - 1) * S::MM);
-        const int slot = i - full - (k > 0 && k < n - 1 ? before : 0);
-        const Real wq = p.wJ ? p.wJ[(size_t)e * Np + i] : p.el_J[e] * m.w[i0] * m.w[i1] * m.w[k];
-        p.T[(size_t)a * EN + (size_t)e * S::NB + slot] = wq * value(v[k]);
-      } else if (p.owner[(size_t)e * Np + i]) {
-        out[(size_t)a * G + l2g[i]] = value(v[k]);
-      }
+    Real w = 1;
+    Real *dst;
+    size_t stride = G;
+    if (LEARNED) {
+      const int b = p.bslot[i];
+      if (b >= 0) {
+        w = p.wJ ? p.wJ[(size_t)e * Np + i] : p.el_J[e] * m.w[i % n] * m.w[(i / n) % n] * m.w[i / (n * n)];
+        dst = p.T + (size_t)a0 * EN + (size_t)e * S::NB + b;
+        stride = EN;
+      } else dst = out + (size_t)a0 * G + l2g[i];
+    } else {
+      if (!p.owner[(size_t)e * Np + i]) continue;
+      dst = out + (size_t)a0 * G + l2g[i];
+    }
+#pragma unroll 4
+    for (int pl = 0; pl < na; ++pl) {
+      *dst = LEARNED ? w * value(pl) : value(pl);
+      dst += stride;
     }
   }
 }
@@ -841,7 +859,9 @@ cudaError_t launch_lines_stage_t(bool affine, const KParams<Real> &p, const Spli
                                  const CurvedGeo<Real> &cg, cudaStream_t s) {
   int pb, ng;
   line_groups<Real, n>(lt.Q, &pb, &ng);
-  const StageMats<Real, n> m = make_stage_mats<Real, n>(h);
+  StageMats<Real, n> m = make_stage_mats<Real, n>(h);
+  if constexpr (sizeof(Real) == 8) m.B = fix_coef(p.B, 62);
+  else m.B = p.B;
   auto go = [&](auto ac) -> cudaError_t {
     constexpr bool AFFINE = decltype(ac)::value;
     const size_t smem = lines_stage_smem<Real, n, AFFINE>(pb, p.wall_max);

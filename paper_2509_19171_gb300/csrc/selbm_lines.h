@@ -23,12 +23,14 @@ struct LatticeRT {
   }
 };
 
-// planar metrics of curved elements: dr_l/dx_k [E][9][Np] (component 3 l + k); FP64: fixed point,
-// times 2^gexp[e]
+// metrics of the stage kernel.  Curved elements: dr_l/dx_k [E][9][Np] (component 3 l + k); FP64: fixed
+// point, times 2^gexp[e].  Affine elements, FP64: -dt sum_k e_k dr_l/dx_k [E][Q][3] in fixed point,
+// times 2^gexp[e Q + a], and the quadrature weights w w w [Np].
 template <typename Real>
 struct CurvedGeo {
   const LineVal<Real> *g;
   const int *gexp;
+  const Real *w3;
 };
 
 // orders whose element tile fits the step's other kernels too (real_size 4 or 8)
@@ -46,5 +48,8 @@ cudaError_t launch_lines_filter(int lat, int N, const KParams<Real> &p, const Sp
 // planar metrics from drdx [E][Np][9]
 template <typename Real>
 cudaError_t launch_curved_geo(const Real *drdx, int E, int Np, LineVal<Real> *g, int *gexp, cudaStream_t s);
+
+// the affine FP64 tables from el_drdx [E][3][3]
+cudaError_t launch_affine_geo(int lat, const double *el_drdx, int E, double dt, long long *c, int *cexp, cudaStream_t s);
 
 }  // namespace slb
