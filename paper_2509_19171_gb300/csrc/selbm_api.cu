@@ -53,7 +53,7 @@ struct selbm {
   // any-order element kernels of the split step: hexahedra where the fused kernels are not
   // compiled, and every FP64 order
   bool use_lines = false;
-  void *d_geo = nullptr, *d_w3 = nullptr;   // metrics of the any-order kernels (CurvedGeo)
+  void *d_geo = nullptr, *d_w3 = nullptr;   // metrics of the split-form kernels (CurvedGeo)
   int *d_gexp = nullptr;
   bool split_form() const { return use_split || use_lines; }
   bool lines_step() const { return use_lines && !(use_split && prec == SELBM_FP32DEV); }
@@ -290,7 +290,7 @@ cudaError_t upload_real(selbm *h) {
   } else {
     if ((e = upload(&p, cast_vec<Real>(S.drdx)))) return e; h->d_drdx = p; h->allocs.push_back(p);
     if ((e = upload(&p, cast_vec<Real>(S.wJ)))) return e; h->d_wJ = p; h->allocs.push_back(p);
-    if (h->lines_step()) {
+    if (h->split_form()) {
       if ((e = alloc(&h->d_geo, (size_t)S.E * S.Np * 9 * sizeof(LineVal<Real>)))) return e;
       if ((e = alloc((void **)&h->d_gexp, (size_t)S.E * sizeof(int)))) return e;
       if ((e = launch_curved_geo<Real>((const Real *)h->d_drdx, S.E, S.Np, (LineVal<Real> *)h->d_geo, h->d_gexp, h->stream))) return e;
@@ -431,8 +431,10 @@ cudaError_t launch_split_stage(selbm *h, const KParams<Real> &p) {
   }
   cudaError_t err = cudaErrorInvalidValue;
   if constexpr (std::is_same<Real, float>::value) {
-    if (h->lat == SELBM_D3Q19) split_stage_d3q19<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
-    else if (h->lat == SELBM_D3Q27) split_stage_d3q27<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
+    KParams<Real> q = p;
+    q.drdx = (const Real *)h->d_geo;        // metrics by component
+    if (h->lat == SELBM_D3Q19) split_stage_d3q19<Real>(h->S.N, h->S.affine, q, sh, h->stream, &err);
+    else if (h->lat == SELBM_D3Q27) split_stage_d3q27<Real>(h->S.N, h->S.affine, q, sh, h->stream, &err);
   }
   return err;
 }
