@@ -421,7 +421,7 @@ __global__ void __launch_bounds__(256) node_features_kernel(const KParams<Real> 
     q[Gs + g] = sqrt(uu);
     if (acc) {
       pm += mass[g] * (double)rho;
-      pk += 0.5 * (double)p.rho0 * mass[g] * (double)uu;
+      pk += mass[g] * (double)uu;
     }
   }
   if (!acc) return;
@@ -434,7 +434,7 @@ __global__ void __launch_bounds__(256) node_features_kernel(const KParams<Real> 
     double sm = 0.0, sk = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) { sm += red[w][0]; sk += red[w][1]; }
     atomicAdd(&acc[0], sm);
-    atomicAdd(&acc[1], sk);
+    atomicAdd(&acc[1], 0.5 * (double)p.rho0 * sk);
   }
 }
 
@@ -445,10 +445,12 @@ constexpr int kCtlWarps = 4;
 template <typename Real, int n>
 __global__ void __launch_bounds__(32 * kCtlWarps, sizeof(Real) == 4 ? 4 : 2)
 element_features_kernel(const KParams<Real> p, const LearnedIn<Real, n> c, const Real *q, Real *X) {
-  constexpr int Np = n * n * n, NL = n * n, nin = 2 * n, WPB = kCtlWarps;
+  // r-lines of odd length in shared memory: lanes along r-lines of n = 8 hit four banks otherwise
+  constexpr int Np = n * n * n, NL = n * n, nin = 2 * n, WPB = kCtlWarps, LS = n | 1, PLN = LS * n;
   static_assert(nin <= 32, "one lane per feature");
-  __shared__ __align__(16) Real sq[WPB][2][Np];
-  __shared__ Real sVi[n * n];
+  __shared__ __align__(16) Real sq[WPB][2][PLN * n];
+  __shared__ __align__(16) Real sVi[n * n];
+  auto at = [](int i) { return i % n + LS * (i / n); };
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int k = threadIdx.x; k < n * n; k += blockDim.x) sVi[k] = c.Vinv[k];
   __syncthreads();                                   // the only block-wide barrier
@@ -472,8 +474,8 @@ element_features_kernel(const KParams<Real> p, const LearnedIn<Real, n> c, const
       for (int r = 0; r < HALF; ++r) {
         const int i = lane + 32 * (r0 + r);
         if (r0 + r < NPL && i < Np) {
-          f0[i] = q[gi[r]];
-          f1[i] = q[Gs + gi[r]];
+          f0[at(i)] = q[gi[r]];
+          f1[at(i)] = q[Gs + gi[r]];
         }
       }
     }
@@ -482,11 +484,11 @@ element_features_kernel(const KParams<Real> p, const LearnedIn<Real, n> c, const
   // modal coefficients of both fields: V^-1 along r, s and t (node order r fastest)
 #pragma unroll 1
   for (int axis = 0; axis < 3; ++axis) {
-    const int stride = axis == 0 ? 1 : (axis == 1 ? n : NL);
+    const int stride = axis == 0 ? 1 : (axis == 1 ? LS : PLN);
 #pragma unroll 1
     for (int t = lane; t < 2 * NL; t += 32) {
       const int f = t / NL, L = t - f * NL;
-      const int base = axis == 0 ? L * n : (axis == 1 ? (L % n) + NL * (L / n) : L);
+      const int base = axis == 0 ? L * LS : (axis == 1 ? (L % n) + PLN * (L / n) : at(L));
       Real *row = sq[wid][f] + base;
       Real v[n];
 #pragma unroll
@@ -504,7 +506,7 @@ element_features_kernel(const KParams<Real> p, const LearnedIn<Real, n> c, const
   for (int i = lane; i < Np; i += 32) {
     const int i0 = i % n, i1 = (i / n) % n, i2 = i / NL;
     const int sh = max(i0, max(i1, i2));
-    const Real q0 = f0[i], q1 = f1[i];
+    const Real q0 = f0[at(i)], q1 = f1[at(i)];
 #pragma unroll
     for (int k = 0; k < n; ++k)
       if (k == sh) { en[0][k] += q0 * q0; en[1][k] += q1 * q1; }
@@ -524,25 +526,28 @@ element_features_kernel(const KParams<Real> p, const LearnedIn<Real, n> c, const
   }
 }
 
-// The network over kMlpEB elements per CTA (weights staged once in shared memory, every thread
-// computing independent outputs): scaled inputs s = 2 (x - lo)/(hi - lo) - 1, h1 = tanh(W1 s + b1),
-// h2 = tanh(W2 h1 + b2), o = W3 h2 + b3 (BF16 weights, Real arithmetic), then the element's
-// transfer function: the paper's quadratic filter at (gamma, kc) = (0.5 sigmoid(o0),
-// 2 + (N-3) sigmoid(o1)), or the fixed filter when a feature leaves [lo, hi] or the drift
-// fallback is on.  sigma_out [E][n].
+// The network over 16 elements per CTA (weights staged once in shared memory): scaled inputs
+// s = 2 (x - lo)/(hi - lo) - 1, h1 = tanh(W1 s + b1), h2 = tanh(W2 h1 + b2), o = W3 h2 + b3 (BF16
+// weights, Real arithmetic), then the element's transfer function: the paper's quadratic filter at
+// (gamma, kc) = (0.5 sigmoid(o0), 2 + (N-3) sigmoid(o1)), or the fixed filter when a feature leaves
+// [lo, hi] or the drift fallback is on.  sigma_out [E][n].  Shared-memory loads bound it: weights
+// are stored with the output fastest (an output-major W1 puts 16 lanes in one bank) and a thread
+// forms one output of four elements, so a weight is loaded once for four products.
 constexpr int kMlpThreads = 256;
 template <typename Real>
 constexpr int mlp_elements_per_cta() { return 16; }
 template <typename Real, int n>
 __global__ void __launch_bounds__(kMlpThreads) mlp_sigma_kernel(const int E, const LearnedIn<Real, n> c, const Real *X) {
   constexpr int H = kHidden, nin = 2 * n, EB = mlp_elements_per_cta<Real>(), T = kMlpThreads;
-  __shared__ float w1[H][nin], w2[H][H + 1], w3[2][H], b1[H], b2[H], b3[2];
-  __shared__ Real sx[EB][nin], h1[EB][H], h2[EB][H], so[EB][2];
+  static_assert(EB * H == 4 * T, "four elements per thread");
+  __shared__ float w1[nin][H], w2[H][H + 1], w3[2][H], b1[H], b2[H], b3[2];
+  __shared__ __align__(16) Real sx[nin][EB], h1[H][EB];
+  __shared__ Real h2[EB][H + 1], so[EB][2];
   __shared__ int inr[EB];
   const int tid = threadIdx.x, e0 = blockIdx.x * EB;
   const __nv_bfloat16 *W1 = c.W, *B1 = W1 + H * nin, *W2 = B1 + H, *B2 = W2 + H * H, *W3 = B2 + H, *B3 = W3 + 2 * H;
-  for (int k = tid; k < H * nin; k += T) w1[k / nin][k % nin] = __bfloat162float(W1[k]);
-  for (int k = tid; k < H * H; k += T) w2[k / H][k % H] = __bfloat162float(W2[k]);
+  for (int k = tid; k < H * nin; k += T) w1[k % nin][k / nin] = __bfloat162float(W1[k]);
+  for (int k = tid; k < H * H; k += T) w2[k % H][k / H] = __bfloat162float(W2[k]);
   for (int k = tid; k < 2 * H; k += T) w3[k / H][k % H] = __bfloat162float(W3[k]);
   for (int k = tid; k < H; k += T) { b1[k] = __bfloat162float(B1[k]); b2[k] = __bfloat162float(B2[k]); }
   if (tid < 2) b3[tid] = __bfloat162float(B3[tid]);
@@ -556,23 +561,32 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_sigma_kernel(const int E, con
       if (!(x >= lo && x <= hi)) atomicAnd(&inr[el], 0);
       sv = Real(2) * (x - lo) / (hi - lo) - Real(1);
     }
-    sx[el][i] = sv;
+    sx[i][el] = sv;
   }
   __syncthreads();
-  for (int k = tid; k < EB * H; k += T) {
-    const int el = k / H, o = k - el * H;
-    Real z = (Real)b1[o];
+  const int o4 = tid % H, e4 = 4 * (tid / H);             // output o4 of elements e4 .. e4 + 3
+  {
+    Real z[4];
 #pragma unroll
-    for (int i = 0; i < nin; ++i) z += (Real)w1[o][i] * sx[el][i];
-    h1[el][o] = tanh(z);
+    for (int q = 0; q < 4; ++q) z[q] = (Real)b1[o4];
+#pragma unroll
+    for (int i = 0; i < nin; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) z[q] += (Real)w1[i][o4] * sx[i][e4 + q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) h1[o4][e4 + q] = tanh(z[q]);
   }
   __syncthreads();
-  for (int k = tid; k < EB * H; k += T) {
-    const int el = k / H, o = k - el * H;
-    Real z = (Real)b2[o];
+  {
+    Real z[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) z[q] = (Real)b2[o4];
 #pragma unroll 8
-    for (int i = 0; i < H; ++i) z += (Real)w2[o][i] * h1[el][i];
-    h2[el][o] = tanh(z);
+    for (int i = 0; i < H; ++i)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) z[q] += (Real)w2[i][o4] * h1[i][e4 + q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) h2[e4 + q][o4] = tanh(z[q]);
   }
   __syncthreads();
   if (tid < 2 * EB) {
