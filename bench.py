@@ -137,11 +137,14 @@ def kernel_bytes(c, Q, rsz, affine, split, learned):
     return kb
 
 
-def launches_per_step(split, learned):
-    """Kernels one step launches: 3 x (stage + assembly), plus the collision/filter
-    prologue of the split form, plus control + drift check + share assembly when learned."""
+def launches_per_step(split, learned, fp64, dim, steps):
+    """Kernels one step launches.  2D: the resident step, one launch for all steps of a call.  3D:
+    3 x (stage + assembly); FP32 split form: a prologue; FP64: filter and collision; learned:
+    node and element features, network, drift check and the assembly of shares besides."""
+    if dim == 2:
+        return 1.0 / steps
     if split:
-        return 6 + (3 if learned else 1)
+        return 6 + (2 if fp64 else 1) + (5 if learned else 0)
     return 6 + (3 if learned else 0)
 
 
@@ -460,14 +463,14 @@ def main():
             "value": value, "ms_per_step": ms / args.steps, "dtype": "f64" if form == "fp64" else "f32",
             "step_form": "population-split" if s.split else "whole-element",
             "kernel_ms": kernel_ms, "kernel_hbm_frac_alg": kernel_frac,
-            "launches_per_step": launches_per_step(s.split, learned),
+            "launches_per_step": launches_per_step(s.split, learned, form == "fp64", case.mesh.dim, args.steps),
             "hbm_gbs_alg_step": step_bytes / (ms / args.steps * 1e-3) / 1e9,
             "bytes_per_update": step_bytes / upd_step,
             "stage23_bytes": kb["stage23"], "stage23_ms": per.get("stage23"),
         }
         if form == "fp64":
-            # FP64 pipe roofline of the stage 2/3 kernel (derivative, metric and stage-combination
-            # flops; the filter and collision run in the prologue or in stage 1)
+            # rate of the stage 2/3 kernel (derivative, metric and stage-combination flops) against
+            # the FP64 pipe's; above 1 where its lines run in 64-bit integers (hexahedra)
             if fp64_tflops is None:
                 fp64_tflops = fp64_peak(torch)
             entry["stage23_flops"] = f23
@@ -500,7 +503,7 @@ def main():
     r = results[main_form]
     if main_form == "fp64":
         achieved = r["stage23_flops"] / (r["stage23_ms"] * 1e-3) / 1e12
-        roof = {"bound": "alu", "kernel": "stage kernel, stages 2 and 3 (FP64 pipe)", "achieved": achieved,
+        roof = {"bound": "alu", "kernel": "stage kernel, stages 2 and 3 (FP64 operations, hexahedra: formed in 64-bit integers)", "achieved": achieved,
                 "peak": fp64_tflops, "unit": "TFLOP/s", "frac": achieved / fp64_tflops,
                 "peak_source": "measured on this GPU: best cuBLAS DGEMM 4096^3", "traffic": None}
     else:
@@ -522,7 +525,7 @@ def main():
             "data": "synthetic",
             "config": workload_config(case, main_form, world),
             "roofline": roof, "forms": results,
-            "gpu_launches": int(results[main_form]["launches_per_step"] * args.steps)}
+            "gpu_launches": int(round(results[main_form]["launches_per_step"] * args.steps))}
     if clocks:
         line["clocks"] = clocks
     if rank == 0 and not args.no_extras:

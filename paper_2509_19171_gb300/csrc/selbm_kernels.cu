@@ -268,8 +268,8 @@ __global__ void __launch_bounds__(512) stage_kernel(const KParams<Real> p) {
 // ---------------------------------------------------------------------------
 // FP64 operations bind the FP64 form as much as memory does (two a clock and SM, about 6 a value):
 // the first copy starts the sum instead of being added to zero, and the force term is left out
-// where there is no force.  Taylor-Green 16^3, D3Q27, N = 7, FP64: 3.94 -> 3.78 ms a step for three
-// assemblies; three parts of 9 populations at 3 CTAs an SM: 3.77 ms, but slower on D3Q19.
+// where there is no force.  Taylor-Green 16^3, D3Q27, N = 7, FP64: 250 -> 198 us an assembly;
+// three parts of 9 populations at 3 CTAs an SM: the same there, slower on D3Q19.
 template <typename Real, int LAT>
 __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2) dss_kernel(const KParams<Real> p) {
   constexpr int Q = Lat<LAT>::Q, DIM = Lat<LAT>::D;
