@@ -12,6 +12,7 @@
 
 #include "../../include/selbm.h"
 #include "selbm_flow2d.h"
+#include "selbm_flow2d_tables.h"
 #include "selbm_kernels.cuh"
 #include "selbm_learn.cuh"
 #include "selbm_lines.h"
@@ -158,57 +159,23 @@ SplitHost split_host(selbm *h) {
                    h->Vm_h.data(), h->Vinv_h.data(), h->sigma.data()};
 }
 
-// tables of the resident 2D step: where a CTA finds the copies and the owner of every boundary
-// node of its elements, and what it fetches from other CTAs
+// tables and buffers of the resident 2D step, for a mesh that the SMs hold (else nothing)
 template <typename Real>
 cudaError_t setup_flow2d(selbm *h) {
   const Setup &S = h->S;
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) return e;
-  const int epc = (S.E + sms - 1) / sms, grid = (S.E + epc - 1) / epc, Nb = S.Nb;
-  std::vector<int32_t> u((size_t)S.E * Nb), off((size_t)S.E * Nb + 1, 0), slot, base((size_t)S.E * Nb), rem, rem_off(1, 0), bas,
-      bas_off(1, 0), at((size_t)S.E * Nb, -1), at_u(S.Gb, -1);
-  for (int k = 0; k < S.Gb; ++k)
-    for (int c = S.bnode_off[k]; c < S.bnode_off[k + 1]; ++c) u[S.bnode_slot[c]] = k;
-  int rmax = 0, bmax = 0;
-  for (int cta = 0; cta < grid; ++cta) {
-    const int e0 = cta * epc, e1 = std::min(S.E, e0 + epc);
-    const size_t rem0 = rem.size(), bas0 = bas.size();
-    for (size_t lb = (size_t)e0 * Nb; lb < (size_t)e1 * Nb; ++lb) {
-      off[lb] = (int32_t)slot.size();
-      const int k = u[lb];
-      for (int c = S.bnode_off[k]; c < S.bnode_off[k + 1]; ++c) {
-        const int s = S.bnode_slot[c], e2 = s / Nb;
-        if (e2 >= e0 && e2 < e1) {
-          slot.push_back(-3 - (s - e0 * Nb));
-          continue;
-        }
-        if (at[s] < 0) { at[s] = (int32_t)(rem.size() - rem0); rem.push_back(e2 * 9 * Nb + s % Nb); }
-        slot.push_back(at[s]);
-      }
-      // the first copy owns the node
-      const int s = S.bnode_slot[S.bnode_off[k]];
-      if ((size_t)s == lb) base[lb] = -1;
-      else if (s / Nb >= e0 && s / Nb < e1) base[lb] = -3 - (s - e0 * Nb);
-      else {
-        if (at_u[k] < 0) { at_u[k] = (int32_t)(bas.size() - bas0); bas.push_back(k); }
-        base[lb] = at_u[k];
-      }
-    }
-    for (size_t r = rem0; r < rem.size(); ++r) at[(size_t)rem[r] / (9 * Nb) * Nb + rem[r] % (9 * Nb)] = -1;
-    for (size_t r = bas0; r < bas.size(); ++r) at_u[bas[r]] = -1;
-    rem_off.push_back((int32_t)rem.size());
-    bas_off.push_back((int32_t)bas.size());
-    rmax = std::max(rmax, (int)(rem.size() - rem0));
-    bmax = std::max(bmax, (int)(bas.size() - bas0));
-  }
-  off[(size_t)S.E * Nb] = (int32_t)slot.size();
-  if (rem.empty()) rem.push_back(0);
-  if (bas.empty()) bas.push_back(0);
+  const int Nb = S.Nb, epc = (S.E + sms - 1) / sms, grid = (S.E + epc - 1) / epc;
   Flow2DArgs<Real> a{};
-  a.E = S.E; a.epc = epc; a.rmax = rmax; a.bmax = bmax;
+  a.E = S.E; a.epc = epc;
+  // without room for fetched shares first: the tables of a mesh that does not fit are not built
   bool fits = false;
+  e = launch_flow2d<Real>(S.N, S.affine, true, a, split_host(h), nullptr, &fits, h->stream);
+  if (e != cudaSuccess || !fits) return e;
+  Flow2DTables t;
+  if (!build_flow2d_tables(S, epc, &t)) return cudaSuccess;
+  a.rmax = t.rmax; a.bmax = t.bmax;
   e = launch_flow2d<Real>(S.N, S.affine, true, a, split_host(h), nullptr, &fits, h->stream);
   if (e != cudaSuccess || !fits) return e;
   auto keep = [&](int32_t **d, const std::vector<int32_t> &v) -> cudaError_t {
@@ -216,12 +183,12 @@ cudaError_t setup_flow2d(selbm *h) {
     if (r == cudaSuccess) h->allocs.push_back(*d);
     return r;
   };
-  if ((e = keep(&h->d_loc_u, u)) || (e = keep(&h->d_loc_off, off)) || (e = keep(&h->d_loc_slot, slot)) ||
-      (e = keep(&h->d_loc_base, base)) || (e = keep(&h->d_rem_off, rem_off)) || (e = keep(&h->d_rem, rem)) ||
-      (e = keep(&h->d_bas_off, bas_off)) || (e = keep(&h->d_bas, bas)))
+  if ((e = keep(&h->d_loc_u, t.u)) || (e = keep(&h->d_loc_off, t.off)) || (e = keep(&h->d_loc_slot, t.slot)) ||
+      (e = keep(&h->d_loc_base, t.base)) || (e = keep(&h->d_rem_off, t.rem_off)) || (e = keep(&h->d_rem, t.rem)) ||
+      (e = keep(&h->d_bas_off, t.bas_off)) || (e = keep(&h->d_bas, t.bas)))
     return e;
-  h->flow_rmax = rmax;
-  h->flow_bmax = bmax;
+  h->flow_rmax = t.rmax;
+  h->flow_bmax = t.bmax;
   auto alloc = [&](void **p, size_t bytes) -> cudaError_t {
     cudaError_t r = cudaMalloc(p, bytes);
     if (r == cudaSuccess) { h->allocs.push_back(*p); r = cudaMemsetAsync(*p, 0, bytes, h->stream); }
@@ -354,7 +321,16 @@ cudaError_t upload_real(selbm *h) {
   if ((e = upload(&dw, wp))) return e; h->d_walls = dw; if (dw) h->allocs.push_back(dw);
   int32_t *q;
   if ((e = upload(&q, woff))) return e; h->d_wall_off = q; h->allocs.push_back(q);
-  return S.dim == 2 && h->use_fast ? setup_flow2d<Real>(h) : cudaSuccess;
+  if (S.dim == 2 && h->use_fast) {
+    // without it the step takes its several-kernel form: no reason to refuse the handle
+    const size_t kept = h->allocs.size();
+    if (setup_flow2d<Real>(h) != cudaSuccess) {
+      cudaGetLastError();
+      h->flow_epc = 0;
+      for (; h->allocs.size() > kept; h->allocs.pop_back()) cudaFree(h->allocs.back());
+    }
+  }
+  return cudaSuccess;
 }
 
 template <typename Real>
