@@ -280,7 +280,8 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2) dss_kernel(con
   const Real *__restrict__ f0 = p.f0;
   Real *__restrict__ fout = p.fout;
   const size_t G = p.Gs;                 // population stride
-  const bool use_f0 = p.A != Real(0);
+  // an argument of weight zero is not read: its buffer may hold the NaN of an earlier state
+  const bool use_f0 = p.A != Real(0), use_in = p.B != Real(0);
   for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < p.Gb; u += gridDim.x * blockDim.x) {
     const int c0 = p.bnode_off[u], c1 = p.bnode_off[u + 1];
     const size_t gid = p.bnode_g[u];
@@ -324,7 +325,8 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2) dss_kernel(con
         const int a = a0 + al;
         if (a >= Q) break;
         const Real base = use_f0 ? p.A * f0[(size_t)a * G + gid] : Real(0);   // stage 1: A = 0
-        Real r = base + p.B * fin[(size_t)a * G + gid] + s[al] * minv;
+        const Real arg = use_in ? fin[(size_t)a * G + gid] : Real(0);         // filtered shares: B = 0
+        Real r = base + p.B * arg + s[al] * minv;
         if (p.has_force) {
           Real eg = 0;
 #pragma unroll
