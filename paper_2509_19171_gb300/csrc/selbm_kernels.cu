@@ -270,7 +270,9 @@ __global__ void __launch_bounds__(512) stage_kernel(const KParams<Real> p) {
 // the first copy starts the sum instead of being added to zero, and the force term is left out
 // where there is no force.  Taylor-Green 16^3, D3Q27, N = 7, FP64: 250 -> 198 us an assembly;
 // three parts of 9 populations at 3 CTAs an SM: the same there, slower on D3Q19.
-template <typename Real, int LAT>
+// SHARES: the shares alone (A = B = 0: the average of filtered copies); f^0 and f^{s-1} are not read, their
+// buffers may hold the NaN of an earlier state.
+template <typename Real, int LAT, bool SHARES>
 __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2) dss_kernel(const KParams<Real> p) {
   constexpr int Q = Lat<LAT>::Q, DIM = Lat<LAT>::D;
   const Real Bdt = p.B * p.dt;
@@ -280,8 +282,7 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2) dss_kernel(con
   const Real *__restrict__ f0 = p.f0;
   Real *__restrict__ fout = p.fout;
   const size_t G = p.Gs;                 // population stride
-  // an argument of weight zero is not read: its buffer may hold the NaN of an earlier state
-  const bool use_f0 = p.A != Real(0), use_in = p.B != Real(0);
+  const bool use_f0 = p.A != Real(0);
   for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < p.Gb; u += gridDim.x * blockDim.x) {
     const int c0 = p.bnode_off[u], c1 = p.bnode_off[u + 1];
     const size_t gid = p.bnode_g[u];
@@ -324,9 +325,12 @@ __global__ void __launch_bounds__(256, sizeof(Real) == 4 ? 4 : 2) dss_kernel(con
       for (int al = 0; al < QH; ++al) {
         const int a = a0 + al;
         if (a >= Q) break;
+        if constexpr (SHARES) {
+          fout[(size_t)a * G + gid] = s[al] * minv;
+          continue;
+        }
         const Real base = use_f0 ? p.A * f0[(size_t)a * G + gid] : Real(0);   // stage 1: A = 0
-        const Real arg = use_in ? fin[(size_t)a * G + gid] : Real(0);         // filtered shares: B = 0
-        Real r = base + p.B * arg + s[al] * minv;
+        Real r = base + p.B * fin[(size_t)a * G + gid] + s[al] * minv;
         if (p.has_force) {
           Real eg = 0;
 #pragma unroll
@@ -397,7 +401,8 @@ static cudaError_t launch_dss_t(const KParams<Real> &p, cudaStream_t s) {
   if (p.Gb == 0) return cudaSuccess;
   const int threads = 256;
   const int blocks = (int)std::min<size_t>(((size_t)p.Gb + threads - 1) / threads, 152 * 32);
-  dss_kernel<Real, LAT><<<blocks, threads, 0, s>>>(p);
+  if (p.A == Real(0) && p.B == Real(0)) dss_kernel<Real, LAT, true><<<blocks, threads, 0, s>>>(p);
+  else dss_kernel<Real, LAT, false><<<blocks, threads, 0, s>>>(p);
   return cudaGetLastError();
 }
 
