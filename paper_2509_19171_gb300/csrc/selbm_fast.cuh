@@ -19,6 +19,7 @@
 #include "selbm_kernels.cuh"
 #include "selbm_lattice.cuh"
 #include "selbm_setup.h"
+#include "selbm_smem.cuh"
 
 namespace slb {
 
@@ -596,17 +597,9 @@ cudaError_t launch_fast_t(const KParams<Real> &p, const double *D, const double 
   m.r = r;
   fill_even_odd(m, D);
   const size_t smem = fast_smem_bytes<Real, LAT, n, AFFINE>(p.wall_max);
-  auto k = stage_fast_kernel<Real, LAT, n, AFFINE>;
-  static thread_local int attr_dev = -1;
-  static thread_local size_t attr_smem = 0;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (attr_dev != dev || attr_smem < smem) {
-    cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    attr_dev = dev;
-    attr_smem = smem;
-  }
+  constexpr auto k = stage_fast_kernel<Real, LAT, n, AFFINE>;
+  const cudaError_t err = raise_smem<k>(smem);
+  if (err != cudaSuccess) return err;
   k<<<p.E, FastShape<LAT, n>::THREADS, smem, s>>>(p, m);
   return cudaGetLastError();
 }

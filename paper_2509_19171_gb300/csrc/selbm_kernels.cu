@@ -7,6 +7,7 @@
 
 #include "selbm_kernels.cuh"
 #include "selbm_setup.h"
+#include "selbm_smem.cuh"
 
 namespace slb {
 
@@ -379,8 +380,8 @@ static int block_for(int lat) { return lat == SELBM_D2Q9 ? 256 : 512; }
 template <typename Real, int LAT, bool AFF>
 static cudaError_t launch_stage_t(const KParams<Real> &p, cudaStream_t s) {
   const size_t smem = stage_smem_bytes(LAT, p.Np, p.n, sizeof(Real));
-  auto k = stage_kernel<Real, LAT, AFF>;
-  cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr auto k = stage_kernel<Real, LAT, AFF>;
+  const cudaError_t err = raise_smem<k>(smem);
   if (err != cudaSuccess) return err;
   k<<<p.E, block_for(LAT), smem, s>>>(p);
   return cudaGetLastError();
@@ -419,8 +420,8 @@ cudaError_t launch_dss(int lat, const KParams<Real> &p, cudaStream_t s) {
 template <typename Real, int LAT>
 static cudaError_t launch_finalize_t(const KParams<Real> &p, cudaStream_t s) {
   const size_t smem = stage_smem_bytes(LAT, p.Np, p.n, sizeof(Real));
-  auto k = finalize_kernel<Real, LAT>;
-  cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr auto k = finalize_kernel<Real, LAT>;
+  const cudaError_t err = raise_smem<k>(smem);
   if (err != cudaSuccess) return err;
   k<<<p.E, block_for(LAT), smem, s>>>(p);
   return cudaGetLastError();

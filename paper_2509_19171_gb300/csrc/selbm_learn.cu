@@ -15,6 +15,7 @@
 #include "selbm_learn.cuh"
 #include "selbm_setup.h"
 #include "selbm_lattice.cuh"
+#include "selbm_smem.cuh"
 
 namespace slb {
 
@@ -230,8 +231,8 @@ template <typename Real, int LAT>
 static cudaError_t launch_control_t(const ControlArgs<Real> &c, cudaStream_t s) {
   const int Q = LT<LAT>::v.Q;
   const size_t smem = (size_t)(Q * c.Np + 2 * c.Np + 2 * c.n * c.n + 2 * c.n + 2 * c.n + 2 * kH + 2 + c.n) * sizeof(Real);
-  auto k = control_kernel<Real, LAT>;
-  cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr auto k = control_kernel<Real, LAT>;
+  const cudaError_t err = raise_smem<k>(smem);
   if (err != cudaSuccess) return err;
   k<<<c.E, 256, smem, s>>>(c);
   return cudaGetLastError();
@@ -319,7 +320,7 @@ cudaError_t launch_element_errors(int E, int dim, int n, int nR, const double *r
   const int Np = dim == 3 ? n * n * n : n * n, NpR = dim == 3 ? nR * nR * nR : nR * nR;
   const int cap = std::max(Np, NpR);
   const size_t smem = (size_t)(2 * cap + n * nR) * sizeof(double);
-  cudaError_t e = cudaFuncSetAttribute(element_errors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = raise_smem<element_errors_kernel>(smem);
   if (e != cudaSuccess) return e;
   element_errors_kernel<<<E, 256, smem, s>>>(dim, n, nR, rho, u, rhoR, uR, I, wq, err);
   return cudaGetLastError();
@@ -621,21 +622,20 @@ static size_t tile_smem(int nin, int ts) {
 // gradient partials grows beyond what the batch needs
 static int tile_samples(int64_t count) { return count <= 8 * 152 ? 8 : (count <= 16 * 304 ? 16 : (count <= 32 * 608 ? 32 : 64)); }
 
+template <int TS>
+static cudaError_t launch_tiles_t(int tiles, const TileArgs &a, int forward_only, cudaStream_t s) {
+  const size_t smem = tile_smem(a.nin, TS);
+  const cudaError_t e = raise_smem<mlp_tile_kernel<TS>>(smem);
+  if (e != cudaSuccess) return e;
+  mlp_tile_kernel<TS><<<tiles, kMlpT, smem, s>>>(a, forward_only);
+  return cudaGetLastError();
+}
 static cudaError_t launch_tiles(int ts, int tiles, const TileArgs &a, int forward_only, cudaStream_t s) {
-  const size_t smem = tile_smem(a.nin, ts);
-  auto go = [&](auto k) -> cudaError_t {
-    if (smem > 48 * 1024) {
-      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-      if (e != cudaSuccess) return e;
-    }
-    k<<<tiles, kMlpT, smem, s>>>(a, forward_only);
-    return cudaGetLastError();
-  };
   switch (ts) {
-    case 8: return go(mlp_tile_kernel<8>);
-    case 16: return go(mlp_tile_kernel<16>);
-    case 32: return go(mlp_tile_kernel<32>);
-    default: return go(mlp_tile_kernel<64>);
+    case 8: return launch_tiles_t<8>(tiles, a, forward_only, s);
+    case 16: return launch_tiles_t<16>(tiles, a, forward_only, s);
+    case 32: return launch_tiles_t<32>(tiles, a, forward_only, s);
+    default: return launch_tiles_t<64>(tiles, a, forward_only, s);
   }
 }
 

@@ -30,6 +30,7 @@
 #include "selbm_fixed.cuh"
 #include "selbm_kernels.cuh"
 #include "selbm_lines.h"
+#include "selbm_smem.cuh"
 #include "selbm_split_stage.cuh"
 
 namespace slb {
@@ -831,22 +832,6 @@ __global__ void __launch_bounds__(256) curved_geo_kernel(const Real *drdx, int N
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
-// dynamic shared-memory limit of kernel K, raised once per device and thread (one set of statics
-// per kernel: kernels of one type are different template values)
-template <auto K>
-cudaError_t raise_smem(size_t smem) {
-  static thread_local int attr_dev = -1;
-  static thread_local size_t attr_smem = 0;
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (attr_dev == dev && attr_smem >= smem) return cudaSuccess;
-  const cudaError_t err = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (err != cudaSuccess) return err;
-  attr_dev = dev;
-  attr_smem = smem;
-  return cudaSuccess;
-}
-
 // Q populations in ng groups of pb, as even as they come
 template <typename Real, int n>
 void line_groups(int Q, int *pb, int *ng) {

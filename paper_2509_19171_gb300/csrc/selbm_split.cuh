@@ -28,6 +28,7 @@
 #include "selbm_collide.cuh"
 #include "selbm_fast.cuh"
 #include "selbm_moments.cuh"
+#include "selbm_smem.cuh"
 #include "selbm_split_stage.cuh"
 
 namespace slb {
@@ -702,27 +703,13 @@ FastMats<Real, n> make_fast_mats(const SplitHost &h) {
   return m;
 }
 
-// sets the kernel's dynamic shared-memory limit once per device (per instantiation)
-#define SLB_SET_SMEM_ONCE(kernel, smem)                                                          \
-  do {                                                                                           \
-    static thread_local int attr_dev_ = -1;                                                      \
-    static thread_local size_t attr_smem_ = 0;                                                   \
-    int dev_ = 0;                                                                                \
-    cudaGetDevice(&dev_);                                                                        \
-    if (attr_dev_ != dev_ || attr_smem_ < (smem)) {                                              \
-      cudaError_t err_ = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem)); \
-      if (err_ != cudaSuccess) return err_;                                                      \
-      attr_dev_ = dev_;                                                                          \
-      attr_smem_ = (smem);                                                                       \
-    }                                                                                            \
-  } while (0)
-
 template <typename Real, int LAT, int n, bool AFFINE, int PBW = 0>
 cudaError_t launch_split_t(const KParams<Real> &p, const SplitHost &h, cudaStream_t s) {
   using S = SplitShape<LAT, n, PBW>;
   const size_t smem = split_smem_bytes<Real, LAT, n, AFFINE, PBW>(p.wall_max);
-  auto k = stage_split_kernel<Real, LAT, n, AFFINE, PBW>;
-  SLB_SET_SMEM_ONCE(k, smem);
+  constexpr auto k = stage_split_kernel<Real, LAT, n, AFFINE, PBW>;
+  const cudaError_t err = raise_smem<k>(smem);
+  if (err != cudaSuccess) return err;
   k<<<p.E * S::NG, S::THREADS, smem, s>>>(p, make_fast_mats<Real, n>(h));
   return cudaGetLastError();
 }
@@ -737,8 +724,9 @@ cudaError_t launch_prologue_t(const KParams<Real> &p, const SplitHost &h, const 
     c.feat_out = lp.feat_out; c.n_fallback = lp.n_fallback; c.outputs = lp.outputs;
   }
   const size_t smem = prologue_smem_bytes<Real, LAT, n, AFFINE, MODE>();
-  auto k = prologue_kernel<Real, LAT, n, AFFINE, MODE>;
-  SLB_SET_SMEM_ONCE(k, smem);
+  constexpr auto k = prologue_kernel<Real, LAT, n, AFFINE, MODE>;
+  const cudaError_t err = raise_smem<k>(smem);
+  if (err != cudaSuccess) return err;
   k<<<p.E, kProThreads, smem, s>>>(p, make_fast_mats<Real, n>(h), c);
   return cudaGetLastError();
 }
