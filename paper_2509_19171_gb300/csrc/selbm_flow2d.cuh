@@ -48,12 +48,17 @@ struct Flow2DShape {
   static constexpr size_t fixed_bytes(bool node) { return (node ? (size_t)n * n * sizeof(Limb) : 0) + (size_t)n * (sizeof(Val) + sizeof(Real)) + (size_t)(Nb + Np + M * M) * sizeof(int) + 64; }
 };
 
+// a word of a packet is one 8-byte access on either side, strong and device-wide, so that a reader
+// sees its value and its tag together
 __device__ __forceinline__ void put_packet(Packet<float> *p, float v, unsigned tag) {
-  __stcg(&p->w[0], ((unsigned long long)tag << 32) | __float_as_uint(v));
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(&p->w[0]), "l"(((unsigned long long)tag << 32) | __float_as_uint(v))
+               : "memory");
 }
 __device__ __forceinline__ void put_packet(Packet<double> *p, double v, unsigned tag) {
   const unsigned long long t = (unsigned long long)tag << 32;
-  __stcg(reinterpret_cast<ulonglong2 *>(p), make_ulonglong2(t | (unsigned)__double2hiint(v), t | (unsigned)__double2loint(v)));
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(&p->w[0]), "l"(t | (unsigned)__double2hiint(v)),
+               "l"(t | (unsigned)__double2loint(v))
+               : "memory");
 }
 __device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long *p) {
   unsigned long long v;
