@@ -37,7 +37,7 @@ enum {
   SELBM_ERR_MESH = -2,      /* non-positive Jacobian, unmatched periodic nodes, bad tags */
   SELBM_ERR_CUDA = -3,      /* a CUDA call failed (text in selbm_last_error) */
   SELBM_ERR_NONFINITE = -4, /* the state holds NaN or Inf */
-  SELBM_ERR_TIMEOUT = -5,   /* a bounded device wait gave up */
+  SELBM_ERR_TIMEOUT = -5,   /* a bounded device wait gave up: the state is lost (see selbm_step) */
   SELBM_ERR_STATE = -6      /* call out of order (e.g. step before init) */
 };
 
@@ -184,10 +184,15 @@ int selbm_get_state(selbm_t *h, double *f, int on_device);
  * Advance nsteps time steps (Sec. 2, summary list): BGK collision with F**,
  * three Shu-Osher SSPRK3 stages of the weak advection with F* and the flux
  * bounce-back wall flux (or the four printed stages, see selbm_set_time_scheme),
- * assembly of shared nodes, explicit filter.  Each step is launched as a captured
- * CUDA graph after one eager step of its kind.
+ * assembly of shared nodes, explicit filter.  A 2D mesh that the SMs hold runs its
+ * steps in one cooperative launch, whose CTAs exchange shares of shared nodes; any
+ * other step is launched as a captured CUDA graph after one eager step of its kind.
  * Asynchronous: enqueues the work and returns.  Errors: SELBM_ERR_STATE
- * (not initialised), SELBM_ERR_CUDA (launch failure).
+ * (not initialised), SELBM_ERR_CUDA (launch failure), SELBM_ERR_TIMEOUT (an exchange of
+ * an earlier step was not answered within seconds and gave up).  After a timeout the
+ * state is lost: selbm_step, the calls that read the state or the learned control, and
+ * the filter setters return SELBM_ERR_TIMEOUT until selbm_init or selbm_set_state has
+ * set a new one (steps and time of selbm_info count the steps that were enqueued).
  */
 int selbm_step(selbm_t *h, int64_t nsteps);
 

@@ -79,6 +79,8 @@ struct selbm {
   int flow_learned = -1;         // whether the resident step with the learned control fits (-1: not asked)
   int flow_pass = 0;
   int *abort_host = nullptr;     // mapped host memory: a bounded wait of the resident step gave up
+  // polls of one wait of the resident step, about a microsecond each; SELBM_FLOW_SPINS in the environment sets it
+  int flow_spins = 4000000;
   int wall_max = 0;
   int n_wallpts = 0;             // wall points (element, node) over all elements
   double *d_xg = nullptr;        // [G][dim] coordinates of unique nodes (uploaded on first use)
@@ -740,9 +742,19 @@ int node_fields(selbm *h, const void *f, bool diag) {
   return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "moments");
 }
 
-// SELBM_ERR_TIMEOUT when a bounded wait has given up (the caller has synchronised the stream)
+// SELBM_ERR_TIMEOUT when a bounded wait has given up (the caller has synchronised the stream): the
+// state is torn until selbm_init or selbm_set_state replaces it
 int wait_status(selbm *h) {
-  return h->abort_host && *(volatile int *)h->abort_host ? h->fail(SELBM_ERR_TIMEOUT, "a wait of the resident 2D step gave up") : SELBM_OK;
+  return h->abort_host && *(volatile int *)h->abort_host
+             ? h->fail(SELBM_ERR_TIMEOUT, "a wait of the resident 2D step gave up: the state has to be set again")
+             : SELBM_OK;
+}
+
+// the same for callers that have not: waits for the stream where the handle may run the resident step
+int settled(selbm *h) {
+  if (!h->abort_host) return SELBM_OK;
+  const cudaError_t e = cudaStreamSynchronize(h->stream);
+  return e == cudaSuccess ? wait_status(h) : h->cuda_fail(e, "step");
 }
 
 // nsteps steps of the resident 2D step, in launches of a bounded length
@@ -761,6 +773,7 @@ cudaError_t run_flow2d(selbm *h, int64_t nsteps, bool probe = false) {
   a.rem_off = h->d_rem_off; a.rem = h->d_rem; a.bas_off = h->d_bas_off; a.bas = h->d_bas;
   a.rmax = h->flow_rmax; a.bmax = h->flow_bmax;
   a.abort = h->abort_host;
+  a.spins = h->flow_spins;
   a.T = h->d_flow_T; a.base = h->d_flow_base; a.f = (Real *)h->FA;
   const SplitHost sh = split_host(h);
   Learn2DArgs<Real> lc{};
@@ -826,6 +839,8 @@ static int create_impl(SetupFn setup, const selbm_params *params, void *cuda_str
     h->use_fast = !(gk && gk[0] == '1');
     const char *ng = std::getenv("SELBM_NO_GRAPH");
     h->graph_enabled = !(ng && ng[0] == '1');
+    const char *fs = std::getenv("SELBM_FLOW_SPINS");
+    if (fs && fs[0]) h->flow_spins = std::max(1, std::atoi(fs));
   }
   std::string err;
   int rc = setup(&h->S, &err);
@@ -970,6 +985,7 @@ int selbm_init(selbm_t *h, const double *rho, const double *u, int on_device) {
   }
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "init");
+  if (h->abort_host) *(volatile int *)h->abort_host = 0;
   h->initialized = true; h->filter_pending = false; h->steps = 0; h->time = 0.0;
   return SELBM_OK;
 }
@@ -990,6 +1006,7 @@ int selbm_set_state(selbm_t *h, const double *f, int on_device) {
                       : launch_set_state<float>(h->lat, df, h->d_first, h->S.G, h->Gs(), nl, h->P.rho0, (float *)h->FA, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "set_state");
+  if (h->abort_host) *(volatile int *)h->abort_host = 0;
   h->initialized = true; h->filter_pending = false;
   return SELBM_OK;
 }
@@ -1046,6 +1063,7 @@ int selbm_step(selbm_t *h, int64_t nsteps) {
   if (!h) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
   if (nsteps < 0) return h->fail(SELBM_ERR_ARG, "nsteps < 0");
+  if (const int rc = wait_status(h)) return rc;      // as far as earlier steps have come
   if (h->learned && h->flow_epc > 0 && h->flow_learned < 0) {
     if (h->prec == SELBM_FP64) run_flow2d<double>(h, 0, true);
     else run_flow2d<float>(h, 0, true);
@@ -1131,6 +1149,7 @@ int selbm_stress(selbm_t *h, double *pi, int on_device) {
 int selbm_set_filter(selbm_t *h, const selbm_filter *f) {
   if (!h || !f) return SELBM_ERR_ARG;
   if (filter_waits(h)) {
+    if (const int rc = settled(h)) return rc;
     // the last step's filter (old settings) must be applied before switching
     int rc = finalize(h);
     if (rc) return rc;
@@ -1315,6 +1334,7 @@ int selbm_radial_profile(selbm_t *h, const double origin[3], const double axis[3
   if (e == cudaSuccess) e = cudaMemcpyAsync(hp.data(), part, hp.size() * 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "radial_profile");
+  if ((rc = wait_status(h))) return rc;
   for (int b = 0; b < nbins; ++b) {
     double su = 0, sm = 0;
     for (int k = 0; k < blocks; ++k) { su += hp[((size_t)k * nbins + b) * 2]; sm += hp[((size_t)k * nbins + b) * 2 + 1]; }
@@ -1391,6 +1411,7 @@ int selbm_set_learned_filter(selbm_t *h, const float *params, const float *lo, c
   for (int i = 0; i < nin; ++i)
     if (!(hi[i] > lo[i])) return h->fail(SELBM_ERR_ARG, "learned filter: hi must exceed lo for every feature");
   if (filter_waits(h)) {
+    if (const int rc = settled(h)) return rc;
     // apply the pending filter with the old settings first
     int rc = finalize(h);
     if (rc) return rc;
@@ -1428,8 +1449,8 @@ int selbm_set_learned_filter(selbm_t *h, const float *params, const float *lo, c
 int selbm_clear_learned_filter(selbm_t *h) {
   if (!h) return SELBM_ERR_ARG;
   if (h->learned && h->filter_pending) {
-    int rc = finalize(h);
-    if (rc) return rc;
+    int rc = settled(h);
+    if (rc || (rc = finalize(h))) return rc;
     cudaError_t e = cudaMemcpyAsync(h->FA, h->BUF, (size_t)h->Q * h->Gs() * h->rsz, cudaMemcpyDeviceToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) return h->cuda_fail(e, "clear_learned_filter");
@@ -1448,6 +1469,7 @@ int selbm_learned_status(selbm_t *h, int64_t out[4]) {
   if (e == cudaSuccess) e = cudaMemsetAsync(h->d_nfb, 0, sizeof(nfb), h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "learned_status");
+  if (const int rc = wait_status(h)) return rc;
   out[0] = flag[0]; out[1] = nfb[0]; out[2] = h->learned ? 1 : 0; out[3] = 0;
   return SELBM_OK;
 }
@@ -1466,7 +1488,7 @@ int selbm_element_sigma(selbm_t *h, double *sigma) {
     for (size_t i = 0; i < cnt; ++i) sigma[i] = tmp[i];
   }
   if (e != cudaSuccess) return h->cuda_fail(e, "element_sigma");
-  return SELBM_OK;
+  return wait_status(h);
 }
 
 int selbm_features(selbm_t *h, float *feat) {
@@ -1486,7 +1508,7 @@ int selbm_features(selbm_t *h, float *feat) {
   e = h->prec == SELBM_FP64 ? run(double()) : run(float());
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return h->cuda_fail(e, "features");
-  return SELBM_OK;
+  return wait_status(h);
 }
 
 int selbm_element_errors(selbm_t *h, selbm_t *ref, double *err) {

@@ -12,7 +12,8 @@
 // knows that they have read its own of exchange k.  Copies of a shared node are summed by every CTA
 // that holds one, in ascending (element, node) order, so that all copies hold the same bits.
 //
-// Waits are bounded: a wait that gives up sets *abort (host memory), and every CTA leaves.
+// Waits are bounded by p.spins polls: a wait that gives up sets *abort (host memory), and every CTA
+// leaves; some may have written their share of the state, so it has to be set anew.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -23,7 +24,6 @@
 namespace slb {
 
 constexpr int kNodeTasks = 3000;            // (population, node) tasks of a CTA up to which FP64 takes a thread per node
-constexpr int kFlowSpins = 4000000;        // polls of one wait, about a microsecond each
 
 template <typename Real, int n>
 struct Flow2DShape {
@@ -321,7 +321,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
     Real v;
     int spin = 0;
     while (!get_packet(q, epoch, v)) {
-      if (++spin >= kFlowSpins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
+      if (++spin >= p.spins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
         *(volatile int *)p.abort = 1;
         s_fail = 1;
         break;
@@ -864,7 +864,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
             double v;
             int spin = 0;
             while (!get_packet(src, pass_tag, v)) {
-              if (++spin >= kFlowSpins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
+              if (++spin >= p.spins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
                 *(volatile int *)p.abort = 1;
                 s_fail = 1;
                 break;

@@ -32,6 +32,7 @@ struct Flow2DArgs {
   const int32_t *bas_off, *bas; // [CTAs + 1] shared-node indices of the owners' values a CTA fetches
   int rmax, bmax;               // most of them
   int *abort;                   // host memory: set when a wait gives up
+  int spins;                    // most polls of one wait
   void *T;                      // [2][E][9][Nb] packets: shares
   void *base;                   // [Gb][10] packets: owner's f^0 and rho of shared nodes after a filter
   Real *f;                      // [9][Gs] state
