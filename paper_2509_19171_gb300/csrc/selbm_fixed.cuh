@@ -15,6 +15,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <algorithm>
 #include <cstdint>
 
 namespace slb {
@@ -38,6 +39,11 @@ __device__ __forceinline__ void fix_mac(Fix128 &s, const Limb &c, const Limb &q)
   s.A += (long long)c.hi * q.hi;
   s.B += (long long)c.hi * q.lo;
   s.B += (long long)c.lo * q.hi;
+}
+// adds C Q with the high word of the lowest product too: the sum is shifted up afterwards
+__device__ __forceinline__ void fix_mac_full(Fix128 &s, const Limb &c, const Limb &q) {
+  fix_mac(s, c, q);
+  s.B += (long long)__mulhi(c.lo, q.lo);
 }
 // (A 2^64 + B 2^32) / 2^(64 - K), 0 <= K <= 31
 template <int K>

@@ -166,7 +166,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   __shared__ double s_red[2][Flow2DShape<Real, n>::TMAX / 32], s_prev[3];
   __shared__ Real s_t[9], s_c[9];                       // weights; B dt 3 t_a e_a . g / B
   __shared__ signed char s_e[9][2], s_o[9];
-  __shared__ Limb s_tc[9];                              // t_a / 2 in fixed point
+  __shared__ Limb s_tc[9];                              // t_a in fixed point
 
   if (tid < 9) {
     static_for<0, 9>([&](auto ac) {
@@ -595,7 +595,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
     };
     if constexpr (F64) {
       // per node the moments and products (see collide_fixed), kept in X: base, P_xx, P_yy, S_xy,
-      // j_x, j_y, exponent (0: the node took the FP64 collision)
+      // j_x, j_y, exponent (0: the node took the FP64 collision), X of the rest population
       int *emn = em + (par ^ 1) * epc * 9;
 #pragma unroll 1
       for (int k = tid; k < epc * 9; k += T) emn[k] = kMinExp;
@@ -607,35 +607,36 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
         long long sr = 0, sx = 0, sy = 0;
 #pragma unroll 3
         for (int a = 0; a < 9; ++a) {
-          const long long v = to_fixed_rn<1>(F[at + a * PS], ex);
+          const long long v = to_fixed_rn<kColShift>(F[at + a * PS], ex);
           sr += v;
           sx += s_e[a][0] * v;
           sy += s_e[a][1] * v;
         }
-        const int sc = ex - (1023 + 52 + 1);
+        const int sc = ex - (1023 + 52 + kColShift);
         double rho = p.rho0 + from_fixed(sr, sc);
         const double inv = 1.0 / rho;
         double vx = from_fixed(sx, sc) * inv, vy = from_fixed(sy, sc) * inv;
         if (forced) { vx += cfix.kappa2 * p.g[0]; vy += cfix.kappa2 * p.g[1]; }
-        const long long ar = sr < 0 ? -sr : sr, aj = (sx < 0 ? -sx : sx) + (sy < 0 ? -sy : sy);
-        if (ex == 2047 || max(exp_of(vx), exp_of(vy)) > 1020 || ar >= (1ll << 60) || aj >= (3ll << 57)) ex = 0;
+        const long long js = ((sx < 0 ? -sx : sx) >> 1) + ((sy < 0 ? -sy : sy) >> 1);
+        if (!fix_in_range<2>(ex, max(exp_of(vx), exp_of(vy)), 2 * js)) ex = 0;
         X[at + 6 * PS] = ex;
         if (ex == 0) {
           rho = collide_fp64(F + at, PS, p.rho0, p.omega, p.dt, p.half_dt, p.g[0], p.g[1], forced);
         } else {
-          const Limb jx = limbs(sx), jy = limbs(sy), ux = limbs(to_fixed<6>(vx, 1022)), uy = limbs(to_fixed<6>(vy, 1022));
+          const Limb jx = limbs(sx), jy = limbs(sy), ux = limbs(fix_velocity(vx)), uy = limbs(fix_velocity(vy));
           Fix128 xx{0, 0}, yy{0, 0}, xy{0, 0};
           fix_mac(xx, jx, ux);
           fix_mac(yy, jy, uy);
           fix_mac(xy, jx, uy);
           fix_mac(xy, jy, ux);
-          const long long P = fix_top<5>(xx), R = fix_top<5>(yy);
-          X[at] = 2 * sr - 3 * (P + R);
+          const long long P = fix_product(xx), R = fix_product(yy);
+          X[at] = fix_base4(sr, P + R);
           X[at + PS] = P;
           X[at + 2 * PS] = R;
-          X[at + 3 * PS] = fix_top<5>(xy);
+          X[at + 3 * PS] = fix_product(xy);
           X[at + 4 * PS] = sx;
           X[at + 5 * PS] = sy;
+          X[at + 7 * PS] = fix_rest(sr, P + R);
         }
         if (forced) {
           srho[el * PS + off[i]] = rho;
@@ -651,11 +652,8 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
         if (ex != 0) {
           const int cx = s_e[a][0], cy = s_e[a][1];
           const long long even = (cx ? x[PS] : 0) + (cy ? x[2 * PS] : 0) + cx * cy * x[3 * PS];
-          const long long x2 = x[0] + 9 * even + 6 * (cx * x[4 * PS] + cy * x[5 * PS]), qa = to_fixed_rn<1>(v, ex);
-          Fix128 fe{0, 1ll << 31}, w{0, 1ll << 28};       // rounded to nearest
-          fix_mac(fe, s_tc[a], limbs(x2));
-          fix_mac(w, cfix.w, limbs(fix_top<0>(fe) - qa));
-          v = from_fixed(qa + fix_top<3>(w), ex - (1023 + 52 + 1));
+          const long long x4 = x[0] + fix_even4(even) + 3 * fix_quarter(cx * x[4 * PS] + cy * x[5 * PS]);
+          v += fix_change(cfix, s_tc[a], a == 0 ? x[7 * PS] : x4, to_fixed_rn<kColShift>(v, ex), ex);
         }
         F[at] = v;
         F0[at] = v;

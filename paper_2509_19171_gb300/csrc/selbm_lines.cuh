@@ -228,11 +228,6 @@ __device__ __forceinline__ void line_filter(const FilterMats<float, n> &m, const
   for (int j = 1; j < H; ++j) { v[j] += ac[0][j] + ac[1][j]; v[n - 1 - j] += ac[0][j] - ac[1][j]; }
   if constexpr (n & 1) v[H] += ac[0][H];
 }
-// adds C Q with the high word of the lowest product too: the sum is shifted up afterwards
-__device__ __forceinline__ void fix_mac_full(Fix128 &s, const Limb &c, const Limb &q) {
-  fix_mac(s, c, q);
-  s.B += (long long)__mulhi(c.lo, q.lo);
-}
 constexpr int kFilterShift = 4;   // |q| < 2^57: the three passes grow a tile by less than 2^4
 // even modes first: their correction is the same at both ends of a pair and leaves the differences
 // that the odd modes read unchanged, so one half's sums are in registers at a time

@@ -91,21 +91,35 @@ __device__ __forceinline__ int node_moments(const Real (&g)[LT<LAT>::v.Q], doubl
 // collision of Sec. 2.1 with F** is
 //   f* = f + omega (t X - f),  X = drho + 3 e.j + 4.5 e e : P - 1.5 tr P,  P = (j v + v j) / 2,
 // since rho (e.u)^2 = e e : (j u), and F** = t (9 (e.u)(e.F) - 3 u.F) with F = rho a enters f* as
-// (1/omega - 1/2) dt omega F**.  The populations become integers at the node's largest exponent
-// (rounded to nearest), moments and X are exact integer sums, and each population takes two
+// (1/omega - 1/2) dt omega F**.  The populations become integers at the node's largest exponent with
+// kColShift bits below its last FP64 bit (rounded to nearest), moments are exact integer sums, X is
+// formed in units of four (t <= 1/9 brings it back below one) and each population takes two
 // fixed-point products (t and omega): about 60 integer instructions where the FP64 form takes 12
-// FP64 ones, at 32 times their issue cost.  rho, 1 / rho and u stay FP64.
-// Nodes beyond the integers' range (|v| >= 1/4, a density or momentum far above the largest
-// deviation, infinities, NaN) take the FP64 collision.
+// FP64 ones, at 32 times their issue cost.  The change omega (t X - f) alone returns to FP64, times
+// 2^w_shift so that a small omega keeps its bits, and is added to f: a population that is small next
+// to the node's largest one keeps all of its own bits.  rho, 1 / rho and u stay FP64.
+// Nodes beyond the integers' range (|v| >= 1/4, a momentum far above the largest deviation,
+// infinities, NaN) take the FP64 collision.
+//
+// Bounds, in units of the integers, m = 2^(53 + kColShift) above every |q|: |sum q| <= 27 m < 2^62;
+// with js = |j_x| + |j_y| + |j_z| < 2^62 (2D: 2^61) and |v_k| < 1/4, |X| / 4 < 7.8 2^60, so that t X and
+// omega (t X - q) stay below 2^63.
+// The corner populations of D3Q27 (t = 1 / 216) are small next to a node's largest one and take three
+// bits more.
+constexpr int kColShift = 4;
+constexpr int speed_class(const VelTab &v, int a) { return v.e[a][0] * v.e[a][0] + v.e[a][1] * v.e[a][1] + v.e[a][2] * v.e[a][2]; }
+constexpr int fine_bits(int cls) { return cls == 3 ? 3 : 0; }
 struct CollideFix {
-  Limb t[4];        // t_c / 2 times 2^64 by speed class
-  Limb w;           // omega times 2^61
+  Limb t[4];        // t_c 2^66 by speed class (rest: 2^64)
+  Limb w;           // omega times 2^(61 + w_shift), in [2^61, 2^62]
+  int w_shift;
   double kappa2;    // 2 kappa
 };
 inline CollideFix make_collide_fix(const double *t_class, double omega, double dt) {
   CollideFix c{};
-  for (int k = 0; k < 4; ++k) c.t[k] = limbs((long long)std::llrint(std::ldexp(0.5 * t_class[k], 64)));
-  c.w = limbs((long long)std::llrint(std::ldexp(omega, 61)));
+  for (int k = 0; k < 4; ++k) c.t[k] = limbs((long long)std::llrint(std::ldexp(t_class[k], k == 0 ? 64 : 66)));
+  c.w_shift = std::max(0, std::min(60, -std::ilogb(omega)));
+  c.w = limbs((long long)std::llrint(std::ldexp(omega, 61 + c.w_shift)));
   c.kappa2 = 2.0 * (1.0 / omega - 0.5) * dt;
   return c;
 }
@@ -113,13 +127,37 @@ template <int LAT>
 CollideFix make_collide_fix(double omega, double dt) {
   constexpr VelTab V = LT<LAT>::v;
   double t[4] = {0, 0, 0, 0};
-  for (int a = 0; a < V.Q; ++a) t[V.e[a][0] * V.e[a][0] + V.e[a][1] * V.e[a][1] + V.e[a][2] * V.e[a][2]] = V.t[a];
+  for (int a = 0; a < V.Q; ++a) t[speed_class(V, a)] = V.t[a];
   return make_collide_fix(t, omega, dt);
+}
+
+// a velocity below 1/4 as an integer times 2^62, and the largest momentum of the integers' range
+__device__ __forceinline__ long long fix_velocity(double v) { return to_fixed_rn<9>(v, 1022); }
+template <int DIM>
+__device__ __forceinline__ bool fix_in_range(int em, int ev, long long js) {
+  return em != 2047 && ev <= 1020 && js < (1ll << (DIM == 2 ? 61 : 62));
+}
+// j v in the integers' units, v from fix_velocity
+__device__ __forceinline__ long long fix_product(const Fix128 &s) { return fix_top<2>(s); }
+// X / 4 of the moving populations: sr / 4 + 3 ej / 4 + (9 even - 3 tr) / 8, each part rounded
+__device__ __forceinline__ long long fix_quarter(long long x) { return (x + 2) >> 2; }
+__device__ __forceinline__ long long fix_base4(long long sr, long long tr) { return fix_quarter(sr) - ((3 * tr + 4) >> 3); }
+__device__ __forceinline__ long long fix_rest(long long sr, long long tr) { return sr - ((3 * tr + 1) >> 1); }
+__device__ __forceinline__ long long fix_even4(long long even) { return even + ((even + 4) >> 3); }
+// omega (t X - q) of one population, as FP64; t from CollideFix, x is X (rest) or X / 4, q has FINE bits
+// more than x
+template <int FINE = 0>
+__device__ __forceinline__ double fix_change(const CollideFix &cf, const Limb &t, long long x, long long q, int em) {
+  Fix128 f{0, 1ll << (31 - FINE)};                       // + 1/2: rounded to nearest
+  fix_mac_full(f, t, limbs(x));
+  Fix128 r{0, 1ll << 28};
+  fix_mac_full(r, cf.w, limbs(fix_top<FINE>(f) - q));
+  return from_fixed(fix_top<3>(r), em - (1023 + 52 + kColShift + FINE) - cf.w_shift);
 }
 
 // what the relaxation of a node's populations needs
 struct NodeRelax {
-  long long base, P[3], S[3], j[3];
+  long long rest, base, P[3], S[3], j[3];
   int em;           // exponent of the node's integers; 0: beyond their range (FP64 collision)
 };
 
@@ -128,14 +166,16 @@ template <int LAT, typename Load>
 __device__ __forceinline__ double collide_moments(const CollideFix &cf, double rho0, const double (&acc)[3], bool forced,
                                                   Load load, long long (&q)[LT<LAT>::v.Q], NodeRelax &r) {
   constexpr VelTab V = LT<LAT>::v;
-  constexpr int Q = V.Q, DIM = V.D, SH = 1;              // |q| <= 2^54
+  constexpr int Q = V.Q, DIM = V.D;
   int em = kMinExp;
   {
     double g[Q];
 #pragma unroll
     for (int a = 0; a < Q; ++a) { g[a] = load(a); em = max(em, exp_of(g[a])); }
-#pragma unroll
-    for (int a = 0; a < Q; ++a) q[a] = to_fixed_rn<SH>(g[a], em);
+    static_for<0, Q>([&](auto ac) {
+      constexpr int a = decltype(ac)::value;
+      q[a] = to_fixed_rn<kColShift + fine_bits(speed_class(V, a))>(g[a], em);
+    });
   }
   long long sr = 0, sj[3] = {0, 0, 0};
   static_for<0, Q>([&](auto ac) {
@@ -143,8 +183,9 @@ __device__ __forceinline__ double collide_moments(const CollideFix &cf, double r
     if constexpr (o == a) {
       sr += q[a];
     } else if constexpr (o > a) {
-      const long long d = q[a] - q[o];
-      sr += q[a] + q[o];
+      constexpr int fine = fine_bits(speed_class(V, a)), half = (1 << fine) >> 1;
+      const long long d = (q[a] - q[o] + half) >> fine;
+      sr += (q[a] + q[o] + half) >> fine;
 #pragma unroll
       for (int k = 0; k < DIM; ++k) {
         if (V.e[a][k] > 0) sj[k] += d;
@@ -152,7 +193,7 @@ __device__ __forceinline__ double collide_moments(const CollideFix &cf, double r
       }
     }
   });
-  const int ex = em - (1023 + 52 + SH);
+  const int ex = em - (1023 + 52 + kColShift);
   const double rho = rho0 + from_fixed(sr, ex);
   const double inv = 1.0 / rho;
   double v[3] = {0, 0, 0};
@@ -163,20 +204,19 @@ __device__ __forceinline__ double collide_moments(const CollideFix &cf, double r
     v[k] = from_fixed(sj[k], ex) * inv;
     if (forced) v[k] += cf.kappa2 * acc[k];
     ev = max(ev, exp_of(v[k]));
-    js += sj[k] < 0 ? -sj[k] : sj[k];
+    js += (sj[k] < 0 ? -sj[k] : sj[k]) >> 2;             // quarters: three sums of 2^62 stay in range
   }
-  const long long sra = sr < 0 ? -sr : sr;
-  r.em = em == 2047 || ev > 1020 || sra >= (1ll << 60) || js >= (3ll << 57) ? 0 : em;
+  r.em = fix_in_range<DIM>(em, ev, js * 4) ? em : 0;
   // P_kk and S_kl = 2 P_kl
   Limb lj[3], lv[3];
 #pragma unroll
-  for (int k = 0; k < DIM; ++k) { lj[k] = limbs(sj[k]); lv[k] = limbs(to_fixed<6>(v[k], 1022)); }   // v 2^59
+  for (int k = 0; k < DIM; ++k) { lj[k] = limbs(sj[k]); lv[k] = limbs(fix_velocity(v[k])); }
   long long tr = 0;
 #pragma unroll
   for (int k = 0; k < DIM; ++k) {
     Fix128 s{0, 0};
     fix_mac(s, lj[k], lv[k]);
-    r.P[k] = fix_top<5>(s);
+    r.P[k] = fix_product(s);
     r.j[k] = sj[k];
     tr += r.P[k];
   }
@@ -187,43 +227,43 @@ __device__ __forceinline__ double collide_moments(const CollideFix &cf, double r
       Fix128 s{0, 0};
       fix_mac(s, lj[k], lv[l]);
       fix_mac(s, lj[l], lv[k]);
-      r.S[k + l - 1] = fix_top<5>(s);                    // xy, xz, yz
+      r.S[k + l - 1] = fix_product(s);                   // xy, xz, yz
     }
-  r.base = 2 * sr - 3 * tr;
+  r.base = fix_base4(sr, tr);
+  r.rest = fix_rest(sr, tr);
   return rho;
 }
 
 // relaxed populations a and its opposite (a <= opposite) of a node within the integers' range
-template <int LAT, int a, typename Store>
-__device__ __forceinline__ void collide_pair(const CollideFix &cf, const NodeRelax &r, long long qa, long long qo, Store store) {
+template <int LAT, int a, typename Load, typename Store>
+__device__ __forceinline__ void collide_pair(const CollideFix &cf, const NodeRelax &r, long long qa, long long qo,
+                                             Load load, Store store) {
   constexpr VelTab V = LT<LAT>::v;
-  constexpr int DIM = V.D, o = LT<LAT>::v.opp[a], ea = V.e[a][0], eb = V.e[a][1], ec = V.e[a][2];
-  constexpr int cls = ea * ea + eb * eb + ec * ec;
-  long long even = 0, ej = 0;
+  constexpr int DIM = V.D, o = LT<LAT>::v.opp[a], cls = speed_class(V, a), fine = fine_bits(cls);
+  if constexpr (o == a) {
+    store(a, load(a) + fix_change(cf, cf.t[0], r.rest, qa, r.em));
+  } else {
+    long long even = 0, ej = 0;
 #pragma unroll
-  for (int k = 0; k < DIM; ++k) {
-    if (V.e[a][k] != 0) even += r.P[k];
-    if (V.e[a][k] > 0) ej += r.j[k];
-    else if (V.e[a][k] < 0) ej -= r.j[k];
+    for (int k = 0; k < DIM; ++k) {
+      if (V.e[a][k] != 0) even += r.P[k];
+      if (V.e[a][k] > 0) ej += r.j[k];
+      else if (V.e[a][k] < 0) ej -= r.j[k];
 #pragma unroll
-    for (int l = k + 1; l < DIM; ++l) {
-      if (V.e[a][k] * V.e[a][l] > 0) even += r.S[k + l - 1];
-      else if (V.e[a][k] * V.e[a][l] < 0) even -= r.S[k + l - 1];
+      for (int l = k + 1; l < DIM; ++l) {
+        if (V.e[a][k] * V.e[a][l] > 0) even += r.S[k + l - 1];
+        else if (V.e[a][k] * V.e[a][l] < 0) even -= r.S[k + l - 1];
+      }
     }
+    const long long e4 = r.base + fix_even4(even), o4 = 3 * fix_quarter(ej);
+    const double fa = load(a), fo = load(o);
+    store(a, fa + fix_change<fine>(cf, cf.t[cls], e4 + o4, qa, r.em));
+    store(o, fo + fix_change<fine>(cf, cf.t[cls], e4 - o4, qo, r.em));
   }
-  const long long e9 = r.base + 9 * even, o6 = 6 * ej;
-  auto relax = [&](int b, long long q, long long x2) {
-    Fix128 f{0, 1ll << 31};                              // + 1/2: rounded to nearest
-    fix_mac(f, cf.t[cls], limbs(x2));
-    Fix128 w{0, 1ll << 28};
-    fix_mac(w, cf.w, limbs(fix_top<0>(f) - q));
-    store(b, from_fixed(q + fix_top<3>(w), r.em - (1023 + 52 + 1)));
-  };
-  relax(a, qa, e9 + o6);
-  if constexpr (o != a) relax(o, qo, e9 - o6);
 }
 
-// load(a) / store(a, value) of the node's deviations (load before any store); returns rho
+// load(a) / store(a, value) of the node's deviations (a population is loaded again before its store:
+// from the cache, as its integer and its value do not both fit the registers); returns rho
 template <int LAT, typename Load, typename Store>
 __device__ __forceinline__ double collide_fixed(const CollideFix &cf, double rho0, double omega, double dt, double half_dt,
                                                 const double (&acc)[3], bool forced, Load load, Store store) {
@@ -242,7 +282,7 @@ __device__ __forceinline__ double collide_fixed(const CollideFix &cf, double rho
   }
   static_for<0, Q>([&](auto ac) {
     constexpr int a = decltype(ac)::value, o = LT<LAT>::v.opp[a];
-    if constexpr (o >= a) collide_pair<LAT, a>(cf, r, q[a], q[o], store);
+    if constexpr (o >= a) collide_pair<LAT, a>(cf, r, q[a], q[o], load, store);
   });
   return rho;
 }
