@@ -137,7 +137,8 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   float *sW2 = sW1 + (LEARNED ? 2 * n * 64 : 0);        // [64][65] W2 transposed
   float *sb = sW2 + (LEARNED ? 64 * 65 : 0);            // b1[64], b2[64], W3[2][64], b3[2]
   int *sin = reinterpret_cast<int *>(sb + (LEARNED ? 4 * 64 + 2 : 0));      // [ne] features in range
-  Val *cf = reinterpret_cast<Val *>(smem_raw + (LEARNED ? (((unsigned char *)(sin + epc) - smem_raw) + 15) / 16 * 16
+  int *sgs = sin + (LEARNED ? epc : 0);                 // FP64: [ne] shift of sge (filter_gain)
+  Val *cf = reinterpret_cast<Val *>(smem_raw + (LEARNED ? (((unsigned char *)(sgs + epc) - smem_raw) + 15) / 16 * 16
                                                         : (size_t)epc * 9 * PS * sizeof(Val)));   // affine [ne][9][2]: -dt e.grad r_l; curved [ne][4][PS]: dr_l/dx_k
   Limb *FQ = reinterpret_cast<Limb *>(cf + (size_t)epc * (AFFINE ? 18 : 4 * PS));   // NODE: [ne][9][PS] f in fixed point
   Limb *sD = FQ + (NODE ? (size_t)epc * 9 * PS : 0);    // NODE: [n][n] D_hat
@@ -184,7 +185,7 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   if (tid == 0) s_fail = 0;
   if (tid < n) {
     sgd[tid] = fm.g[tid];
-    if constexpr (F64) sgk[tid] = __double2ll_rn(fm.g[tid] * 0x1p60);
+    if constexpr (F64) sgk[tid] = filter_gain(fm.g[tid], filter_gain_shift(fm, fm.ex));
     else sgk[tid] = fm.g[tid];
   }
 #pragma unroll 1
@@ -513,10 +514,11 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
       __syncthreads();
       tiles(Cn{}, ne, [&](int el, int k) {
         const bool use_net = sin[el] && !s_flag;
-        Real g = fm.g[k];
+        Real g = fm.g[k], last = 0;                         // last: g of the highest mode, the largest
         if (use_net) {
           const Real gam = Real(0.5) / (Real(1) + exp(-sO[2 * el])), kc = Real(2) + Real(n - 4) / (Real(1) + exp(-sO[2 * el + 1]));
           g = 0;
+          last = (Real(1) - gam) - Real(1);
           if (k > kc) {
             const Real r = (Real(k) - kc) / (Real(n - 1) - kc);
             // sigma = 1 - gamma r^2 rounded as the transfer function that is handed out
@@ -526,8 +528,11 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
           atomicAdd(lc.n_fallback, 1);
         }
         sged[el * n + k] = g;
-        if constexpr (F64) sge[el * n + k] = __double2ll_rn(g * 0x1p60);
-        else sge[el * n + k] = g;
+        if constexpr (F64) {
+          const int sh = filter_gain_shift(fm, use_net ? exp_of(last) : fm.ex);
+          sge[el * n + k] = filter_gain(g, sh);
+          if (k == 0) sgs[el] = sh;
+        } else sge[el * n + k] = g;
         lc.sigma_out[(size_t)(e0 + el) * n + k] = g + Real(1);
       });
       __syncthreads();
@@ -555,7 +560,8 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
               slow_filter_row<n>(fm, LEARNED ? sged + q / 9 * n : sgd, row, st);
               return;
             }
-            line_filter<n>(fm, LEARNED ? sge + q / 9 * n : sgk, v);
+            if constexpr (LEARNED) line_filter<n>(fm, sge + q / 9 * n, sgs[q / 9], v);
+            else line_filter<n>(fm, sgk, filter_gain_shift(fm, fm.ex), v);
           } else line_filter<n>(fm, LEARNED ? sge + q / 9 * n : sgk, v);
 #pragma unroll
           for (int k = 1; k < n - 1; ++k) row[k * st] = v[k];
@@ -565,7 +571,9 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
       if constexpr (F64) {
         tiles(CNp{}, ntile, [&](int q, int i) {
           const int ex = em[par * epc * 9 + q], at = q * PS + off[i];
-          F[at] = ex == 2047 ? __longlong_as_double(X[at]) : from_fixed(X[at], ex - (1023 + 52 + kFilterShift));
+          // the tile's change alone, see lines_filter_kernel
+          F[at] = ex == 2047 ? __longlong_as_double(X[at])
+                             : F[at] + from_fixed(X[at] - to_fixed<kFilterShift>(F[at], ex), ex - (1023 + 52 + kFilterShift));
         });
         __syncthreads();
       }

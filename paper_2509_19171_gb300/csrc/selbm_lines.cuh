@@ -90,6 +90,7 @@ struct FilterMats {
   Real g[n];                                 // sigma_k - 1 of the fixed filter
   Real w[n];
   int cw, cu;
+  int ex;                                    // biased exponent of the largest |g|
 };
 
 template <typename Real, int n>
@@ -136,6 +137,7 @@ FilterMats<Real, n> make_filter_mats(const SplitHost &h) {
   m.cu = fix_shift(ru, 61);
   for (int k = 0; k < n; ++k) {
     m.g[k] = (Real)(h.fixed_sigma[k] - 1.0);
+    if (h.fixed_sigma[k] != 1.0) m.ex = std::max(m.ex, std::max(0, 1023 + std::ilogb(h.fixed_sigma[k] - 1.0)));
     m.w[k] = (Real)h.w[k];
     for (int j = 0; j < S::HE; ++j) {
       const double u = j == 0 || k < 2 ? 0.0 : h.Vm[j * n + k], w = k < 2 ? 0.0 : h.Vinv[k * n + j];
@@ -228,13 +230,27 @@ __device__ __forceinline__ void line_filter(const FilterMats<float, n> &m, const
   for (int j = 1; j < H; ++j) { v[j] += ac[0][j] + ac[1][j]; v[n - 1 - j] += ac[0][j] - ac[1][j]; }
   if constexpr (n & 1) v[H] += ac[0][H];
 }
-constexpr int kFilterShift = 4;   // |q| < 2^57: the three passes grow a tile by less than 2^4
-// even modes first: their correction is the same at both ends of a pair and leaves the differences
-// that the odd modes read unchanged, so one half's sums are in registers at a time
+// |q| < 2^57: a pass grows a tile's largest value by at most 3.8 for transfer functions in [0, 1]
+// (N <= 9; N = 14: 5.0), three passes stay below 2^63 and the sums of a pair before the last below 2^62.
+constexpr int kFilterShift = 4;
+// sigma_k - 1 is taken times 2^(60 + shift): a weak filter's change keeps its bits.  ex: largest exponent
+// of |sigma_k - 1| (at most 1)
 template <int n>
-__device__ __forceinline__ void line_filter(const FilterMats<double, n> &m, const long long *g, long long (&v)[n]) {
+__host__ __device__ __forceinline__ int filter_up(const FilterMats<double, n> &m) { return 123 - m.cu - m.cw; }
+template <int n>
+__device__ __forceinline__ int filter_gain_shift(const FilterMats<double, n> &m, int ex) {
+  return min(max(1022 - ex, 0), filter_up(m));
+}
+__device__ __forceinline__ long long filter_gain(double g, int shift) { return __double2ll_rn(scalbn(g, 60 + shift)); }
+// v <- v + sum_k g_k U_k (W_k . v), g from filter_gain.  Even modes first: their correction is the same at
+// both ends of a pair and leaves the differences that the odd modes read unchanged, so one half's sums are
+// in registers at a time (and the even half's fractions).  Rounding: s = W_k . v to a fraction of v's unit
+// times g, both halves' corrections together to the nearest unit.
+template <int n>
+__device__ __forceinline__ void line_filter(const FilterMats<double, n> &m, const long long *g, int shift, long long (&v)[n]) {
   constexpr int H = n / 2, HE = (n + 1) / 2;
-  const int up = 125 - m.cu - m.cw;                     // to the units of v
+  const int up = filter_up(m) - shift;                  // to the units of v
+  int fe[HE];                                           // fractions of the even half, in 2^-29
   auto half = [&](auto qc) {
     constexpr int q = decltype(qc)::value, K = q ? H : HE;
     Limb x[K];
@@ -245,13 +261,13 @@ __device__ __forceinline__ void line_filter(const FilterMats<double, n> &m, cons
     for (int j = 0; j < K; ++j) ac[j] = Fix128{0, 0};
 #pragma unroll
     for (int k = 2 + q; k < n; k += 2) {
-      const long long gk = g[k];                        // (sigma_k - 1) 2^60
+      const long long gk = g[k];
       if (gk != 0) {
-        Fix128 s{0, 0}, t{0, 0};
+        Fix128 s{0, 1ll << 26}, t{0, 1ll << 27};
 #pragma unroll
-        for (int j = 0; j < K; ++j) fix_mac(s, m.W[k][j], x[j]);
-        fix_mac_full(t, limbs(gk), limbs(fix_top<3>(s)));
-        const Limb y = limbs(fix_top<4>(t));            // g s in units of 2^(61 - cw)
+        for (int j = 0; j < K; ++j) fix_mac_full(s, m.W[k][j], x[j]);
+        fix_mac_full(t, limbs(gk), limbs(fix_top<5>(s)));
+        const Limb y = limbs(fix_top<4>(t));            // g s in units of 2^(59 - cw - shift)
 #pragma unroll
         for (int j = 1; j < K; ++j) fix_mac_full(ac[j], m.U[k][j], y);
       }
@@ -259,9 +275,17 @@ __device__ __forceinline__ void line_filter(const FilterMats<double, n> &m, cons
 #pragma unroll
     for (int j = 1; j < K; ++j) {
       const long long a = (long long)((unsigned long long)ac[j].A << up) + (ac[j].B >> (32 - up));
-      v[j] += a;
-      if (2 * j != n - 1) v[n - 1 - j] += q ? -a : a;
+      const int f = (int)(((unsigned)ac[j].B << up) >> 3);
+      if constexpr (q == 0) {
+        fe[j] = f;
+        v[j] += a;
+        if (2 * j != n - 1) v[n - 1 - j] += a;
+      } else {
+        v[j] += a + ((fe[j] + f + (1 << 28)) >> 29);
+        v[n - 1 - j] += ((fe[j] - f + (1 << 28)) >> 29) - a;
+      }
     }
+    if constexpr (q == 1 && (n & 1)) v[H] += (fe[H] + (1 << 28)) >> 29;
   };
   half(std::integral_constant<int, 0>{});
   half(std::integral_constant<int, 1>{});
@@ -708,17 +732,23 @@ lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Re
   Val *sgk = tile + pb * PS;                                 // [n] sigma_k - 1
   Real *sgd = reinterpret_cast<Real *>(sgk + n);             // [n] the same as a Real
   int *em = reinterpret_cast<int *>(sgd + n);                // [pb]
+  int *gsh = em + pb;                                        // FP64: shift of sgk (filter_gain)
   const int e = blockIdx.x / ng, a0 = (blockIdx.x - e * ng) * pb;
   const int na = min(pb, Q - a0);
   const int tid = threadIdx.x;
   const int32_t *l2g = p.l2g + (size_t)e * Np;
   const size_t G = p.Gs;
   if (F64 && tid < pb) em[tid] = kMinExp;
-  if (tid < n) {
-    const Real g = LEARNED ? sigma[(size_t)e * n + tid] - Real(1) : m.g[tid];
-    sgd[tid] = g;
-    if constexpr (F64) sgk[tid] = __double2ll_rn(g * 0x1p60);
-    else sgk[tid] = g;
+  if (tid < 32) {
+    const int k = min(tid, n - 1);
+    const Real g = LEARNED ? sigma[(size_t)e * n + k] - Real(1) : m.g[k];
+    Val gk;
+    if constexpr (F64) {
+      const int sh = filter_gain_shift(m, LEARNED ? __reduce_max_sync(0xffffffffu, exp_of(g)) : m.ex);
+      gk = filter_gain(g, sh);
+      if (tid == 0) *gsh = sh;
+    } else gk = g;
+    if (tid < n) { sgd[tid] = g; sgk[tid] = gk; }
   }
   if (F64) __syncthreads();
   gather_lines<Real, n, kFilterShift>(tile, em, p.fin + (size_t)a0 * G, G, l2g, na, tid);
@@ -741,6 +771,8 @@ lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Re
 #pragma unroll
         for (int j = 0; j < n; ++j) v[j] = __double_as_longlong(o[j]);
       }
+    } else if constexpr (F64) {
+      line_filter<n>(m, sgk, *gsh, v);
     } else {
       line_filter<n>(m, sgk, v);
     }
@@ -768,10 +800,15 @@ lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Re
 #pragma unroll 1
   for (int i = tid; i < Np; i += T) {
     const Val *v = tile + tile_offset<Real, n>(i);
+    const Real *src = p.fin + (size_t)a0 * G + l2g[i];
+    // FP64: the value that came in plus the tile's change, so that neither small values nor modes that
+    // stay lose bits to the tile's scale
     auto value = [&](int pl) -> Real {
       if constexpr (F64) {
         const int ex = em[pl];
-        return ex == 2047 ? __longlong_as_double(v[pl * PS]) : from_fixed(v[pl * PS], ex - (1023 + 52 + kFilterShift));
+        if (ex == 2047) return __longlong_as_double(v[pl * PS]);
+        const double in = __ldg(src + (size_t)pl * G);
+        return in + from_fixed(v[pl * PS] - to_fixed<kFilterShift>(in, ex), ex - (1023 + 52 + kFilterShift));
       } else return v[pl * PS];
     };
     Real w = 1;
