@@ -802,7 +802,7 @@ lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Re
     const Val *v = tile + tile_offset<Real, n>(i);
     const Real *src = p.fin + (size_t)a0 * G + l2g[i];
     // FP64: the value that came in plus the tile's change, so that neither small values nor modes that
-    // stay lose bits to the tile's scale
+    // stay lose bits to the tile's scale (the loop over the group is unrolled: its loads go out together)
     auto value = [&](int pl) -> Real {
       if constexpr (F64) {
         const int ex = em[pl];
@@ -825,11 +825,12 @@ lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Re
       if (!p.owner[(size_t)e * Np + i]) continue;
       dst = out + (size_t)a0 * G + l2g[i];
     }
-#pragma unroll 4
-    for (int pl = 0; pl < na; ++pl) {
-      *dst = LEARNED ? w * value(pl) : value(pl);
-      dst += stride;
-    }
+#pragma unroll
+    for (int pl = 0; pl < S::PB; ++pl)
+      if (pl < na) {
+        *dst = LEARNED ? w * value(pl) : value(pl);
+        dst += stride;
+      }
   }
 }
 
