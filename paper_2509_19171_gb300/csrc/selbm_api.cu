@@ -79,8 +79,8 @@ struct selbm {
   int flow_learned = -1;         // whether the resident step with the learned control fits (-1: not asked)
   int flow_pass = 0;
   int *abort_host = nullptr;     // mapped host memory: a bounded wait of the resident step gave up
-  // polls of one wait of the resident step, about a microsecond each; SELBM_FLOW_SPINS in the environment sets it
-  int flow_spins = 4000000;
+  // polls of one wait of the resident step; SELBM_FLOW_SPINS in the environment lowers it
+  int flow_spins = kFlowSpins;
   int wall_max = 0;
   int n_wallpts = 0;             // wall points (element, node) over all elements
   double *d_xg = nullptr;        // [G][dim] coordinates of unique nodes (uploaded on first use)
@@ -773,7 +773,7 @@ cudaError_t run_flow2d(selbm *h, int64_t nsteps, bool probe = false) {
   a.rem_off = h->d_rem_off; a.rem = h->d_rem; a.bas_off = h->d_bas_off; a.bas = h->d_bas;
   a.rmax = h->flow_rmax; a.bmax = h->flow_bmax;
   a.abort = h->abort_host;
-  a.spins = h->flow_spins;
+  a.spin0 = kFlowSpins - h->flow_spins;
   a.T = h->d_flow_T; a.base = h->d_flow_base; a.f = (Real *)h->FA;
   const SplitHost sh = split_host(h);
   Learn2DArgs<Real> lc{};
@@ -840,7 +840,7 @@ static int create_impl(SetupFn setup, const selbm_params *params, void *cuda_str
     const char *ng = std::getenv("SELBM_NO_GRAPH");
     h->graph_enabled = !(ng && ng[0] == '1');
     const char *fs = std::getenv("SELBM_FLOW_SPINS");
-    if (fs && fs[0]) h->flow_spins = std::max(1, std::atoi(fs));
+    if (fs && fs[0]) h->flow_spins = std::min(kFlowSpins, std::max(1, std::atoi(fs)));
   }
   std::string err;
   int rc = setup(&h->S, &err);

@@ -12,7 +12,7 @@
 // knows that they have read its own of exchange k.  Copies of a shared node are summed by every CTA
 // that holds one, in ascending (element, node) order, so that all copies hold the same bits.
 //
-// Waits are bounded by p.spins polls: a wait that gives up sets *abort (host memory), and every CTA
+// Waits are bounded, by kFlowSpins - p.spin0 polls: a wait that gives up sets *abort (host memory), and every CTA
 // leaves; some may have written their share of the state, so it has to be set anew.
 #pragma once
 #include <cuda_runtime.h>
@@ -320,9 +320,9 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
   // the packet of this exchange, polled within a bound
   auto wait_packet = [&](const Packet<Real> *q) -> Real {
     Real v;
-    int spin = 0;
+    int spin = p.spin0;
     while (!get_packet(q, epoch, v)) {
-      if (++spin >= p.spins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
+      if (++spin >= kFlowSpins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
         *(volatile int *)p.abort = 1;
         s_fail = 1;
         break;
@@ -868,9 +868,9 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
           for (int k = 0; k < 2; ++k) {
             const Packet<double> *src = lc.sums + ((size_t)(pass & 1) * gridDim.x + c) * 2 + k;
             double v;
-            int spin = 0;
+            int spin = p.spin0;
             while (!get_packet(src, pass_tag, v)) {
-              if (++spin >= p.spins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
+              if (++spin >= kFlowSpins || ((spin & 4095) == 0 && *(volatile int *)p.abort != 0)) {
                 *(volatile int *)p.abort = 1;
                 s_fail = 1;
                 break;
