@@ -79,8 +79,6 @@ struct selbm {
   int flow_learned = -1;         // whether the resident step with the learned control fits (-1: not asked)
   int flow_pass = 0;
   int *abort_host = nullptr;     // mapped host memory: a bounded wait of the resident step gave up
-  // polls of one wait of the resident step; SELBM_FLOW_SPINS in the environment lowers it
-  int flow_spins = kFlowSpins;
   int wall_max = 0;
   int n_wallpts = 0;             // wall points (element, node) over all elements
   double *d_xg = nullptr;        // [G][dim] coordinates of unique nodes (uploaded on first use)
@@ -177,6 +175,10 @@ cudaError_t setup_flow2d(selbm *h) {
   if (e != cudaSuccess || !fits) return e;
   Flow2DTables t;
   if (!build_flow2d_tables(S, epc, &t)) return cudaSuccess;
+  // SELBM_FLOW_STALL=1 in the environment: one share is looked for where nobody writes (the row after the
+  // last element), so that a wait runs out
+  const char *stall = std::getenv("SELBM_FLOW_STALL");
+  if (stall && stall[0] == '1') t.rem[0] = S.E * 9 * Nb;
   a.rmax = t.rmax; a.bmax = t.bmax;
   e = launch_flow2d<Real>(S.N, S.affine, true, a, split_host(h), nullptr, &fits, h->stream);
   if (e != cudaSuccess || !fits) return e;
@@ -196,7 +198,7 @@ cudaError_t setup_flow2d(selbm *h) {
     if (r == cudaSuccess) { h->allocs.push_back(*p); r = cudaMemsetAsync(*p, 0, bytes, h->stream); }
     return r;
   };
-  if ((e = alloc(&h->d_flow_T, (size_t)4 * S.E * 9 * Nb * sizeof(Real)))) return e;
+  if ((e = alloc(&h->d_flow_T, (size_t)(4 * S.E + 2) * 9 * Nb * sizeof(Real)))) return e;
   if ((e = alloc((void **)&h->d_flow_sums, (size_t)2 * grid * 2 * 16))) return e;
   if ((e = alloc(&h->d_flow_base, (size_t)S.Gb * 20 * sizeof(Real)))) return e;
   if (!S.affine && sizeof(Real) == 8) {
@@ -773,7 +775,6 @@ cudaError_t run_flow2d(selbm *h, int64_t nsteps, bool probe = false) {
   a.rem_off = h->d_rem_off; a.rem = h->d_rem; a.bas_off = h->d_bas_off; a.bas = h->d_bas;
   a.rmax = h->flow_rmax; a.bmax = h->flow_bmax;
   a.abort = h->abort_host;
-  a.spin0 = kFlowSpins - h->flow_spins;
   a.T = h->d_flow_T; a.base = h->d_flow_base; a.f = (Real *)h->FA;
   const SplitHost sh = split_host(h);
   Learn2DArgs<Real> lc{};
@@ -839,8 +840,6 @@ static int create_impl(SetupFn setup, const selbm_params *params, void *cuda_str
     h->use_fast = !(gk && gk[0] == '1');
     const char *ng = std::getenv("SELBM_NO_GRAPH");
     h->graph_enabled = !(ng && ng[0] == '1');
-    const char *fs = std::getenv("SELBM_FLOW_SPINS");
-    if (fs && fs[0]) h->flow_spins = std::min(kFlowSpins, std::max(1, std::atoi(fs)));
   }
   std::string err;
   int rc = setup(&h->S, &err);

@@ -11,10 +11,6 @@ struct Packet {
   unsigned long long w[sizeof(Real) / 4];
 };
 
-// polls of one wait, about a microsecond each.  A launch with a lower limit starts its counts above zero:
-// a limit read in the polling loop itself made the FP32 shear layer (32 x 32, N = 8) 1.16 -> 1.34 ms a pass.
-constexpr int kFlowSpins = 4000000;
-
 template <typename Real>
 struct Flow2DArgs {
   int E, Gs, epc, nsteps;
@@ -36,7 +32,6 @@ struct Flow2DArgs {
   const int32_t *bas_off, *bas; // [CTAs + 1] shared-node indices of the owners' values a CTA fetches
   int rmax, bmax;               // most of them
   int *abort;                   // host memory: set when a wait gives up
-  int spin0;                    // polls of one wait are counted from here to kFlowSpins
   void *T;                      // [2][E][9][Nb] packets: shares
   void *base;                   // [Gb][10] packets: owner's f^0 and rho of shared nodes after a filter
   Real *f;                      // [9][Gs] state
