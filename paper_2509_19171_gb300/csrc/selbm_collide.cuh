@@ -36,13 +36,14 @@ __device__ __forceinline__ Real bgk_collide(Real (&g)[LT<LAT>::v.Q], Real rho0, 
   }
   // opposite velocities share the even part of f^eq (and F**); f + omega (f^eq - f) keeps an
   // equilibrium exactly.  The rounded weights carry momentum 3 sum t e e = 1 + delta (delta the
-  // relative rounding of t, one value for all moving classes): 3 j is formed with 1 - delta, else
-  // the velocity would drift by omega delta every step (7e-9 in FP32; a folded constant 3 t: 3e-8).
+  // relative rounding of t, one value for all moving classes): the odd part t (3 e.j) is formed with
+  // 1 - delta in the same rounding, else the velocity would drift by omega delta every step (7e-9 in
+  // FP32; a folded constant 3 t: 3e-8; 1 - delta in 3 j: its few bits round unevenly, 1e-8).
   constexpr double delta = (double)Real(V.t[1]) / V.t[1] - 1.0;
   const Real r45 = Real(4.5) * rho, base = drho - Real(1.5) * rho * uu;
   Real j3[3] = {0, 0, 0};
 #pragma unroll
-  for (int k = 0; k < DIM; ++k) j3[k] = Real(3) * j[k] - Real(3.0 * delta) * j[k];
+  for (int k = 0; k < DIM; ++k) j3[k] = Real(3) * j[k];
   static_for<0, Q>([&](auto ac) {
     constexpr int a = decltype(ac)::value, o = LT<LAT>::v.opp[a];
     if constexpr (o >= a) {
@@ -54,7 +55,8 @@ __device__ __forceinline__ Real bgk_collide(Real (&g)[LT<LAT>::v.Q], Real rho0, 
       }
       const Real t = Real(V.t[a]);
       Real even = o == a ? t * base : t * (base + (r45 * eu) * eu);
-      const Real odd = t * ej;
+      Real odd = t * ej;
+      if constexpr (delta != 0.0) odd = fma(t, ej, Real(-delta * V.t[a]) * ej);
       Real Fss = 0;
       if (has_force) {
         Fss = t * (Real(9) * eu * eF - Real(3) * uF);
