@@ -78,6 +78,7 @@ struct selbm {
   void *d_flow_T = nullptr, *d_flow_base = nullptr, *d_flow_sums = nullptr;
   int flow_learned = -1;         // whether the resident step with the learned control fits (-1: not asked)
   int flow_pass = 0;
+  bool flow_refuse = false;      // SELBM_FLOW_REFUSE=1 in the environment: launches of the resident step are refused
   int *abort_host = nullptr;     // mapped host memory: a bounded wait of the resident step gave up
   int wall_max = 0;
   int n_wallpts = 0;             // wall points (element, node) over all elements
@@ -797,7 +798,8 @@ cudaError_t run_flow2d(selbm *h, int64_t nsteps, bool probe = false) {
     a.pending = h->filter_pending;
     a.epoch = h->flow_epoch;
     lc.pass = h->flow_pass;
-    const cudaError_t e = launch_flow2d<Real>(h->S.N, h->S.affine, false, a, sh, h->learned ? &lc : nullptr, nullptr, h->stream);
+    const cudaError_t e = h->flow_refuse ? cudaErrorCooperativeLaunchTooLarge
+                                         : launch_flow2d<Real>(h->S.N, h->S.affine, false, a, sh, h->learned ? &lc : nullptr, nullptr, h->stream);
     if (e != cudaSuccess) return e;
     const int passes = h->learned ? a.nsteps - (h->filter_pending ? 0 : 1) : 0;
     h->flow_epoch += 3u * (unsigned)a.nsteps + (unsigned)passes;
@@ -840,6 +842,8 @@ static int create_impl(SetupFn setup, const selbm_params *params, void *cuda_str
     h->use_fast = !(gk && gk[0] == '1');
     const char *ng = std::getenv("SELBM_NO_GRAPH");
     h->graph_enabled = !(ng && ng[0] == '1');
+    const char *fr = std::getenv("SELBM_FLOW_REFUSE");
+    h->flow_refuse = fr && fr[0] == '1';
   }
   std::string err;
   int rc = setup(&h->S, &err);
@@ -1068,8 +1072,13 @@ int selbm_step(selbm_t *h, int64_t nsteps) {
     else run_flow2d<float>(h, 0, true);
   }
   if (h->flow_epc > 0 && !h->timing && !h->field_on && h->scheme == 0 && (!h->learned || h->flow_learned == 1)) {
+    const int64_t from = h->steps;
     const cudaError_t e = h->prec == SELBM_FP64 ? run_flow2d<double>(h, nsteps) : run_flow2d<float>(h, nsteps);
-    return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "step");
+    if (e != cudaErrorCooperativeLaunchTooLarge) return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "step");
+    // the device has fewer SMs for this context than it says: the several-kernel step from here on
+    cudaGetLastError();
+    h->flow_epc = 0;
+    nsteps -= h->steps - from;
   }
   for (int64_t k = 0; k < nsteps; ++k) {
     const bool filt = filter_waits(h);

@@ -940,9 +940,10 @@ cudaError_t launch_flow2d_t(const Flow2DArgs<Real> &p, const SplitHost &h, bool 
   auto bytes = [&](bool node) {
     return S::fixed_bytes(node) + p.epc * S::element_bytes(affine, node) + fetched + (lc ? S::learned_bytes(p.epc) : 0);
   };
+  const int grid = (p.E + p.epc - 1) / p.epc;
   if (probe) {
-    *fits = coop && (p.E + p.epc - 1) / p.epc <= sms && bytes(false) <= (size_t)most - 1024;
-    return cudaSuccess;
+    *fits = coop && bytes(false) <= (size_t)most - 1024;
+    if (!*fits) return cudaSuccess;
   }
   auto go = [&](auto ac, auto nc, auto lrn) -> cudaError_t {
     constexpr bool AFFINE = decltype(ac)::value, NODE = decltype(nc)::value, LEARNED = decltype(lrn)::value;
@@ -951,13 +952,19 @@ cudaError_t launch_flow2d_t(const Flow2DArgs<Real> &p, const SplitHost &h, bool 
     const int T = std::min(S::TMAX, 32 * std::max(4, 9 * p.epc * (NODE ? (S::Np + 31) / 32 : 1)));
     cudaError_t err = raise_smem<flow2d_kernel<Real, n, AFFINE, NODE, LEARNED>>(smem);
     if (err != cudaSuccess) return err;
+    if (probe) {
+      int ctas = 0;
+      err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, flow2d_kernel<Real, n, AFFINE, NODE, LEARNED>, T, smem);
+      *fits = err == cudaSuccess && grid <= ctas * sms;
+      return err;
+    }
     StageMats<Real, n> m = make_stage_mats<Real, n>(h);
     FilterMats<Real, n> fm = make_filter_mats<Real, n>(h);
     Flow2DArgs<Real> a = p;
     CollideFix cf = make_collide_fix<SELBM_D2Q9>((double)p.omega, (double)p.dt);
     Learn2DArgs<Real> la = lc ? *lc : Learn2DArgs<Real>{};
     void *args[] = {&a, &m, &fm, &cf, &la};
-    return cudaLaunchCooperativeKernel((const void *)flow2d_kernel<Real, n, AFFINE, NODE, LEARNED>, dim3((p.E + p.epc - 1) / p.epc),
+    return cudaLaunchCooperativeKernel((const void *)flow2d_kernel<Real, n, AFFINE, NODE, LEARNED>, dim3(grid),
                                        dim3(T), args, smem, s);
   };
   using Yes = std::true_type;

@@ -44,3 +44,25 @@ def test_mesh_beyond_the_sms(P, prec):
         f = o.step(f)
         s.step(1)
         assert rel(s.get_state(), o.to_local(f)) <= (1e-12 if prec == P.FP64 else 1e-6)
+
+
+def channel():
+    return W.box_mesh((6, 5), (0, 0), (1, 0.8), (True, False), walls={2: 1, 3: 2}, wall_velocity=[[0, 0], [0.02, 0]])
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_refused_cooperative_launch(P, monkeypatch, prec):
+    """A device that refuses the cooperative launch (here: its error code) steps in the several-kernel form."""
+    filt = {"shape": 0, "gamma": 0.1, "kc": 4.0}
+    out = []
+    for refuse in (False, True):
+        if refuse:
+            monkeypatch.setenv("SELBM_FLOW_REFUSE", "1")
+        s = P.SELBM(channel(), "D2Q9", 6, 1e-3, precision=prec, filt=filt, body_accel=(1e-4, 0.0, 0.0))
+        s.init_from(W.shear_layer_init(U0=0.02, kappa=5.0))
+        s.step(3)
+        s.step(2)
+        assert s.steps == 5
+        out.append(s.get_state())
+        s.close()
+    assert 0 < rel(out[1], out[0]) <= (1e-12 if prec == 0 else 1e-6)
