@@ -1062,6 +1062,17 @@ static void build_step_graph(selbm *h, int slot) {
   }
 }
 
+// whether the caller captures the handle's stream: a replayed resident step would find the exchange
+// numbers of its first run
+static bool capturing(selbm *h) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st != cudaStreamCaptureStatusNone;
+}
+
 int selbm_step(selbm_t *h, int64_t nsteps) {
   if (!h) return SELBM_ERR_ARG;
   if (!h->initialized) return h->fail(SELBM_ERR_STATE, "state not initialised");
@@ -1071,7 +1082,7 @@ int selbm_step(selbm_t *h, int64_t nsteps) {
     if (h->prec == SELBM_FP64) run_flow2d<double>(h, 0, true);
     else run_flow2d<float>(h, 0, true);
   }
-  if (h->flow_epc > 0 && !h->timing && !h->field_on && h->scheme == 0 && (!h->learned || h->flow_learned == 1)) {
+  if (h->flow_epc > 0 && !h->timing && !h->field_on && h->scheme == 0 && (!h->learned || h->flow_learned == 1) && !capturing(h)) {
     const int64_t from = h->steps;
     const cudaError_t e = h->prec == SELBM_FP64 ? run_flow2d<double>(h, nsteps) : run_flow2d<float>(h, nsteps);
     if (e != cudaErrorCooperativeLaunchTooLarge) return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "step");

@@ -66,3 +66,31 @@ def test_refused_cooperative_launch(P, monkeypatch, prec):
         out.append(s.get_state())
         s.close()
     assert 0 < rel(out[1], out[0]) <= (1e-12 if prec == 0 else 1e-6)
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+def test_captured_by_the_caller(P, monkeypatch, prec):
+    """Steps that the caller captures into a graph of its own and replays."""
+    import torch
+    monkeypatch.setenv("SELBM_NO_GRAPH", "1")
+    filt = {"shape": 0, "gamma": 0.1, "kc": 4.0}
+    stream = torch.cuda.Stream()
+    a, b = (P.SELBM(channel(), "D2Q9", 6, 1e-3, precision=prec, filt=filt, stream=stream.cuda_stream) for _ in range(2))
+    for s in (a, b):
+        s.timers(True)                                    # the kernels of the several-kernel form are loaded
+        s.init_from(W.shear_layer_init(U0=0.02, kappa=5.0))
+        s.step(2)
+        s.timers(False)
+        s.step(2)
+        s.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream):
+        a.step(3)
+    with torch.cuda.stream(stream):
+        for _ in range(3):
+            g.replay()
+    b.step(9)
+    assert rel(a.get_state(), b.get_state()) <= 9 * (1e-12 if prec == 0 else 1e-6)
+    a.step(2)                                             # the resident step goes on from there
+    b.step(2)
+    assert rel(a.get_state(), b.get_state()) <= 11 * (1e-12 if prec == 0 else 1e-6)
