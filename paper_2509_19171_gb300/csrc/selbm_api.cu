@@ -30,7 +30,10 @@ cudaError_t upload(T **dst, const std::vector<T> &src) {
   if (src.empty()) return cudaSuccess;
   cudaError_t e = cudaMalloc((void **)dst, src.size() * sizeof(T));
   if (e != cudaSuccess) return e;
-  return cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
+  // a copy from pageable memory may still be under way when cudaMemcpy returns, and a handle's stream may
+  // be one that does not wait for the default stream
+  e = cudaMemcpy(*dst, src.data(), src.size() * sizeof(T), cudaMemcpyHostToDevice);
+  return e == cudaSuccess ? cudaStreamSynchronize(cudaStreamLegacy) : e;
 }
 
 template <typename R>
@@ -695,6 +698,7 @@ int set_filter_internal(selbm *h, const selbm_filter &f) {
       std::vector<float> sg(h->sigma.begin(), h->sigma.end());
       e = cudaMemcpy(h->d_fixsig, sg.data(), sg.size() * 4, cudaMemcpyHostToDevice);
     }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // see upload()
   }
   if (e != cudaSuccess) return h->cuda_fail(e, "set_filter");
   return SELBM_OK;
@@ -1543,6 +1547,7 @@ int selbm_element_errors(selbm_t *h, selbm_t *ref, double *err) {
   if (e == cudaSuccess) e = cudaMalloc((void **)&wq, nl * sizeof(double));
   if (e == cudaSuccess) e = cudaMemcpy(I, Ih.data(), Ih.size() * sizeof(double), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy(wq, h->S.wJ.data(), nl * sizeof(double), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);   // see upload()
   int rc = SELBM_OK;
   if (e == cudaSuccess) {
     double *rho = buf, *u = buf + nl, *rhoR = buf + nl * (1 + dim), *uR = rhoR + nlr;
