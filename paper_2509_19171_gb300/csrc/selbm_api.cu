@@ -57,9 +57,10 @@ struct selbm {
   // any-order element kernels of the split step: hexahedra where the fused kernels are not
   // compiled, and every FP64 order
   bool use_lines = false;
-  void *d_geo = nullptr, *d_w3 = nullptr;   // metrics of the split-form kernels (CurvedGeo)
+  void *d_geo = nullptr, *d_w3 = nullptr;   // affine FP64: coefficients and weights of the any-order kernels (LineGeo)
   int *d_gexp = nullptr;
   bool split_form() const { return use_split || use_lines; }
+  MetricLayout metrics() const { return S.affine ? kMetricsAffine : split_form() ? kMetricsByComponent : kMetricsByNode; }
   bool lines_step() const { return use_lines && !(use_split && prec == SELBM_FP32DEV); }
   std::vector<double> Vm_h, Vinv_h;   // modal <-> nodal matrices
   // learned per-element filter control
@@ -263,12 +264,29 @@ cudaError_t upload_real(selbm *h) {
       }
     }
   } else {
-    if ((e = upload(&p, cast_vec<Real>(S.drdx)))) return e; h->d_drdx = p; h->allocs.push_back(p);
+    std::vector<Real> m(S.drdx.size());
+    std::vector<int> top;
+    if (h->metrics() == kMetricsByComponent) {
+      // and the largest biased exponent of an element's metrics (FP64 lines)
+      top.assign(S.E, 1);
+      for (size_t el = 0; el < (size_t)S.E; ++el) {
+        double mx = 0;
+        for (int i = 0; i < S.Np; ++i)
+          for (int c = 0; c < 9; ++c) {
+            const double v = S.drdx[(el * S.Np + i) * 9 + c];
+            m[(el * 9 + c) * S.Np + i] = (Real)v;
+            mx = std::max(mx, std::fabs(v));
+          }
+        if (mx > 0) top[el] = std::max(1, std::ilogb(mx) + 1023);
+      }
+    } else {
+      m.assign(S.drdx.begin(), S.drdx.end());
+    }
+    if ((e = upload(&p, m))) return e; h->d_drdx = p; h->allocs.push_back(p);
     if ((e = upload(&p, cast_vec<Real>(S.wJ)))) return e; h->d_wJ = p; h->allocs.push_back(p);
-    if (h->split_form()) {
-      if ((e = alloc(&h->d_geo, (size_t)S.E * S.Np * 9 * sizeof(LineVal<Real>)))) return e;
-      if ((e = alloc((void **)&h->d_gexp, (size_t)S.E * sizeof(int)))) return e;
-      if ((e = launch_curved_geo<Real>((const Real *)h->d_drdx, S.E, S.Np, (LineVal<Real> *)h->d_geo, h->d_gexp, h->stream))) return e;
+    if (!top.empty()) {
+      int *q;
+      if ((e = upload(&q, top))) return e; h->d_gexp = q; h->allocs.push_back(q);
     }
   }
   if ((e = upload(&p, cast_vec<Real>(S.gll.w)))) return e; h->d_gllw = p; h->allocs.push_back(p);
@@ -410,15 +428,13 @@ template <typename Real>
 cudaError_t launch_split_stage(selbm *h, const KParams<Real> &p) {
   const SplitHost sh = split_host(h);
   if (h->lines_step()) {
-    const CurvedGeo<Real> cg{(const LineVal<Real> *)h->d_geo, h->d_gexp, (const Real *)h->d_w3};
-    return launch_lines_stage<Real>(h->lat, h->S.N, h->S.affine, p, sh, cg, h->stream);
+    const LineGeo<Real> lg{(const LineVal<Real> *)h->d_geo, h->d_gexp, (const Real *)h->d_w3};
+    return launch_lines_stage<Real>(h->lat, h->S.N, h->S.affine, p, sh, lg, h->stream);
   }
   cudaError_t err = cudaErrorInvalidValue;
   if constexpr (std::is_same<Real, float>::value) {
-    KParams<Real> q = p;
-    q.drdx = (const Real *)h->d_geo;        // metrics by component
-    if (h->lat == SELBM_D3Q19) split_stage_d3q19<Real>(h->S.N, h->S.affine, q, sh, h->stream, &err);
-    else if (h->lat == SELBM_D3Q27) split_stage_d3q27<Real>(h->S.N, h->S.affine, q, sh, h->stream, &err);
+    if (h->lat == SELBM_D3Q19) split_stage_d3q19<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
+    else if (h->lat == SELBM_D3Q27) split_stage_d3q27<Real>(h->S.N, h->S.affine, p, sh, h->stream, &err);
   }
   return err;
 }
@@ -1270,10 +1286,10 @@ int selbm_diagnostics(selbm_t *h, double out[8]) {
   if (e == cudaSuccess) {
     const double mu = h->P.rho0 * h->P.nu;
     e = h->prec == SELBM_FP64
-            ? launch_eps<double>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const double *)h->d_el_drdx,
+            ? launch_eps<double>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->metrics(), (const double *)h->d_el_drdx,
                                  (const double *)h->d_drdx, (const double *)h->d_el_J, (const double *)h->d_wJ,
                                  (const double *)h->d_gllw, (const double *)h->d_D, mu, part, d_eps, h->stream)
-            : launch_eps<float>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const float *)h->d_el_drdx,
+            : launch_eps<float>(u_l, (int)dim, h->S.n1, h->S.Np, h->S.E, h->metrics(), (const float *)h->d_el_drdx,
                                 (const float *)h->d_drdx, (const float *)h->d_el_J, (const float *)h->d_wJ,
                                 (const float *)h->d_gllw, (const float *)h->d_D, mu, part, d_eps, h->stream);
   }
@@ -1309,10 +1325,10 @@ int selbm_wall_stress(selbm_t *h, const double dir[3], double *tau) {
   cudaError_t e = launch_expand_fields(dim, h->d_fld, h->S.G, h->d_l2g, nl, nullptr, u_l, h->stream);
   if (e == cudaSuccess)
     e = h->prec == SELBM_FP64
-            ? launch_wall_stress<double>(u_l, dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const double *)h->d_el_drdx,
+            ? launch_wall_stress<double>(u_l, dim, h->S.n1, h->S.Np, h->S.E, h->metrics(), (const double *)h->d_el_drdx,
                                          (const double *)h->d_drdx, (const double *)h->d_D, h->d_walls, h->d_wall_off, d,
                                          mu, part, h->stream)
-            : launch_wall_stress<float>(u_l, dim, h->S.n1, h->S.Np, h->S.E, h->S.affine, (const float *)h->d_el_drdx,
+            : launch_wall_stress<float>(u_l, dim, h->S.n1, h->S.Np, h->S.E, h->metrics(), (const float *)h->d_el_drdx,
                                         (const float *)h->d_drdx, (const float *)h->d_D, h->d_walls, h->d_wall_off, d,
                                         mu, part, h->stream);
   std::vector<double> hp(2 * (size_t)h->n_wallpts);

@@ -497,7 +497,7 @@ __global__ void stress_kernel(const Real *buf, const int32_t *l2g, int G, int Gs
 // gradients by D_hat along each reference axis and the chain rule; one CTA per element,
 // per-element sums into partial[e] (summed in element order afterwards)
 template <typename Real>
-__global__ void eps_kernel(const double *u, int dim, int n, int Np, int affine, const Real *el_drdx, const Real *drdx,
+__global__ void eps_kernel(const double *u, int dim, int n, int Np, int layout, const Real *el_drdx, const Real *drdx,
                            const Real *el_J, const Real *wJ, const Real *gllw, const Real *Dm, double mu,
                            double *partial) {
   __shared__ double red[256];
@@ -519,9 +519,7 @@ __global__ void eps_kernel(const double *u, int dim, int n, int Np, int affine, 
       for (int c = 0; c < dim; ++c) {
         double s = 0.0;
         for (int l = 0; l < dim; ++l) {
-          const double m = affine ? (double)el_drdx[((size_t)e * dim + l) * dim + k]
-                                  : (double)drdx[(((size_t)e * Np + i) * dim + l) * dim + k];
-          s += m * dr[l][c];
+          s += metric_of(layout, el_drdx, drdx, e, Np, i, dim, l, k) * dr[l][c];
         }
         g[k][c] = s;
       }
@@ -531,7 +529,7 @@ __global__ void eps_kernel(const double *u, int dim, int n, int Np, int affine, 
       for (int b = a + 1; b < dim; ++b) off += (g[a][b] + g[b][a]) * (g[a][b] + g[b][a]);
     const double dens = 2.0 * mu * diag - (2.0 / 3.0) * mu * div * div + mu * off;
     double w;
-    if (affine) {
+    if (layout == kMetricsAffine) {
       w = (double)el_J[e] * (double)gllw[ii[0]] * (double)gllw[ii[1]] * (dim == 3 ? (double)gllw[ii[2]] : 1.0);
     } else {
       w = (double)wJ[(size_t)e * Np + i];
@@ -561,10 +559,10 @@ __global__ void sum_kernel(const double *partial, int count, double *out) {
 }
 
 template <typename Real>
-cudaError_t launch_eps(const double *u, int dim, int n, int Np, int E, int affine, const Real *el_drdx, const Real *drdx,
+cudaError_t launch_eps(const double *u, int dim, int n, int Np, int E, int layout, const Real *el_drdx, const Real *drdx,
                        const Real *el_J, const Real *wJ, const Real *gllw, const Real *Dm, double mu, double *partial,
                        double *out, cudaStream_t s) {
-  eps_kernel<Real><<<E, 256, 0, s>>>(u, dim, n, Np, affine, el_drdx, drdx, el_J, wJ, gllw, Dm, mu, partial);
+  eps_kernel<Real><<<E, 256, 0, s>>>(u, dim, n, Np, layout, el_drdx, drdx, el_J, wJ, gllw, Dm, mu, partial);
   sum_kernel<<<1, 256, 0, s>>>(partial, E, out);
   return cudaGetLastError();
 }

@@ -33,7 +33,7 @@ struct KParams {
   const int32_t *bslot;      // [Np] boundary slot of each local node, -1 inside
   const Real *el_drdx;       // [E][dim][dim] affine metrics
   const Real *el_J;          // [E]
-  const Real *drdx;          // [E][Np][dim][dim] general metrics
+  const Real *drdx;          // general metrics: [E][Np][dim][dim], split form [E][9][Np] (component 3 l + k)
   const Real *wJ;            // [E][Np]
   const Real *gllw;          // [n]
   const Real *Dm, *Fm;       // [n][n]
@@ -171,9 +171,19 @@ inline bool split_compiled(int lat, int N) {
   return (lat == SELBM_D3Q19 && (N == 4 || N == 7)) || (lat == SELBM_D3Q27 && (N == 5 || N == 7));
 }
 
+// where a handle holds dr_l/dx_k: per element, per node, or per node by component (hexahedra in the split form)
+enum MetricLayout { kMetricsByNode = 0, kMetricsAffine = 1, kMetricsByComponent = 2 };
+template <typename Real>
+__device__ __forceinline__ double metric_of(int layout, const Real *el_drdx, const Real *drdx, int e, int Np, int i, int dim, int l,
+                                            int k) {
+  const int c = l * dim + k, d2 = dim * dim;
+  return layout == kMetricsAffine ? (double)el_drdx[(size_t)e * d2 + c]
+                                  : (double)drdx[layout == kMetricsByNode ? ((size_t)e * Np + i) * d2 + c : ((size_t)e * d2 + c) * Np + i];
+}
+
 // pipe statistics (selbm_stats.cu)
 template <typename Real>
-cudaError_t launch_wall_stress(const double *u, int dim, int n, int Np, int E, int affine, const Real *el_drdx,
+cudaError_t launch_wall_stress(const double *u, int dim, int n, int Np, int E, int layout, const Real *el_drdx,
                                const Real *drdx, const Real *Dm, const void *walls, const int32_t *wall_off,
                                const double dir[3], double mu, double *out, cudaStream_t s);
 cudaError_t launch_radial_profile(const double *u, int dim, const double *xg, const double *mass, int G,
@@ -181,7 +191,7 @@ cudaError_t launch_radial_profile(const double *u, int dim, const double *xg, co
                                   int blocks, double *partial, cudaStream_t s);
 
 template <typename Real>
-cudaError_t launch_eps(const double *u, int dim, int n, int Np, int E, int affine, const Real *el_drdx, const Real *drdx,
+cudaError_t launch_eps(const double *u, int dim, int n, int Np, int E, int layout, const Real *el_drdx, const Real *drdx,
                        const Real *el_J, const Real *wJ, const Real *gllw, const Real *Dm, double mu, double *partial,
                        double *out, cudaStream_t s);
 

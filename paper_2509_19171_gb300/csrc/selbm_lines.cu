@@ -7,9 +7,9 @@ namespace slb {
 
 template <typename Real>
 cudaError_t launch_lines_stage(int lat, int N, bool affine, const KParams<Real> &p, const SplitHost &h,
-                               const CurvedGeo<Real> &cg, cudaStream_t s) {
+                               const LineGeo<Real> &lg, cudaStream_t s) {
   const LatticeRT lt = lat == SELBM_D3Q19 ? lattice_rt<SELBM_D3Q19>() : lattice_rt<SELBM_D3Q27>();
-  return N <= 6 ? lines_stage_part<Real, 0>(N, affine, p, h, lt, cg, s) : lines_stage_part<Real, 1>(N, affine, p, h, lt, cg, s);
+  return N <= 6 ? lines_stage_part<Real, 0>(N, affine, p, h, lt, lg, s) : lines_stage_part<Real, 1>(N, affine, p, h, lt, lg, s);
 }
 
 template <typename Real>
@@ -17,12 +17,6 @@ cudaError_t launch_lines_filter(int lat, int N, const KParams<Real> &p, const Sp
                                 cudaStream_t s) {
   const int Q = lat == SELBM_D3Q19 ? LT<SELBM_D3Q19>::v.Q : LT<SELBM_D3Q27>::v.Q;
   return N <= 6 ? lines_filter_part<Real, 0>(N, p, h, Q, sigma, out, s) : lines_filter_part<Real, 1>(N, p, h, Q, sigma, out, s);
-}
-
-template <typename Real>
-cudaError_t launch_curved_geo(const Real *drdx, int E, int Np, LineVal<Real> *g, int *gexp, cudaStream_t s) {
-  curved_geo_kernel<Real><<<E, 256, 0, s>>>(drdx, Np, g, gexp);
-  return cudaGetLastError();
 }
 
 // affine elements, FP64: -dt sum_k e_k dr_l/dx_k in fixed point, c [E][Q][3] times 2^cexp[E][Q]
@@ -61,10 +55,9 @@ cudaError_t launch_flow2d(int N, bool affine, bool probe, const Flow2DArgs<Real>
 
 #define SLB_INST(Real)                                                                                                    \
   template cudaError_t launch_lines_stage<Real>(int, int, bool, const KParams<Real> &, const SplitHost &,                 \
-                                                const CurvedGeo<Real> &, cudaStream_t);                                   \
+                                                const LineGeo<Real> &, cudaStream_t);                                   \
   template cudaError_t launch_lines_filter<Real>(int, int, const KParams<Real> &, const SplitHost &, const Real *, Real *, \
                                                  cudaStream_t);                                                          \
-  template cudaError_t launch_curved_geo<Real>(const Real *, int, int, LineVal<Real> *, int *, cudaStream_t);             \
   template cudaError_t launch_flow2d<Real>(int, bool, bool, const Flow2DArgs<Real> &, const SplitHost &,              \
                                              const Learn2DArgs<Real> *, bool *, cudaStream_t);
 SLB_INST(float)

@@ -383,6 +383,7 @@ __device__ __noinline__ double slow_deriv(const double *D, const long long *row,
 // ---------------------------------------------------------------------------
 // advection stage
 // ---------------------------------------------------------------------------
+constexpr int kMetricShift = 5;
 template <typename Real, int n, bool AFFINE>
 constexpr size_t lines_stage_smem(int pb, int wall_max) {
   using S = LineShape<Real, n>;
@@ -395,7 +396,7 @@ constexpr size_t lines_stage_smem(int pb, int wall_max) {
 
 template <typename Real, int n, bool AFFINE>
 __global__ void __launch_bounds__(LineShape<Real, n>::T, LineShape<Real, n>::F64 ? 3 : (n <= 8 ? 5 : 3))
-lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const LatticeRT lt, const CurvedGeo<Real> cg,
+lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const LatticeRT lt, const LineGeo<Real> lg,
                    const int pb, const int ng) {
   using S = LineShape<Real, n>;
   using Val = LineVal<Real>;
@@ -427,10 +428,10 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
     if constexpr (AFFINE && F64) {
       // -dt sum_k e_k dr_l/dx_k in fixed point from the table, times B
       const size_t row = (size_t)e * lt.Q + a0 + tid;
-      ge[tid] = cg.gexp[row];
+      ge[tid] = lg.gexp[row];
 #pragma unroll
       for (int l = 0; l < 3; ++l) {
-        const long long c = cg.g[row * 3 + l];
+        const long long c = lg.g[row * 3 + l];
         Fix128 t{0, 1ll << 29};
         fix_mac(t, m.B, limbs(c));
         cf[tid * 3 + l] = fix_top<2>(t);
@@ -460,7 +461,7 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
   }
   if constexpr (F64 && AFFINE) {
     const double J = p.el_J[e];
-    for (int i = tid; i < Np; i += T) sw[i] = J * cg.w3[i];
+    for (int i = tid; i < Np; i += T) sw[i] = J * lg.w3[i];
   }
   if (F64) __syncthreads();                            // em
   gather_lines<Real, n, SHIFT>(tile, em, p.fin + (size_t)a0 * G, G, l2g, na, tid);
@@ -469,11 +470,17 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
   auto stage_metrics = [&](int l) {
     if constexpr (!AFFINE) {
       __syncthreads();
-      const Val *src = cg.g + ((size_t)e * 9 + 3 * l) * Np;
+      const Real *src = p.drdx + ((size_t)e * 9 + 3 * l) * Np;
+      const int top = F64 ? lg.gexp[e] : 0;
       for (int i = tid; i < Np; i += T) {
         const int o = tile_offset<Real, n>(i);
 #pragma unroll
-        for (int k = 0; k < 3; ++k) sg[k * PS + o] = src[(size_t)k * Np + i];
+        for (int k = 0; k < 3; ++k) {
+          const Real v = __ldg(src + (size_t)k * Np + i);
+          // fixed point: magnitudes below 2^58, three of them below 2^60
+          if constexpr (F64) sg[k * PS + o] = to_fixed_rn<kMetricShift>(v, top);
+          else sg[k * PS + o] = v;
+        }
       }
       __syncthreads();
     }
@@ -528,8 +535,8 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
       } else {
         const int off = base + j * st;
         const int i = off % S::LS + n * ((off / S::LS) % n) + n * n * (off / S::PLN);
-        const double *gm = p.drdx + ((size_t)e * Np + i) * 9 + 3 * ax;
-        for (int k = 0; k < 3; ++k) c += sgn(k, a0 + pl) * gm[k];
+        const double *gm = p.drdx + ((size_t)e * 9 + 3 * ax) * Np + i;
+        for (int k = 0; k < 3; ++k) c += sgn(k, a0 + pl) * gm[k * Np];
       }
       return c * slow_deriv<n>(m.D, tile + pl * PS + base, st, j);
     } else return 0.0;
@@ -636,7 +643,7 @@ lines_stage_kernel(const KParams<Real> p, const StageMats<Real, n> m, const Latt
     // value of a sum: curved elements carry -B dt here
     int ex = 0;
     if constexpr (F64) {
-      const int gs = AFFINE ? ge[pl] : cg.gexp[e];
+      const int gs = AFFINE ? ge[pl] : 1023 + 52 + kMetricShift - lg.gexp[e];
       ex = 125 - gs - m.cb + em[pl] - FixScale<n>::EXP0;
     }
     auto value = [&](Val x) -> Real {
@@ -834,34 +841,6 @@ lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Re
   }
 }
 
-// planar copy of the metrics of curved elements, component-major inside an element
-template <typename Real>
-__global__ void __launch_bounds__(256) curved_geo_kernel(const Real *drdx, int Np, LineVal<Real> *g, int *gexp) {
-  const int e = blockIdx.x;
-  const Real *src = drdx + (size_t)e * Np * 9;
-  LineVal<Real> *dst = g + (size_t)e * Np * 9;
-  if constexpr (sizeof(Real) == 8) {
-    __shared__ int emax;
-    if (threadIdx.x == 0) emax = 1;
-    __syncthreads();
-    int ex = 1;
-    for (int i = threadIdx.x; i < 9 * Np; i += blockDim.x) ex = max(ex, exp_of(src[i]));
-    atomicMax(&emax, ex);
-    __syncthreads();
-    const int sh = 1080 - emax;                          // magnitudes below 2^58, three of them below 2^60
-    if (threadIdx.x == 0) gexp[e] = sh;
-    for (int i = threadIdx.x; i < 9 * Np; i += blockDim.x) {
-      const int node = i / 9, c = i - node * 9;
-      dst[(size_t)c * Np + node] = __double2ll_rn(scalbn(src[i], sh));
-    }
-  } else {
-    for (int i = threadIdx.x; i < 9 * Np; i += blockDim.x) {
-      const int node = i / 9, c = i - node * 9;
-      dst[(size_t)c * Np + node] = src[i];
-    }
-  }
-}
-
 // ---------------------------------------------------------------------------
 // launchers
 // ---------------------------------------------------------------------------
@@ -874,7 +853,7 @@ void line_groups(int Q, int *pb, int *ng) {
 
 template <typename Real, int n>
 cudaError_t launch_lines_stage_t(bool affine, const KParams<Real> &p, const SplitHost &h, const LatticeRT &lt,
-                                 const CurvedGeo<Real> &cg, cudaStream_t s) {
+                                 const LineGeo<Real> &lg, cudaStream_t s) {
   int pb, ng;
   line_groups<Real, n>(lt.Q, &pb, &ng);
   StageMats<Real, n> m = make_stage_mats<Real, n>(h);
@@ -885,7 +864,7 @@ cudaError_t launch_lines_stage_t(bool affine, const KParams<Real> &p, const Spli
     const size_t smem = lines_stage_smem<Real, n, AFFINE>(pb, p.wall_max);
     const cudaError_t err = raise_smem<lines_stage_kernel<Real, n, AFFINE>>(smem);
     if (err != cudaSuccess) return err;
-    lines_stage_kernel<Real, n, AFFINE><<<p.E * ng, LineShape<Real, n>::T, smem, s>>>(p, m, lt, cg, pb, ng);
+    lines_stage_kernel<Real, n, AFFINE><<<p.E * ng, LineShape<Real, n>::T, smem, s>>>(p, m, lt, lg, pb, ng);
     return cudaGetLastError();
   };
   return affine ? go(std::true_type{}) : go(std::false_type{});
@@ -911,7 +890,7 @@ cudaError_t launch_lines_filter_t(const KParams<Real> &p, const SplitHost &h, in
 // translation units by order: part 0 N <= 6, part 1 above
 template <typename Real, int PART>
 cudaError_t lines_stage_part(int N, bool affine, const KParams<Real> &p, const SplitHost &h, const LatticeRT &lt,
-                             const CurvedGeo<Real> &cg, cudaStream_t s);
+                             const LineGeo<Real> &lg, cudaStream_t s);
 template <typename Real, int PART>
 cudaError_t lines_filter_part(int N, const KParams<Real> &p, const SplitHost &h, int Q, const Real *sigma, Real *out,
                               cudaStream_t s);

@@ -23,11 +23,11 @@ struct LatticeRT {
   }
 };
 
-// metrics of the stage kernel.  Curved elements: dr_l/dx_k [E][9][Np] (component 3 l + k); FP64: fixed
-// point, times 2^gexp[e].  Affine elements, FP64: -dt sum_k e_k dr_l/dx_k [E][Q][3] in fixed point,
-// times 2^gexp[e Q + a], and the quadrature weights w w w [Np].
+// tables of the stage kernel beside the metrics.  Affine elements, FP64: -dt sum_k e_k dr_l/dx_k [E][Q][3] in fixed
+// point, times 2^gexp[e Q + a], and the quadrature weights w w w [Np].  Curved elements, FP64: gexp[e], the
+// largest biased exponent of the element's metrics.
 template <typename Real>
-struct CurvedGeo {
+struct LineGeo {
   const LineVal<Real> *g;
   const int *gexp;
   const Real *w3;
@@ -39,16 +39,12 @@ inline bool lines_compiled(int real_size, int N) { return N >= 2 && N <= (real_s
 // one Runge-Kutta stage of the element kernels (see selbm_split_stage.cuh for its terms)
 template <typename Real>
 cudaError_t launch_lines_stage(int lat, int N, bool affine, const KParams<Real> &p, const SplitHost &h,
-                               const CurvedGeo<Real> &cg, cudaStream_t s);
+                               const LineGeo<Real> &lg, cudaStream_t s);
 // filtered p.fin: sigma NULL: the fixed filter, every unique node to out; else element transfer
 // functions sigma [E][n], element-interior nodes to out and shares wJ f of the others to p.T
 template <typename Real>
 cudaError_t launch_lines_filter(int lat, int N, const KParams<Real> &p, const SplitHost &h, const Real *sigma, Real *out,
                                 cudaStream_t s);
-// planar metrics from drdx [E][Np][9]
-template <typename Real>
-cudaError_t launch_curved_geo(const Real *drdx, int E, int Np, LineVal<Real> *g, int *gexp, cudaStream_t s);
-
 // the affine FP64 tables from el_drdx [E][3][3]
 cudaError_t launch_affine_geo(int lat, const double *el_drdx, int E, double dt, long long *c, int *cexp, cudaStream_t s);
 

@@ -5,13 +5,13 @@ namespace slb {
 
 template <>
 cudaError_t lines_stage_part<float, 0>(int N, bool affine, const KParams<float> &p, const SplitHost &h, const LatticeRT &lt,
-                                          const CurvedGeo<float> &cg, cudaStream_t s) {
+                                          const LineGeo<float> &lg, cudaStream_t s) {
   switch (N) {
-    case 2: return launch_lines_stage_t<float, 3>(affine, p, h, lt, cg, s);
-    case 3: return launch_lines_stage_t<float, 4>(affine, p, h, lt, cg, s);
-    case 4: return launch_lines_stage_t<float, 5>(affine, p, h, lt, cg, s);
-    case 5: return launch_lines_stage_t<float, 6>(affine, p, h, lt, cg, s);
-    case 6: return launch_lines_stage_t<float, 7>(affine, p, h, lt, cg, s);
+    case 2: return launch_lines_stage_t<float, 3>(affine, p, h, lt, lg, s);
+    case 3: return launch_lines_stage_t<float, 4>(affine, p, h, lt, lg, s);
+    case 4: return launch_lines_stage_t<float, 5>(affine, p, h, lt, lg, s);
+    case 5: return launch_lines_stage_t<float, 6>(affine, p, h, lt, lg, s);
+    case 6: return launch_lines_stage_t<float, 7>(affine, p, h, lt, lg, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -5,13 +5,13 @@ namespace slb {
 
 template <>
 cudaError_t lines_stage_part<float, 1>(int N, bool affine, const KParams<float> &p, const SplitHost &h, const LatticeRT &lt,
-                                          const CurvedGeo<float> &cg, cudaStream_t s) {
+                                          const LineGeo<float> &lg, cudaStream_t s) {
   switch (N) {
-    case 7: return launch_lines_stage_t<float, 8>(affine, p, h, lt, cg, s);
-    case 8: return launch_lines_stage_t<float, 9>(affine, p, h, lt, cg, s);
-    case 9: return launch_lines_stage_t<float, 10>(affine, p, h, lt, cg, s);
-    case 10: return launch_lines_stage_t<float, 11>(affine, p, h, lt, cg, s);
-    case 11: return launch_lines_stage_t<float, 12>(affine, p, h, lt, cg, s);
+    case 7: return launch_lines_stage_t<float, 8>(affine, p, h, lt, lg, s);
+    case 8: return launch_lines_stage_t<float, 9>(affine, p, h, lt, lg, s);
+    case 9: return launch_lines_stage_t<float, 10>(affine, p, h, lt, lg, s);
+    case 10: return launch_lines_stage_t<float, 11>(affine, p, h, lt, lg, s);
+    case 11: return launch_lines_stage_t<float, 12>(affine, p, h, lt, lg, s);
   }
   return cudaErrorInvalidValue;
 }

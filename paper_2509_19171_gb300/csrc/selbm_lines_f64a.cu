@@ -5,13 +5,13 @@ namespace slb {
 
 template <>
 cudaError_t lines_stage_part<double, 0>(int N, bool affine, const KParams<double> &p, const SplitHost &h, const LatticeRT &lt,
-                                          const CurvedGeo<double> &cg, cudaStream_t s) {
+                                          const LineGeo<double> &lg, cudaStream_t s) {
   switch (N) {
-    case 2: return launch_lines_stage_t<double, 3>(affine, p, h, lt, cg, s);
-    case 3: return launch_lines_stage_t<double, 4>(affine, p, h, lt, cg, s);
-    case 4: return launch_lines_stage_t<double, 5>(affine, p, h, lt, cg, s);
-    case 5: return launch_lines_stage_t<double, 6>(affine, p, h, lt, cg, s);
-    case 6: return launch_lines_stage_t<double, 7>(affine, p, h, lt, cg, s);
+    case 2: return launch_lines_stage_t<double, 3>(affine, p, h, lt, lg, s);
+    case 3: return launch_lines_stage_t<double, 4>(affine, p, h, lt, lg, s);
+    case 4: return launch_lines_stage_t<double, 5>(affine, p, h, lt, lg, s);
+    case 5: return launch_lines_stage_t<double, 6>(affine, p, h, lt, lg, s);
+    case 6: return launch_lines_stage_t<double, 7>(affine, p, h, lt, lg, s);
   }
   return cudaErrorInvalidValue;
 }

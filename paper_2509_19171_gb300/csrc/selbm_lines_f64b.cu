@@ -5,11 +5,11 @@ namespace slb {
 
 template <>
 cudaError_t lines_stage_part<double, 1>(int N, bool affine, const KParams<double> &p, const SplitHost &h, const LatticeRT &lt,
-                                          const CurvedGeo<double> &cg, cudaStream_t s) {
+                                          const LineGeo<double> &lg, cudaStream_t s) {
   switch (N) {
-    case 7: return launch_lines_stage_t<double, 8>(affine, p, h, lt, cg, s);
-    case 8: return launch_lines_stage_t<double, 9>(affine, p, h, lt, cg, s);
-    case 9: return launch_lines_stage_t<double, 10>(affine, p, h, lt, cg, s);
+    case 7: return launch_lines_stage_t<double, 8>(affine, p, h, lt, lg, s);
+    case 8: return launch_lines_stage_t<double, 9>(affine, p, h, lt, lg, s);
+    case 9: return launch_lines_stage_t<double, 10>(affine, p, h, lt, lg, s);
   }
   return cudaErrorInvalidValue;
 }

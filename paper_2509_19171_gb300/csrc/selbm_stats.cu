@@ -11,7 +11,7 @@ namespace slb {
 // the node from the GLL derivative along every reference axis and the chain rule, then
 // for every wall face through the node w_s J_s (-mu n.grad(u.d)) and w_s J_s
 template <typename Real>
-__global__ void wall_stress_kernel(const double *u, int dim, int n, int Np, int affine, const Real *el_drdx,
+__global__ void wall_stress_kernel(const double *u, int dim, int n, int Np, int layout, const Real *el_drdx,
                                    const Real *drdx, const Real *Dm, const WallPt<Real> *walls, const int32_t *wall_off,
                                    double d0, double d1, double d2, double mu, double *out) {
   const int e = blockIdx.x;
@@ -36,11 +36,8 @@ __global__ void wall_stress_kernel(const double *u, int dim, int n, int Np, int 
     }
     double grad[3] = {0, 0, 0};
     for (int c = 0; c < dim; ++c)
-      for (int l = 0; l < dim; ++l) {
-        const double g = affine ? (double)el_drdx[((size_t)e * dim + l) * dim + c]
-                                : (double)drdx[(((size_t)e * Np + i) * dim + l) * dim + c];
-        grad[c] += g * dr[l];
-      }
+      for (int l = 0; l < dim; ++l)
+        grad[c] += metric_of(layout, el_drdx, drdx, e, Np, i, dim, l, c) * dr[l];
     double num = 0, den = 0;
     for (int f = 0; f < wp.nf; ++f) {
       double dn = 0;
@@ -85,10 +82,10 @@ __global__ void radial_profile_kernel(const double *u, int dim, const double *xg
 }
 
 template <typename Real>
-cudaError_t launch_wall_stress(const double *u, int dim, int n, int Np, int E, int affine, const Real *el_drdx,
+cudaError_t launch_wall_stress(const double *u, int dim, int n, int Np, int E, int layout, const Real *el_drdx,
                                const Real *drdx, const Real *Dm, const void *walls, const int32_t *wall_off,
                                const double dir[3], double mu, double *out, cudaStream_t s) {
-  wall_stress_kernel<Real><<<E, 64, 0, s>>>(u, dim, n, Np, affine, el_drdx, drdx, Dm, (const WallPt<Real> *)walls,
+  wall_stress_kernel<Real><<<E, 64, 0, s>>>(u, dim, n, Np, layout, el_drdx, drdx, Dm, (const WallPt<Real> *)walls,
                                             wall_off, dir[0], dir[1], dir[2], mu, out);
   return cudaGetLastError();
 }
