@@ -119,7 +119,8 @@ struct selbm {
   int32_t *d_wall_off = nullptr, *d_first = nullptr;
   uint8_t *d_owner = nullptr;
   double *d_mass = nullptr, *d_partial = nullptr, *d_diag = nullptr;
-  double *d_fld = nullptr;       // [1 + dim][G] rho and u on unique nodes (allocated on first use)
+  // [1 + dim][G] rho and u on unique nodes: in f^2, which holds nothing between steps
+  double *fld() { return (double *)F2; }
   double *d_io = nullptr;  // staging for host <-> device FP64 arrays
   size_t io_bytes = 0;
   std::vector<void *> allocs;
@@ -744,22 +745,12 @@ int filtered_state(selbm *h, const void **f) {
   return finalize(h);
 }
 
-// rho and u of a state on unique nodes -> d_fld [1 + dim][G] (kept by the handle); diag: the
-// quadrature sums into d_diag too
+// rho and u of a state on unique nodes -> fld() [1 + dim][G]; diag: the quadrature sums into d_diag too
 int node_fields(selbm *h, const void *f, bool diag) {
-  const size_t G = h->S.G;
-  if (!h->d_fld) {
-    cudaError_t e = cudaMalloc((void **)&h->d_fld, (1 + (size_t)h->S.dim) * G * sizeof(double));
-    if (e != cudaSuccess) {
-      h->d_fld = nullptr;
-      return h->cuda_fail(e, "field buffer");
-    }
-    h->allocs.push_back(h->d_fld);
-  }
   auto run = [&](auto tag) -> cudaError_t {
     using Real = decltype(tag);
-    return diag ? launch_diag<Real>(h->lat, (const Real *)f, h->d_mass, h->S.G, h->Gs(), h->P.rho0, h->d_fld, h->d_partial, h->d_diag, h->stream)
-                : launch_node_fields<Real>(h->lat, (const Real *)f, h->S.G, h->Gs(), h->P.rho0, h->d_fld, h->stream);
+    return diag ? launch_diag<Real>(h->lat, (const Real *)f, h->d_mass, h->S.G, h->Gs(), h->P.rho0, h->fld(), h->d_partial, h->d_diag, h->stream)
+                : launch_node_fields<Real>(h->lat, (const Real *)f, h->S.G, h->Gs(), h->P.rho0, h->fld(), h->stream);
   };
   const cudaError_t e = h->prec == SELBM_FP64 ? run(double()) : run(float());
   return e == cudaSuccess ? SELBM_OK : h->cuda_fail(e, "moments");
@@ -1143,7 +1134,7 @@ int selbm_moments(selbm_t *h, double *rho, double *u, int on_device) {
     if ((rc = ensure_io(h, nl * (1 + d) * 8))) return rc;
     dr = h->d_io; du = h->d_io + nl;
   }
-  cudaError_t e = launch_expand_fields((int)d, h->d_fld, h->S.G, h->d_l2g, nl, dr, du, h->stream);
+  cudaError_t e = launch_expand_fields((int)d, h->fld(), h->S.G, h->d_l2g, nl, dr, du, h->stream);
   if (e == cudaSuccess && !on_device) {
     e = cudaMemcpyAsync(rho, dr, nl * 8, cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(u, du, nl * d * 8, cudaMemcpyDeviceToHost, h->stream);
@@ -1282,7 +1273,7 @@ int selbm_diagnostics(selbm_t *h, double out[8]) {
   const size_t nl = h->nloc(), dim = h->S.dim;
   if ((rc = ensure_io(h, nl * (1 + dim) * 8 + (h->S.E + 1) * 8))) return rc;
   double *u_l = h->d_io + nl, *part = h->d_io + nl * (1 + dim), *d_eps = h->d_diag + 6;
-  cudaError_t e = launch_expand_fields((int)dim, h->d_fld, h->S.G, h->d_l2g, nl, nullptr, u_l, h->stream);
+  cudaError_t e = launch_expand_fields((int)dim, h->fld(), h->S.G, h->d_l2g, nl, nullptr, u_l, h->stream);
   if (e == cudaSuccess) {
     const double mu = h->P.rho0 * h->P.nu;
     e = h->prec == SELBM_FP64
@@ -1322,7 +1313,7 @@ int selbm_wall_stress(selbm_t *h, const double dir[3], double *tau) {
   if ((rc = ensure_io(h, (nl * (1 + dim) + 2 * (size_t)h->n_wallpts) * 8))) return rc;
   double *u_l = h->d_io + nl, *part = h->d_io + nl * (1 + dim);
   const double mu = h->P.rho0 * h->P.nu;
-  cudaError_t e = launch_expand_fields(dim, h->d_fld, h->S.G, h->d_l2g, nl, nullptr, u_l, h->stream);
+  cudaError_t e = launch_expand_fields(dim, h->fld(), h->S.G, h->d_l2g, nl, nullptr, u_l, h->stream);
   if (e == cudaSuccess)
     e = h->prec == SELBM_FP64
             ? launch_wall_stress<double>(u_l, dim, h->S.n1, h->S.Np, h->S.E, h->metrics(), (const double *)h->d_el_drdx,
@@ -1368,7 +1359,7 @@ int selbm_radial_profile(selbm_t *h, const double origin[3], const double axis[3
   const int blocks = 256;
   if ((rc = ensure_io(h, (size_t)blocks * 2 * nbins * 8))) return rc;
   double *part = h->d_io;
-  e = launch_radial_profile(h->d_fld + h->S.G, dim, h->d_xg, h->d_mass, h->S.G, o, a, radius, nbins, blocks, part, h->stream);
+  e = launch_radial_profile(h->fld() + h->S.G, dim, h->d_xg, h->d_mass, h->S.G, o, a, radius, nbins, blocks, part, h->stream);
   std::vector<double> hp((size_t)blocks * 2 * nbins);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hp.data(), part, hp.size() * 8, cudaMemcpyDeviceToHost, h->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
