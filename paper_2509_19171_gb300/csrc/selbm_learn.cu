@@ -619,8 +619,12 @@ static size_t tile_smem(int nin, int ts) {
 }
 
 // samples per tile: about one tile per SM, so that neither the samples of one CTA nor the number of
-// gradient partials grows beyond what the batch needs
-static int tile_samples(int64_t count) { return count <= 8 * 152 ? 8 : (count <= 16 * 304 ? 16 : (count <= 32 * 608 ? 32 : 64)); }
+// gradient partials grows beyond what the batch needs; fewer where a wide input layer fills the shared memory
+static int tile_samples(int64_t count, int nin) {
+  int ts = count <= 8 * 152 ? 8 : (count <= 16 * 304 ? 16 : (count <= 32 * 608 ? 32 : 64));
+  while (ts > 8 && tile_smem(nin, ts) > 227 * 1024) ts /= 2;
+  return ts;
+}
 
 template <int TS>
 static cudaError_t launch_tiles_t(int tiles, const TileArgs &a, int forward_only, cudaStream_t s) {
@@ -648,7 +652,7 @@ static cudaError_t launch_reduce(const float *gpart, const float *lpart, int til
 
 cudaError_t mlp_grad(const float *params, int nin, int N, const float *X, const float *Y, int64_t M, float *grad,
                      float *loss, cudaStream_t s) {
-  const int P = mlp_nparams(nin), ts = tile_samples(M);
+  const int P = mlp_nparams(nin), ts = tile_samples(M, nin);
   const int tiles = (int)((M + ts - 1) / ts);
   float *gpart = nullptr, *lpart = nullptr;
   cudaError_t e = cudaMalloc(&gpart, (size_t)tiles * P * sizeof(float));
@@ -667,7 +671,7 @@ cudaError_t mlp_grad(const float *params, int nin, int N, const float *X, const 
 
 cudaError_t mlp_forward(const float *params, int nin, int N, const float *X, int64_t M, int bf16, float *out,
                         cudaStream_t s) {
-  const int ts = tile_samples(M), tiles = (int)((M + ts - 1) / ts);
+  const int ts = tile_samples(M, nin), tiles = (int)((M + ts - 1) / ts);
   TileArgs a{params, nin, N, X, nullptr, M, 0, M, 0, 0, nullptr, nullptr, out, bf16};
   cudaError_t e = launch_tiles(ts, tiles, a, 1, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -679,7 +683,7 @@ cudaError_t mlp_train(float *params, float *m, float *v, int nin, int N, const f
                       cudaStream_t s) {
   const int P = mlp_nparams(nin);
   const int64_t most = std::min<int64_t>(batch, M), nb = (M + batch - 1) / batch;
-  const int ts = tile_samples(most), tiles = (int)((most + ts - 1) / ts);
+  const int ts = tile_samples(most, nin), tiles = (int)((most + ts - 1) / ts);
   int h = 1;
   while ((int64_t)1 << (2 * h) < M) ++h;
   // the loss of every minibatch stays on the device and is read once an epoch
