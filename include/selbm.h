@@ -159,9 +159,9 @@ const char *selbm_last_error(const selbm_t *h);
 
 /*
  * Sizes and scalars: out_i[0..8] = E, Np, Q, G (unique nodes), dim, N,
- * precision, steps taken, step form (0: whole-element stage kernels, 1:
- * population-split stages after a per-element prologue); out_d[0..3] = dt,
- * tau, lambda, time.
+ * precision, steps taken, step form of the kernel timers (0: whole-element stage
+ * kernels, and 2D meshes; 1: population-split stages, the filter and the collision
+ * before them); out_d[0..3] = dt, tau, lambda, time.
  */
 int selbm_info(const selbm_t *h, int64_t out_i[9], double out_d[4]);
 /* Lattice table: e[Q][3] (zero-padded in 2D), t[Q], opposite[Q]. */
@@ -364,9 +364,10 @@ int selbm_mesh_check_nodes(const selbm_mesh_nodes *mesh, int32_t lattice, int32_
  *          the population-split form also the collision and the assembly of
  *          the filtered copies of shared nodes)
  *   k = 4: population-split form: prologue (fixed filter + collision, or the
- *          collision alone when no filter is pending)
- * The population-split form is the default for hexahedral meshes at the
- * compiled orders (D3Q19: N = 4, 7; D3Q27: N = 5, 7), in both precisions.
+ *          collision alone when no filter is pending; one kernel or two)
+ * A group of kernels counts as one launch.  The population-split form is the default
+ * for hexahedral meshes, FP32 up to N = 11 and FP64 up to N = 9.  While the timers are
+ * on, a 2D mesh takes the whole-element form in place of the one resident launch.
  */
 #define SELBM_TIMER_KINDS 5
 int selbm_timers(selbm_t *h, int enable);

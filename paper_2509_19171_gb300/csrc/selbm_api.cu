@@ -951,7 +951,7 @@ int selbm_info(const selbm_t *h, int64_t out_i[9], double out_d[4]) {
   if (out_i) {
     out_i[0] = h->S.E; out_i[1] = h->S.Np; out_i[2] = h->Q; out_i[3] = h->S.G;
     out_i[4] = h->S.dim; out_i[5] = h->S.N; out_i[6] = h->prec; out_i[7] = h->steps;
-    out_i[8] = h->use_split ? 1 : 0;
+    out_i[8] = h->split_form() ? 1 : 0;
   }
   if (out_d) { out_d[0] = h->dt; out_d[1] = h->tau; out_d[2] = h->lam; out_d[3] = h->time; }
   return SELBM_OK;
