@@ -127,7 +127,8 @@ def kernel_bytes(c, Q, rsz, affine, split, learned):
           "assembly": ((ENb + 2 * Gb) + 2 * (ENb + 3 * Gb)) * Q * rsz / 3}
     if split:
         kb["stage1"] = (G + Gint + ENb) * Q * rsz + geo                # f^0 -> f^1 (interior), trace
-        kb["prologue"] = 2 * G * Q * rsz                               # f -> (filter, collision) -> f^0
+        # f -> (filter, collision) -> f^0: one kernel in FP32, two in FP64
+        kb["prologue"] = (4 if rsz == 8 else 2) * G * Q * rsz
         # learned: f -> features, network, per-element filter; interior f^0 + boundary shares;
         # then the shares' assembly + collision on shared nodes
         kb["learned"] = (G + Gint + ENb) * Q * rsz + (ENb + Gb) * Q * rsz + (0 if affine else E * Np * rsz)
@@ -362,7 +363,8 @@ def workload_config(case, form, world):
     nloc = case.mesh.nelem * (case.order + 1) ** dim
     return {"workload": f"{case.name}: {case.lattice}, {case.mesh.nelem} elements, N={case.order}, "
                         f"{nloc} local nodes, {nloc * Q} populations",
-            "form": form, "filter": case.filt, "l2": "inputs larger than L2 (no flush)",
+            "form": form, "filter": case.filt,
+            "l2": "state in shared memory between steps" if dim == 2 else "inputs larger than L2 (no flush)",
             "parallelism": f"replicas x{world}"}
 
 
@@ -426,8 +428,8 @@ def main():
     hbm = float(pk["hbm_gbs"])
 
     forms = [f for f in args.forms.split(",") if f]
-    if "fp32dev_learned" in forms and not os.path.exists(WEIGHTS):
-        forms.remove("fp32dev_learned")
+    if "fp32dev_learned" in forms and not (os.path.exists(WEIGHTS) and len(np.load(WEIGHTS)["lo"]) == 2 * (case.order + 1)):
+        forms.remove("fp32dev_learned")                                  # no weights at this order
     main_form = "fp32dev_learned" if "fp32dev_learned" in forms else forms[-1]
     order = [f for f in forms if f != main_form] + [main_form]
     results, fields, clocks = {}, {}, None
@@ -445,7 +447,9 @@ def main():
         if sampler:
             clocks = sampler.stop(dev_index)
         ms = max_over_ranks(ms, dist, "cuda")
-        t = kernel_times(torch, s, ksteps)
+        # kernel timers take a 2D mesh off the resident step that was timed: no kernel figures there
+        resident = case.mesh.dim == 2
+        t = {} if resident else kernel_times(torch, s, ksteps)
         e, _, _ = s.lattice_table()
         nz_axes = float(np.abs(e).astype(bool).sum(1).mean()) if info["affine"] else float(case.mesh.dim)
         Q = s.Q
@@ -461,14 +465,14 @@ def main():
         step_bytes += kb["learned"] if learned else (kb["prologue"] if s.split else 0)
         entry = {
             "value": value, "ms_per_step": ms / args.steps, "dtype": "f64" if form == "fp64" else "f32",
-            "step_form": "population-split" if s.split else "whole-element",
+            "step_form": "resident" if resident else "population-split" if s.split else "whole-element",
             "kernel_ms": kernel_ms, "kernel_hbm_frac_alg": kernel_frac,
             "launches_per_step": launches_per_step(s.split, learned, form == "fp64", case.mesh.dim, args.steps),
-            "hbm_gbs_alg_step": step_bytes / (ms / args.steps * 1e-3) / 1e9,
-            "bytes_per_update": step_bytes / upd_step,
+            "hbm_gbs_alg_step": None if resident else step_bytes / (ms / args.steps * 1e-3) / 1e9,
+            "bytes_per_update": None if resident else step_bytes / upd_step,
             "stage23_bytes": kb["stage23"], "stage23_ms": per.get("stage23"),
         }
-        if form == "fp64":
+        if form == "fp64" and not resident:
             # rate of the stage 2/3 kernel (derivative, metric and stage-combination flops) against
             # the FP64 pipe's; above 1 where its lines run in 64-bit integers (hexahedra)
             if fp64_tflops is None:
@@ -495,13 +499,17 @@ def main():
             r, u = fields[form]
             du = np.linalg.norm(u - u64, axis=-1)
             results[form]["err_vs_fp64"] = {
-                "after_steps": args.warmup + args.steps + ksteps,
+                "after_steps": args.warmup + args.steps + (0 if case.mesh.dim == 2 else ksteps),
                 "u_max_over_U0": float(du.max() / case.U0), "u_rms_over_U0": float(np.sqrt((du ** 2).mean()) / case.U0),
                 "rho_max": float(np.abs(r - r64).max()), "rho_rms": float(np.sqrt(((r - r64) ** 2).mean()))}
         if main_form != "fp64":
             results[main_form]["speedup_vs_fp64"] = results[main_form]["value"] / results["fp64"]["value"]
     r = results[main_form]
-    if main_form == "fp64":
+    if r["step_form"] == "resident":
+        # the state stays in shared memory: three exchanges of shares between CTAs a step bound it, not a pipe
+        roof = {"bound": "latency", "kernel": f"flow2d_kernel<{r['dtype']}, N={case.order}> (all steps of a call)",
+                "achieved": r["ms_per_step"] * 1e3, "peak": None, "unit": "us / step", "frac": None, "traffic": None}
+    elif main_form == "fp64":
         achieved = r["stage23_flops"] / (r["stage23_ms"] * 1e-3) / 1e12
         roof = {"bound": "alu", "kernel": "stage kernel, stages 2 and 3 (FP64 operations, hexahedra: formed in 64-bit integers)", "achieved": achieved,
                 "peak": fp64_tflops, "unit": "TFLOP/s", "frac": achieved / fp64_tflops,
