@@ -8,9 +8,11 @@
 // integer at the tile's largest exponent, a coefficient a signed integer of up to 62 bits, and a
 // product is formed from 32-bit signed limbs,
 //   C q / 2^64 = Ch Qh + (Ch Ql + Cl Qh) / 2^32 (+ Cl Ql / 2^64, below the last place kept),
-// three IMAD.WIDE instead of one DFMA that costs 32 times an issue slot.  The rounding of a
-// product sum is then about 2^-57 of (row sum of |coefficients|) x (largest value), below the
-// 2^-53 of the FP64 operations it replaces; the results return to FP64 rounded to nearest.
+// three IMAD.WIDE instead of one DFMA that costs 32 times an issue slot.  The dropped lowest products are
+// at most a quarter of the sum's last place each, before the shift of a result by up to three bits: a line
+// of n terms is off by at most n 2^-59 of (row sum of |coefficients|) x (tile's largest value), 2^-57 and
+// less on average (figures in selbm_fixed_lines.cuh); where that matters the high word of the lowest
+// product is added too.  The results return to FP64 rounded to nearest.
 #pragma once
 #include <cuda_runtime.h>
 

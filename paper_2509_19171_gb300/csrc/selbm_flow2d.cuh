@@ -809,8 +809,8 @@ flow2d_kernel(const Flow2DArgs<Real> p, const StageMats<Real, n> m, const Filter
             Fix128 sr{0, 0}, ss{0, 0}, y{0, 0};
 #pragma unroll 3
             for (int c = 0; c < n; ++c) {
-              fix_mac(sr, dr[c], fr[c]);
-              fix_mac(ss, ds[c], fs[LS * c]);
+              fix_mac_line<n>(sr, dr[c], fr[c]);
+              fix_mac_line<n>(ss, ds[c], fs[LS * c]);
             }
             fix_mac(y, limbs(coef(0, q, a, o)), limbs(fix_top<3>(sr)));
             fix_mac(y, limbs(coef(1, q, a, o)), limbs(fix_top<3>(ss)));

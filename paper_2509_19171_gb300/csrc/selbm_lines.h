@@ -2,12 +2,10 @@
 #pragma once
 #include <type_traits>
 
+#include "selbm_fixed_lines.cuh"
 #include "selbm_kernels.cuh"
 
 namespace slb {
-
-template <typename Real>
-using LineVal = std::conditional_t<sizeof(Real) == 8, long long, float>;   // a line's value
 
 // velocity set at run time
 struct LatticeRT {

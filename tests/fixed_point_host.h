@@ -11,9 +11,11 @@
 #define __global__
 #define __forceinline__ inline
 #define __noinline__
+using std::fma;
 using std::isfinite;
 using std::max;
 using std::min;
+using std::scalbn;
 
 template <typename To, typename From>
 To host_bits(From v) {

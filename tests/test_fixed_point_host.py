@@ -1,7 +1,8 @@
-"""The arithmetic of the collision, compiled for the host and compared with long
+"""The arithmetic of the collision and of the FP64 lines, compiled for the host and compared with long
 double: the collision in fixed point is no further from it than the FP64 collision is, for every
 speed class (small populations included) and from small to full relaxation, and stays bounded on
-populations that span many decades; the FP32 collision keeps the momentum on average."""
+populations that span many decades; the FP32 collision keeps the momentum on average; derivative and
+filter of a line in fixed point are no further off than the same even-odd products in FP64."""
 import os
 import shutil
 import subprocess
@@ -160,6 +161,172 @@ int all() { return check<LAT>(0.04, 1.99) + check<LAT>(0.04, 0.7) + check<LAT>(0
 int main() { return all<SELBM_D2Q9>() + all<SELBM_D3Q19>() + all<SELBM_D3Q27>() ? 1 : 0; }
 """
 
+LINES = r"""
+#include <cuda_runtime.h>
+#include <cstdio>
+#include <random>
+#include <vector>
+#include "selbm_fixed_lines.cuh"
+using namespace slb;
+using L = long double;
+struct Host { const double *D, *w, *Vm, *Vinv, *fixed_sigma; };
+
+template <int n>
+struct Basis {
+  double xi[n], D[n * n], V[n * n], Vi[n * n], w[n] = {};
+  static double leg(int k, double x) {
+    double a = 1, b = x;
+    if (k == 0) return 1;
+    for (int i = 2; i <= k; ++i) { const double c = ((2 * i - 1) * x * b - (i - 1) * a) / i; a = b; b = c; }
+    return b;
+  }
+  Basis() {
+    const int N = n - 1;
+    for (int i = 0; i < n; ++i) {
+      double x = -std::cos(std::acos(-1.0) * i / N);
+      if (i && i < N)
+        for (int it = 0; it < 60; ++it) x -= (x * leg(N, x) - leg(N - 1, x)) / (n * leg(N, x));
+      xi[i] = x;
+    }
+    for (int i = 0; i <= N / 2; ++i) { const double t = (xi[i] - xi[N - i]) / 2; xi[i] = t; xi[N - i] = -t; }
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j) {
+        L p = 0;
+        if (i == j) {
+          for (int k = 0; k < n; ++k)
+            if (k != j) p += 1.L / ((L)xi[j] - xi[k]);
+        } else {
+          p = 1.L / ((L)xi[j] - xi[i]);
+          for (int m = 0; m < n; ++m)
+            if (m != i && m != j) p *= ((L)xi[i] - xi[m]) / ((L)xi[j] - xi[m]);
+        }
+        D[i * n + j] = (double)p;
+        V[i * n + j] = j < 2 ? (j ? xi[i] : 1.0) : leg(j, xi[i]) - leg(j - 2, xi[i]);
+      }
+    for (int i = 0; i < n; ++i)
+      for (int j = 0; j < n; ++j) D[(N - i) * n + N - j] = -D[i * n + j];
+    if (n & 1) D[(N / 2) * n + N / 2] = 0;
+    L a[n][2 * n];
+    for (int i = 0; i < n; ++i)
+      for (int k = 0; k < n; ++k) { a[i][k] = V[i * n + k]; a[i][n + k] = i == k; }
+    for (int c = 0; c < n; ++c) {
+      int p = c;
+      for (int r = c; r < n; ++r) if (fabsl(a[r][c]) > fabsl(a[p][c])) p = r;
+      for (int k = 0; k < 2 * n; ++k) std::swap(a[c][k], a[p][k]);
+      const L d = a[c][c];
+      for (int k = 0; k < 2 * n; ++k) a[c][k] /= d;
+      for (int r = 0; r < n; ++r)
+        if (r != c) { const L f = a[r][c]; for (int k = 0; k < 2 * n; ++k) a[r][k] -= f * a[c][k]; }
+    }
+    for (int i = 0; i < n; ++i)
+      for (int k = 0; k < n; ++k) Vi[i * n + k] = (double)a[i][n + k];
+  }
+};
+
+template <int n>
+int derivative() {
+  const Basis<n> b;
+  const Host h{b.D, b.w, nullptr, nullptr, nullptr};
+  const StageMats<double, n> m = make_stage_mats<double, n>(h);
+  std::mt19937_64 r(2);
+  std::normal_distribution<double> G;
+  constexpr int N = n - 1, SHIFT = FixScale<n>::SHIFT;
+  L e0 = 0, e1 = 0;
+  for (int it = 0; it < 3000; ++it) {
+    double v[n], top = 0;
+    const double a = G(r), c = G(r), k = 1 + 2 * std::fabs(G(r));
+    for (int j = 0; j < n; ++j) { v[j] = 0.5 * a + c * std::sin(k * b.xi[j] + a); top = std::max(top, std::fabs(v[j])); }
+    int em = kMinExp;
+    for (int j = 0; j < n; ++j) { v[j] /= top; em = std::max(em, exp_of(v[j])); }
+    long long q[n], d[n];
+    for (int j = 0; j < n; ++j) q[j] = to_fixed<SHIFT>(v[j], em);
+    line_deriv<n>(m, q, d);
+    for (int j = 0; j < n; ++j) {
+      L ex = 0;
+      for (int i = 0; i < n; ++i) ex += (L)b.D[j * n + i] * v[i];
+      const int jj = 2 * j <= N ? j : N - j;
+      double se = 0, so = 0;
+      for (int i = 0; i < n / 2; ++i) {
+        const double x = b.D[jj * n + i], y = b.D[jj * n + N - i];
+        se = std::fma(2 * jj == N ? 0.0 : 0.5 * (x + y), v[i] + v[N - i], se);
+        so = std::fma(0.5 * (x - y), v[i] - v[N - i], so);
+      }
+      if ((n & 1) && 2 * jj != N) se = std::fma(b.D[jj * n + N / 2], v[N / 2], se);
+      const L x0 = (L)(2 * j <= N ? so + se : se - so) - ex;
+      const L x1 = (L)from_fixed(d[j], 61 - m.cb + em - FixScale<n>::EXP0) - ex;
+      e0 += x0 * x0;
+      e1 += x1 * x1;
+    }
+  }
+  if (e1 <= e0) return 0;
+  std::printf("derivative n = %d: fixed %Lg fp64 %Lg\n", n, sqrtl(e1), sqrtl(e0));
+  return 1;
+}
+
+// three passes over a tile; the result is the value plus the tile's change
+template <int n>
+int filter(double gamma) {
+  const Basis<n> b;
+  double sg[n];
+  const double kc = std::max(1, n - 3);
+  for (int k = 0; k < n; ++k) { const double r = (k - kc) / (n - 1 - kc); sg[k] = k > kc ? 1 - gamma * r * r : 1; }
+  const Host h{nullptr, b.w, b.V, b.Vi, sg};
+  const FilterMats<double, n> m = make_filter_mats<double, n>(h);
+  const int shift = filter_gain_shift(m, m.ex);
+  long long g[n];
+  for (int k = 0; k < n; ++k) g[k] = filter_gain(sg[k] - 1, shift);
+  std::mt19937_64 r(3);
+  std::normal_distribution<double> G;
+  L e0 = 0, e1 = 0;
+  for (int it = 0; it < 3; ++it) {
+    std::vector<double> v(n * n * n), a;
+    for (double &x : v) x = G(r);
+    a = v;
+    std::vector<L> x(v.begin(), v.end());
+    int em = kMinExp;
+    for (double y : v) em = std::max(em, exp_of(y));
+    std::vector<long long> t;
+    for (double y : v) t.push_back(to_fixed<kFilterShift>(y, em));
+    for (int ax = 0, st = 1; ax < 3; ++ax, st *= n)
+      for (int l = 0; l < n * n; ++l) {
+        const int base = ax == 0 ? l * n : ax == 1 ? (l % n) + (l / n) * n * n : l;
+        long long q[n];
+        double o[n];
+        L y[n];
+        for (int k = 0; k < n; ++k) { q[k] = t[base + k * st]; o[k] = a[base + k * st]; y[k] = x[base + k * st]; }
+        line_filter<n>(m, g, shift, q);
+        for (int k = 2; k < n; ++k) {
+          double s = 0;
+          L S = 0;
+          for (int j = 0; j < n; ++j) { s = std::fma(b.Vi[k * n + j], a[base + j * st], s); S += (L)b.Vi[k * n + j] * x[base + j * st]; }
+          s *= sg[k] - 1;
+          S *= (L)sg[k] - 1;
+          for (int j = 1; j < n - 1; ++j) { o[j] = std::fma(b.V[j * n + k], s, o[j]); y[j] += (L)b.V[j * n + k] * S; }
+        }
+        for (int k = 1; k < n - 1; ++k) { t[base + k * st] = q[k]; a[base + k * st] = o[k]; x[base + k * st] = y[k]; }
+      }
+    for (size_t i = 0; i < v.size(); ++i) {
+      const double f = v[i] + from_fixed(t[i] - to_fixed<kFilterShift>(v[i], em), em - (1023 + 52 + kFilterShift));
+      e0 += ((L)a[i] - x[i]) * ((L)a[i] - x[i]);
+      e1 += ((L)f - x[i]) * ((L)f - x[i]);
+    }
+  }
+  if (e1 <= e0) return 0;
+  std::printf("filter n = %d gamma %g: fixed %Lg fp64 %Lg\n", n, gamma, sqrtl(e1), sqrtl(e0));
+  return 1;
+}
+
+template <int n>
+int all() {
+  int bad = derivative<n>();
+  if constexpr (n > 3)
+    for (double gamma : {0.01, 0.1, 0.5, 1.0}) bad += filter<n>(gamma);
+  if constexpr (n < 15) return bad + all<n + 1>();
+  else return bad;
+}
+int main() { return all<3>() ? 1 : 0; }
+"""
+
 
 def run_host(tmp_path, source):
     gxx = shutil.which("g++")
@@ -180,3 +347,7 @@ def test_collision(tmp_path):
 
 def test_fp32_momentum(tmp_path):
     run_host(tmp_path, MOMENTUM)
+
+
+def test_lines(tmp_path):
+    run_host(tmp_path, LINES)
