@@ -18,10 +18,12 @@ bool split_stage_d3q19(int N, bool affine, const KParams<Real> &p, const SplitHo
   return false;
 }
 
-// which: 0 collision on unique nodes, 1 assembly of learned-filter shares + collision
+// which: 0 collision on unique nodes, 1 assembly of learned-filter shares + collision (FP32)
 template <typename Real>
 cudaError_t split_collide_d3q19(int which, const KParams<Real> &p, cudaStream_t s) {
-  return which == 0 ? launch_collide_nodes_t<Real, SELBM_D3Q19>(p, s) : launch_dss_collide_t<Real, SELBM_D3Q19>(p, s);
+  if (which == 0) return launch_collide_nodes_t<Real, SELBM_D3Q19>(p, s);
+  if constexpr (sizeof(Real) == 4) return launch_dss_collide_t<Real, SELBM_D3Q19>(p, s);
+  return cudaErrorInvalidValue;
 }
 
 template bool split_stage_d3q19<float>(int, bool, const KParams<float> &, const SplitHost &, cudaStream_t, cudaError_t *);

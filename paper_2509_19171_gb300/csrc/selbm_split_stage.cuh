@@ -9,13 +9,6 @@
 #include "selbm_fast.cuh"
 
 namespace slb {
-// asynchronous global -> shared copy of one value (cp.async, 4 or 8 bytes)
-template <typename Real>
-__device__ __forceinline__ void cp_async(Real *dst, const Real *src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  if constexpr (sizeof(Real) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(d), "l"(src) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 template <int LAT, int n, int PBW = 0>
@@ -82,8 +75,8 @@ __device__ __forceinline__ void axpy_line(Real (&acc)[n], Real s, const Real (&w
 // asynchronous copy of one value to a shared-memory byte address
 template <typename Real>
 __device__ __forceinline__ void cp_async_s(unsigned dst, const Real *src) {
-  if constexpr (sizeof(Real) == 4) asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
-  else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(dst), "l"(src) : "memory");
+  static_assert(sizeof(Real) == 4, "FP64 lines gather through registers");
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(dst), "l"(src) : "memory");
 }
 
 __device__ __forceinline__ void cp_async16_s(unsigned dst, const void *src) {
@@ -95,7 +88,7 @@ __device__ __forceinline__ void cp_async16_s(unsigned dst, const void *src) {
 // component, [E][9][Np] (3 l + k)
 // ---------------------------------------------------------------------------
 template <typename Real, int LAT, int n, bool AFFINE, int PBW = 0>
-__global__ void __launch_bounds__(SplitShape<LAT, n, PBW>::THREADS, (sizeof(Real) == 4 ? (AFFINE ? (PBW > 9 ? 4 : 5) : (PBW > 0 ? 3 : 4)) : 2))
+__global__ void __launch_bounds__(SplitShape<LAT, n, PBW>::THREADS, AFFINE ? (PBW > 9 ? 4 : 5) : (PBW > 0 ? 3 : 4))
 stage_split_kernel(const KParams<Real> p, const FastMats<Real, n> m) {
   using S = SplitShape<LAT, n, PBW>;
   constexpr int Q = S::Q, DIM = 3, Np = S::Np, NL = S::NL, T = S::THREADS, PB = S::PB, NG = S::NG;
@@ -105,7 +98,6 @@ stage_split_kernel(const KParams<Real> p, const FastMats<Real, n> m) {
   constexpr VelTab V = LT<LAT>::v;
   constexpr uint32_t POS[3] = {vel_mask(V, 0, 1), vel_mask(V, 1, 1), vel_mask(V, 2, 1)};
   constexpr uint32_t NEG[3] = {vel_mask(V, 0, -1), vel_mask(V, 1, -1), vel_mask(V, 2, -1)};
-  constexpr int KU = sizeof(Real) == 4 ? n : 2;
   constexpr unsigned RS = sizeof(Real);
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Real *sf = reinterpret_cast<Real *>(smem_raw);   // [PB][PS] f^{s-1} of the group
@@ -453,22 +445,22 @@ stage_split_kernel(const KParams<Real> p, const FastMats<Real, n> m) {
         }
         if (c1 != Real(0)) {
           Real dr[n];
-          if (KU == n) load_line<Real, n>(sDi1, 0, dr);
-#pragma unroll KU
+          load_line<Real, n>(sDi1, 0, dr);
+#pragma unroll
           for (int k = 0; k < n; ++k) {
             Real w[n];
             load_line<Real, n>(fa + yline(k), TI::sw(k), w);
-            axpy_line<Real, n>(adv, c1 * (KU == n ? dr[k] : sDi1[k]), w);
+            axpy_line<Real, n>(adv, c1 * dr[k], w);
           }
         }
         if (c2 != Real(0)) {
           Real dr[n];
-          if (KU == n) load_line<Real, n>(sDi2, 0, dr);
-#pragma unroll KU
+          load_line<Real, n>(sDi2, 0, dr);
+#pragma unroll
           for (int k = 0; k < n; ++k) {
             Real w[n];
             load_t(k, w);
-            axpy_line<Real, n>(adv, c2 * (KU == n ? dr[k] : sDi2[k]), w);
+            axpy_line<Real, n>(adv, c2 * dr[k], w);
           }
         }
       } else {
@@ -488,28 +480,28 @@ stage_split_kernel(const KParams<Real> p, const FastMats<Real, n> m) {
         }
         {
           Real d[n], dr[n];
-          if (KU == n) load_line<Real, n>(sDi1, 0, dr);
+          load_line<Real, n>(sDi1, 0, dr);
 #pragma unroll
           for (int j = 0; j < n; ++j) d[j] = 0;
-#pragma unroll KU
+#pragma unroll
           for (int k = 0; k < n; ++k) {
             Real w[n];
             load_line<Real, n>(fa + yline(k), TI::sw(k), w);
-            axpy_line<Real, n>(d, KU == n ? dr[k] : sDi1[k], w);
+            axpy_line<Real, n>(d, dr[k], w);
           }
 #pragma unroll
           for (int j = 0; j < n; ++j) adv[j] += coef(j, 1) * d[j];
         }
         {
           Real d[n], dr[n];
-          if (KU == n) load_line<Real, n>(sDi2, 0, dr);
+          load_line<Real, n>(sDi2, 0, dr);
 #pragma unroll
           for (int j = 0; j < n; ++j) d[j] = 0;
-#pragma unroll KU
+#pragma unroll
           for (int k = 0; k < n; ++k) {
             Real w[n];
             load_t(k, w);
-            axpy_line<Real, n>(d, KU == n ? dr[k] : sDi2[k], w);
+            axpy_line<Real, n>(d, dr[k], w);
           }
 #pragma unroll
           for (int j = 0; j < n; ++j) adv[j] += coef(j, 2) * d[j];
