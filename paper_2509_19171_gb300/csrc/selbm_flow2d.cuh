@@ -26,7 +26,13 @@ namespace slb {
 // polls of one wait, below a microsecond each.  A constant: with a limit from the launch's arguments, in any
 // form of the loop, the FP32 shear layer (32 x 32, N = 8) takes 1.35 instead of 1.15 ms a pass.
 constexpr int kFlowSpins = 4000000;
-constexpr int kNodeTasks = 3000;            // (population, node) tasks of a CTA up to which FP64 takes a thread per node
+// (population, node) tasks of a CTA up to which FP64 takes a thread per node and not per line.  Few tasks
+// leave threads idle in lines, many repeat the line's products.  us a step, node / line: 576 tasks (N = 7, one
+// element) 21.1 / 23.4, 1296 (N = 11, one) 34.2 / 42.2, 2187 (N = 8, three) 45.8 / 46.9, 2304 (N = 7, four)
+// 53.2 / 51.1, 2592 (N = 11, two) 56.7 / 60.7, 2916 (N = 8, four) 57.9 / 56.9, 3456 (N = 7, six) 74.3 / 68.4,
+// 3888 (N = 11, three) 80.9 / 82.2, 4050 (N = 14, two) 85.7 / 89.3: the line lies where neither side loses
+// more than a tenth.
+constexpr int kNodeTasks = 3000;
 
 template <typename Real, int n>
 struct Flow2DShape {
