@@ -12,7 +12,10 @@
 // precision and element kind serves both lattices.  Every pass forms its line products in the
 // even-odd form (the GLL nodes are symmetric, so derivative and filter map even parts to odd or
 // even parts: half the multiply-adds).  FP32 lines are FP32; FP64 lines are 64-bit fixed point
-// (selbm_fixed.cuh), since two FP64 operations per clock and SM bound everything else.
+// (selbm_fixed_lines.cuh), since two FP64 operations per clock and SM bound everything else.  FP64,
+// Taylor-Green 16^3, N = 7, D3Q27: a stage 798 us (2.59 ms in FP64 arithmetic), integer multiply-adds at 53 %
+// and issue at 51 % of their peaks with 35 % of the warps (80 registers and 41 KB: three CTAs); the filter
+// 632 us, ALU 61 %.
 //
 // The t-pass comes last and writes global memory itself: lanes run over (i0, i1), so a store of
 // one t-index is as coalesced as a node-ordered copy, and f^0, the wall-free result and the share
@@ -526,7 +529,8 @@ constexpr size_t lines_filter_smem(int pb) {
 
 // LEARNED: the element's transfer function sigma[e][n]; element-interior nodes to out, weighted
 // shares wJ f of boundary nodes to the trace.  Otherwise the fixed filter; every node is written
-// by its owner (the copies agree).
+// by its owner (the copies agree).  Writing the integers back instead of the value plus the tile's change
+// would take 588 us instead of 632 (FP64, as above), and the low bits of values small next to the tile's largest.
 template <typename Real, int n, bool LEARNED>
 __global__ void __launch_bounds__(LineShape<Real, n>::T, LineShape<Real, n>::F64 ? 3 : (n <= 8 ? 5 : 3))
 lines_filter_kernel(const KParams<Real> p, const FilterMats<Real, n> m, const Real *sigma, Real *out, const int Q,

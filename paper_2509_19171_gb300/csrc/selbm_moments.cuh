@@ -97,7 +97,8 @@ __device__ __forceinline__ int node_moments(const Real (&g)[LT<LAT>::v.Q], doubl
 // fixed-point products (t and omega): about 60 integer instructions where the FP64 form takes 12
 // FP64 ones, at 32 times their issue cost.  The change omega (t X - f) alone returns to FP64, times
 // 2^w_shift so that a small omega keeps its bits, and is added to f: a population that is small next
-// to the node's largest one keeps all of its own bits.  rho, 1 / rho and u stay FP64.
+// to the node's largest one keeps all of its own bits.  rho, 1 / rho and u stay FP64.  Taylor-Green 16^3,
+// D3Q27: 244 us a launch (1.09 ms in FP64 arithmetic), ALU 58 % at 24 % warps.
 // Nodes beyond the integers' range (|v| >= 1/4, a momentum far above the largest deviation,
 // infinities, NaN) take the FP64 collision.
 //
